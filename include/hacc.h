@@ -458,25 +458,23 @@ hacc_status hacc_tune(hacc_ctx *ctx, const hacc_box *box, const hacc_split *spli
  * cells.  HACC_EINVAL for other values. */
 hacc_status hacc_set_stencil(hacc_ctx *ctx, int32_t cells_per_rcut);
 
-/* Work items of the pair kernel in the single-box force paths (hacc_sr_force,
- * hacc_subcycle, hacc_step, hacc_diagnostics, hacc_tune and their host forms),
- * the batched and served paths and the multi-level step (whose small events
- * split every cell into smaller items still); the cell/offset paths and
- * hacc_sr_force_noalloc use cap = 0.  A work item is a set of particles of
- * one chaining-mesh cell that one warp runs against the cell's neighbours; a
- * neighbour particle farther than r_cut from the item's bounding box is
- * skipped, so items that cover a small part of their cell evaluate fewer
- * pairs, but every item stages all of its neighbours.
+/* Work items of the pair kernel (hacc_sr_force, hacc_subcycle, hacc_step,
+ * hacc_diagnostics, the batches; the multi-level step may split every cell
+ * into smaller items still).  A work item is a run of consecutive particles of
+ * one chaining-mesh cell in clusters of 8, processed by one warp; a neighbour
+ * particle farther than r_cut from a cluster's bounding box is skipped.
  * cap in [16, 160]: within each cell of up to 512 particles the particles are
- * ordered by their 4x4x4 sub-cell (Morton order, ties by input row; larger
- * cells by input row alone), and a cell of m <= split_max particles becomes
- * ceil(m / cap) items of consecutive particles of near-equal size; a denser
- * cell becomes ceil(m / 160) items (split_max = 0: no such limit).
- * cap = 0: input row order within cells and items of up to 160 particles.
- * cap = -1 (the default): 48 for calls of up to 2^22 particles (short
- * launches, whose tail the longest items of dense cells set) and 0 above.
- * The forces are sums over the same pairs for every setting (the summation
- * order differs, so results differ by FP32 rounding).  HACC_EINVAL for a cap
+ * ordered by their 4x4x4 sub-cell (along a Hilbert curve, ties by input row;
+ * larger cells by input row), so that clusters are compact; a cell is cut into
+ * items of at most cap and at most 64 particles, or of at most 64 where it
+ * holds more than split_max (split_max = 0: no such limit).
+ * cap = 0: input row order within cells, items of up to 64 particles, and
+ * neighbours skipped by the item's bounds alone.
+ * cap = -1 (default): by the box's size, 8 particles up to 2^13, 16 up to
+ * 2^16, 32 up to 2^20, 64 above (small boxes have few items to spread over the
+ * chip); a box of a batch follows its own size.  The cell/offset paths use 64,
+ * hacc_sr_force_noalloc row order with items of 64 skipped per cluster.
+ * Forces differ between settings only by the order of FP32 sums.  Errors: cap
  * outside {-1, 0} and [16, 160] or split_max < 0. */
 hacc_status hacc_set_item_cap(hacc_ctx *ctx, int32_t cap, int32_t split_max);
 

@@ -394,10 +394,10 @@ class Context:
         self._check(lib().hacc_set_variant(self._h, int(variant)), "hacc_set_variant")
 
     def set_item_cap(self, cap: int, split_max: int = 0):
-        """Particles per force work item at most: 16..160 with the cell's particles in sub-cell
-        order (cells above split_max particles keep items of up to 160, 0 = no such limit),
-        0 for input-row order and items of up to 160, or -1 (default): 48 for calls of up to
-        2^22 particles, else 0."""
+        """Particles per force work item at most: 16..160 (64 at most in effect) with the cell's
+        particles in sub-cell order (cells above split_max particles keep items of up to 64, 0 = no
+        such limit), 0 for input-row order and items of up to 64 culled as a whole, or -1 (default):
+        8 to 64 by the box's size."""
         self._check(lib().hacc_set_item_cap(self._h, int(cap), int(split_max)), "hacc_set_item_cap")
 
     def set_stencil(self, cells_per_rcut: int):

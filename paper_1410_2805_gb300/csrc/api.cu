@@ -282,6 +282,7 @@ hacc_status run_sorted_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts
     fl.within = within;
     fl.mass_flag = w->b.mass_flag;
     fl.variant = ctx->variant;
+    fl.cull = item_cap_for(ctx, n) != 0;
     if (ctx->counting && mode != kModePotential && !within) {
         HACC_CUDA(candidate_count(g, w->b.cell_start, ctx->d_pairs, s), "candidate count");
         fl.within = ctx->d_pairs + 1;
@@ -425,7 +426,7 @@ hacc_status hacc_set_stencil(hacc_ctx *ctx, int32_t cells_per_rcut) {
 
 hacc_status hacc_set_item_cap(hacc_ctx *ctx, int32_t cap, int32_t split_max) {
     HACC_TRY(enter(ctx));
-    if (cap != -1 && cap != 0 && (cap < kItemCapMin || cap > kItemMax))
+    if (cap != -1 && cap != 0 && (cap < kItemCapMin || cap > kItemCapMax))
         return set_error(ctx, HACC_EINVAL, "item cap must be -1, 0 or in [16, 160]");
     if (split_max < 0) return set_error(ctx, HACC_EINVAL, "split_max must be >= 0");
     ctx->item_cap = cap;
@@ -490,6 +491,7 @@ hacc_status hacc_tune(hacc_ctx *ctx, const hacc_box *box, const hacc_split *spli
         const int cap = kTuneCaps[k / (2 * kForceVariants)];
         ctx->queue_order = (k / kForceVariants) % 2;
         ctx->variant = k % kForceVariants;
+        ctx->item_cap = cap;
         st = subcycle_work(cap, true);   // warm-up, from pos_m
         if (st != HACC_OK) break;
         cudaEventRecord(e0, s);
@@ -1079,7 +1081,7 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
         for (int l = 1; l <= lmax; ++l)
             if (ev[k].kt.h[l] != 0.0f) kicked += present[l];
         const int64_t per_item = kicked / ((int64_t)ctx->num_sms * 64);
-        caps[k] = (int)std::max<int64_t>(kItemMin, std::min<int64_t>(kItemMax, per_item / 32 * 32));
+        caps[k] = (int)std::max<int64_t>(kCluster, std::min<int64_t>(kItemMax, per_item / kCluster * kCluster));
         if (icap) caps[k] = std::min(caps[k], icap);
     }
 

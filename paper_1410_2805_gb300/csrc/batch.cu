@@ -129,7 +129,7 @@ uint64_t plan_key(const Plan &pl) {
 }
 
 // Launch shape of a batched pass: the tuned one for this batch geometry, else
-// the context's variant and item cap.
+// the context's variant and item cap (-1: each box's automatic one).
 struct Shape {
     int variant, cap, order;
 };
@@ -137,7 +137,7 @@ struct Shape {
 Shape batch_shape(const hacc_ctx *ctx, const Plan &pl) {
     if (ctx->btune_key && ctx->btune_key == plan_key(pl))
         return Shape{ctx->btune_variant, ctx->btune_cap, ctx->btune_order};
-    return Shape{ctx->variant, item_cap_for(ctx, pl.n_total), ctx->queue_order};
+    return Shape{ctx->variant, ctx->item_cap, ctx->queue_order};
 }
 
 // One tick on the device tables `tab` (nbox entries).
@@ -168,6 +168,7 @@ hacc_status run_tick(hacc_ctx *ctx, const ForceConsts &fc, const Plan &pl, const
     fl.evaluated = ctx->counting ? ctx->d_pairs + 2 : nullptr;
     fl.mass_flag = w.b.mass_flag;
     fl.variant = sh.variant;
+    fl.cull = sh.cap != 0;
     if (sh.order && pl.n_total >= kHeavyFirstMinN) {
         HACC_CUDA_RETURN(items_heavy_first(w.b, max_items(pl.n_total, pl.ncell_total), s), "item order");
         fl.order = w.b.order;
@@ -432,7 +433,7 @@ extern "C" hacc_status hacc_batch_diagnostics(hacc_ctx *ctx, const hacc_split *s
     float4 *vp = const_cast<float4 *>(reinterpret_cast<const float4 *>(vel_pool));
     // the pools are only read: the binning writes wrapped copies to scratch
     HACC_CUDA_RETURN(bin_build_batch(pl.nbox, w.tables, pl.n_total, pl.ncell_total, pp, vp, w.P, w.ID, w.b,
-                                     ctx->d_flags, s, item_cap_for(ctx, pl.n_total), ctx->split_max),
+                                     ctx->d_flags, s, ctx->item_cap, ctx->split_max),
                      "batched binning");
     HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.b.perm, w.P, w.Ps, nullptr, nullptr, w.ID, w.IDs, s), "gather");
     HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.IDs, vp, w.Vs, nullptr, nullptr, nullptr, nullptr, s),

@@ -18,14 +18,13 @@ enum DeviceFlag : int {
     kFlagItems = 4,    // a work-item list ran out of room (an internal bound failed)
 };
 
-// Chunking of a chaining-mesh cell into force work items: a cell of n
-// particles is one item when n <= cap, else ceil(n/cap) items of near-equal
-// size; each item is processed by one warp (see item_shape in bin.cu).
-constexpr int kItemMax = 160;   // particles per work item at most (5 per lane)
-constexpr int kItemMin = 32;    // smallest per-event item cap of the multi-level step
-constexpr int kItemCapMin = 16; // smallest item cap of any path (sizes the item arrays)
-constexpr int kDefaultItemCap = 48;  // item cap of the automatic choice for small calls
-constexpr int64_t kAutoItemCapMaxN = (int64_t)1 << 22;  // largest call that the automatic choice splits
+// Chunking of a chaining-mesh cell into force work items: consecutive
+// clusters of kCluster particles of the cell's order, at most kItemMax
+// particles an item; each item is processed by one warp (sr_force.cu).
+constexpr int kCluster = 8;
+constexpr int kItemMax = 64;    // particles per work item at most (two per lane)
+// item caps of the settings (hacc_set_item_cap); above kItemMax they mean kItemMax
+constexpr int kItemCapMin = 16, kItemCapMax = 160;
 constexpr int kDefaultSplitMax = INT32_MAX;  // cells above this keep items of up to kItemMax
 
 struct Scratch {
@@ -88,13 +87,17 @@ struct hacc_ctx {
 };
 
 namespace hacc {
+// Automatic item cap of a box of n particles: smaller items for smaller boxes,
+// so that their few items spread over the chip.  A box of a batch follows its
+// own size, so that its sums are the same alone, in any mix and in a call of
+// its own.
+__host__ __device__ inline int auto_item_cap(int64_t n) {
+    return n <= (1 << 13) ? 8 : (n <= (1 << 16) ? 16 : (n <= (1 << 20) ? 32 : kItemMax));
+}
 // Item cap of a force call over n particles (hacc_set_item_cap): the set
-// value, or automatically kDefaultItemCap up to kAutoItemCapMaxN particles
-// (short launches, where the longest items of dense cells set the tail) and
-// cell-wide items above.
+// value, or the automatic one.
 inline int item_cap_for(const hacc_ctx *ctx, int64_t n) {
-    if (ctx->item_cap >= 0) return ctx->item_cap;
-    return n <= kAutoItemCapMaxN ? kDefaultItemCap : 0;
+    return ctx->item_cap >= 0 ? ctx->item_cap : auto_item_cap(n);
 }
 }  // namespace hacc
 
@@ -244,7 +247,7 @@ size_t scan_tmp_elems(int64_t len);
 constexpr int kItemClasses = 16;
 constexpr int64_t kHeavyFirstMinN = (int64_t)1 << 20;   // smaller calls keep the plain order
 cudaError_t items_heavy_first(const BinBuffers &b, int64_t max_items, cudaStream_t s);
-int64_t max_items(int64_t n, int64_t ncell);
+int64_t max_items(int64_t n, int64_t ncell, bool sub_order = true);
 // sub_order = false leaves out the sub-cell arrays (item_cap must then be 0).
 void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_order = true);
 
@@ -252,19 +255,18 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
 // counts, the permutation, cell starts and force work items.  vel may be
 // null (no drift).  dst may equal src.  item_cap = 0: ascending input row
 // within each cell (the stable counting sort) and items of up to kItemMax;
-// item_cap in [kItemCapMin, kItemMax]: within each cell of up to kBigCell
-// particles the rows are ordered by the particle's 4x4x4 sub-cell (Morton
-// order, z bit first; ties by input row), and the work items are runs of at
-// most item_cap particles of that order, so an item covers a compact part of
-// its cell; cells of more than split_max particles get items of up to
-// kItemMax.  sub_level (nullable, n kick counts aligned with src): order each
-// cell by (kick count, octant, input row) instead, so that the particles of a
-// kick count are consecutive.
+// item_cap in [kCluster, kItemCapMax]: within each cell of up to kBigCell
+// particles the rows are ordered by the particle's 4x4x4 sub-cell (along a
+// Hilbert curve; ties by input row), so that clusters of consecutive particles
+// are compact, and the work items are runs of at most item_cap particles (at
+// most kItemMax) cut between clusters; cells of more than split_max particles
+// get items of up to kItemMax.  sub_level (nullable, n kick counts aligned with
+// src): order each cell by (kick count, octant, input row) instead, so that the
+// particles of a kick count are consecutive.
 // sorted_input: src is in the cell order of a previous binning of the same
 // particles (the sub-cycle loop), which makes the in-cell ordering cheap.
-// With an item cap (and no kick counts), a cell that becomes one work item
-// keeps input-row order: the sub-cell order only shapes the items of cells
-// that are cut into several.
+// With an item cap (and no kick counts), a cell of a single cluster keeps
+// input-row order.
 cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const float4 *vel, float drift,
                       float4 *dst, const BinBuffers &b, int *d_flags, bool make_items, cudaStream_t s,
                       int item_cap = 0, int split_max = kDefaultSplitMax, const int32_t *sub_level = nullptr,
@@ -275,7 +277,8 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
 // pool row boxes[b].row_off + t - part_base is streamed by pre, wrapped,
 // binned into global cell cell_base + local id; dst[t] = its position,
 // id[t] = its pool row.  Work items carry the box in item.w >> 8.  item_cap
-// as for bin_build (ties in the sub-cell order by scratch index).
+// as for bin_build (ties in the sub-cell order by scratch index), or -1: each
+// box's automatic cap.
 cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int64_t ncell_total,
                             const float4 *pos_pool, const float4 *vel_pool, float4 *dst, int32_t *id,
                             const BinBuffers &b, int *d_flags, cudaStream_t s, int item_cap = 0,
@@ -353,6 +356,7 @@ struct ForceLaunch {
     const int32_t *n_items;     // device count
     const int32_t *cell_start;
     int *work_counter;          // zeroed before launch
+    bool cull = true;           // select the neighbours per cluster, else by the item's bounds alone
     int mode;
     // kModeForce: out[perm[i]] (perm null: out[i])
     float4 *out;

@@ -7,31 +7,46 @@
 // cut at s < r_cut^2 with a select instead of a branch (the paper folds the
 // cutoff test into the force evaluation the same way, with fsel).
 //
-// GPU mapping.  Work item = up to 160 particles of one cell (one warp; K of
-// them per lane, K = 1..5, in 1-8 lane groups, by cell occupancy).  Because
-// cells are numbered x-fastest, the three cells (ix-1, ix, ix+1) of each of
-// the 9 (dy, dz) rows are one contiguous run of the cell-sorted particle
-// array (a second run when the row wraps in x).  The lanes first write the
-// item's runs into a per-warp table; the runs are then staged as one stream,
-// 32 candidates per round with coalesced 16-byte loads, into a per-warp
-// shared-memory tile, keeping only the candidates within reach of the item's
-// bounding box.  Every lane reads each staged j with one broadcast 16-byte
-// shared load and evaluates it against its K particles, accumulating in FP32
-// registers.  Work items are taken from an atomic counter so that clustered
-// cells do not leave SMs idle.  With the finer mesh (stencil radius R = 2)
-// the rows are 25 and the runs 5 cells long.
+// GPU mapping.  A work item is up to 64 consecutive particles of one cell in
+// clusters of 8, run by one warp.  The binning orders each cell's particles
+// along a Hilbert curve of 4x4x4 sub-cells, so a cluster is compact: its
+// bounds are about 0.5 cell widths a side, where a whole cell's are 0.9.
+//   stage   The particles j of the neighbour cells are read in x-runs of
+//           consecutive sorted particles ((2R+1)^2 rows, a second run when a
+//           row wraps), 64 at a time; those within reach of the item's bounds
+//           go to a per-warp shared tile (ballot + prefix count).
+//   select  Per cluster, the tile's entries within reach of the cluster's own
+//           bounds are compacted into a list (a lane per entry).
+//   pairs   Four lanes hold the cluster's 8 particles, two each, and eight
+//           lane groups share the list, two entries a step: four pairs per
+//           lane and step, as two packed FP32 chains (fma.rn.f32x2), the two
+//           entries in the two halves.
+// What bounds it: the FP32 pipe and the issue slots together.  A pair of the
+// pair loop alone takes 21-22 cycles a warp and scheduler, with any number of
+// warps: 16 FMA-pipe cycles (an f32x2 operation holds the pipe two cycles, three
+// when its three operands are different registers), the rsqrt, and the select.
+// Scalar arithmetic takes 24-25.  Of a launch on 128^3 Zel'dovich particles
+// (0.91 ms), the pairs take 0.50 ms, selecting and staging 0.34 ms, the rest
+// 0.07 ms.  So every pair not evaluated counts:
+// Why clusters of 8: per particle of a Zel'dovich box, 970 candidates lie in
+// the 27 cells, 655 within reach of a cell's bounds, 390 of an 8-cluster's and
+// 285 of a 4-cluster's, 154 inside the cutoff.  A select test costs 40 warp
+// instructions per 32 entries and cluster, so 4-clusters would pay in tests
+// what they save in pairs.  Items of 64 share one staging among 8 clusters
+// (256^3 box: 6.9 ms a launch against 7.3 with items of 32, 8.6 with 16);
+// smaller calls take smaller items to spread over the chip (auto_item_cap).
+// Against one warp per cell-wide item whose lanes evaluate all that is within
+// reach of the cell (scalar, 5 particles a lane): 256^3 launch 9.3 -> 6.9 ms,
+// 128^3 1.19 -> 0.91 ms, 32^3 122 -> 57 us; 256^3 full step 53.3 -> 40.6
+// ms, 24 boxes x 4 sub-cycles 26.7 -> 19.1 ms, 32^3 force call 194 -> 141 us.
 //
-// Periodic images without rounding error: for a neighbour row that wraps on
-// the low side (cell -1 -> nc-1), the staged j coordinates get -L (they lie in
-// [2L/3, L), so x - L is exact); for a row that wraps on the high side
-// (cell nc -> 0), the i coordinates get -L instead (same argument).  Either
-// way r_ij = x_j' - x_i' carries only the rounding of one subtraction.
-//
-// Per evaluated pair (FP32): 3 FADD (r), 3 FFMA (t = s + eps), 1 MUFU rsqrt,
-// 1 FMUL + 1 FFMA (t^-3/2 - P5), 5 FFMA (P5 in t), 1 FMUL (mass; dropped when
-// all masses are equal), 1 compare, 3 predicated FFMA (accumulate inside the
-// cutoff); P5 is re-expanded in t = s + eps on the host, and the cutoff test
-// is t < fl(r_cut^2 + eps).
+// Periodic images without rounding error: an item whose cell lies within R of
+// a high face (per axis) runs in the frame moved by -L: its own particles and
+// the neighbours of unwrapped rows get -L (they lie in [L/2, L) for nc >= 4R:
+// exact; for smaller nc only particles half a cutoff or more apart are
+// rounded), those of rows that wrap high stay.  Elsewhere the neighbours of
+// rows that wrap low get -L (exact, in [2L/3, L)).  So r_ij = x_j' - x_i'
+// carries only the rounding of one subtraction.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -52,6 +67,7 @@ struct KParams {
     int *work_counter;
     int nc;
     int R;            // neighbour cells per side of a cell's own (1: 27 cells, 2: 125 cells)
+    int cull;         // 1: select per cluster; 0: by the item's bounds alone
     float L;
     float T, eps, G;
     float q0, q1, q2, q3, q4, q5;
@@ -82,328 +98,120 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     return y;
 }
 
-// The pair-force constants, held in registers for the whole item.
-struct PairConsts {
-    float eps, T, q0, q1, q2, q3, q4, q5;
+// Two FP32 values in one 64-bit register pair; each operation rounds its
+// halves as the scalar one does.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+// A value that all lanes hold, known as such to the compiler: branches and
+// loop bounds made of it stay warp-uniform (no reconvergence code).
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+// A value that all lanes hold, to be kept in a register of its own: it looks
+// like any other result of a shuffle, where a constant would be loaded and
+// doubled again in every round of the pair loop.
+__device__ __forceinline__ float keep(float v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ f32x2 keep2(float v) {
+    v = keep(v);
+    return pack2(v, v);
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+constexpr int kTile = 384;                // staged entries of a warp at most
+constexpr int kRound = 64;                // candidates staged per round
+constexpr int kRing = 128;                // list entries held: two chunks
+constexpr int kChunk = 64;                // list entries per call of the pair loop
+constexpr int kMaxClusters = kItemMax / kCluster;
+constexpr int kMaxRuns = 50;              // 2 (2R+1)^2 for R = 2
+
+// A warp's shared memory.  Runs: (first, end, bits, b1) of the sorted
+// particles of each x-run, with (b2, d0) for the cell/offset form; bits 1/2/4:
+// the staged j's x/y/z get -L; in the cell/offset form bits 0-3 and 4-7 hold
+// dy + 2 and dz + 2, bits 8-13 the wrap flags (1/2/4 low in x/y/z, 8/16/32
+// high), and the x cell step of entry j is d0 + (j >= b1) + (j >= b2).
+template <bool CI, bool POT>
+struct WarpMem {
+    float4 tile[kTile];
+    float x[kRing], y[kRing], z[kRing], m[kRing];   // the list
+    float4 own[kItemMax];                 // the item's particles in its frame
+    float sum[3][kItemMax];               // and their sums
+    float4 lo[kMaxClusters + 1], hi[kMaxClusters + 1];   // bounds of its clusters, and its own (last)
+    int4 runs[kMaxRuns];
+    int2 steps[CI ? kMaxRuns : 1];
+    int tile_id[POT ? kTile : 1];         // sorted index of each entry (the j != i test of the potential)
+    int id[POT ? kRing : 1];
 };
 
-// Accumulate the interaction of one staged j (already image-shifted) with
-// the K i-particles of this lane.  UM: all masses equal (the mass is applied
-// once in the epilogue).
-template <int K, bool COUNT, bool POT, bool EPS0, bool UM>
-__device__ __forceinline__ void interact(const KParams &P, const PairConsts &C, float4 pj, int jidx, int iself, int lpg,
-                                         const float (&xi)[K],
-                                         const float (&yi)[K], const float (&zi)[K], float (&ax)[K],
-                                         float (&ay)[K], float (&az)[K], unsigned &cnt) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float dx = pj.x - xi[k];
-        float dy = pj.y - yi[k];
-        float dz = pj.z - zi[k];
-        float t = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, C.eps)));
-        float r = rsqrt_approx(t);
-        const bool in = t < C.T;
-        if (POT) {
-            // phi(s) = -(t)^(-1/2) - U(t) - phi0, U in t = s + eps
-            float u = __fmaf_rn(P.u6, t, P.u5);
-            u = __fmaf_rn(u, t, P.u4);
-            u = __fmaf_rn(u, t, P.u3);
-            u = __fmaf_rn(u, t, P.u2);
-            u = __fmaf_rn(u, t, P.u1);
-            u = __fmaf_rn(u, t, P.u0);
-            float ph = -r - u - P.phi0;
-            const bool self = jidx == iself + lpg * k;   // i's own row (sorted index)
-            ax[k] += (in && !self) ? ph * pj.w : 0.0f;
+// The item's neighbour cells as x-runs of consecutive sorted particles, one
+// lane per run: row (dz, dy) of the (2R+1)^2 rows gives run `row` (cells
+// cx-R..cx+R, or the part of them in [0, nc)) and, when rows wrap in x, run
+// span^2 + row (the wrapped part).  fr: axes on which the item runs in the
+// frame moved by -L.  Returns the number of runs.
+template <bool CI, bool POT>
+__device__ __forceinline__ int build_runs(const KParams &P, WarpMem<CI, POT> &S, int cbase, int nc, int cx, int cy,
+                                          int cz, int R, int fr, int lane) {
+    const int span = 2 * R + 1, rows = span * span;
+    const int lo = cx - R, hi = cx + R;
+    const bool wraps = lo < 0 || hi >= nc;
+    const int nrun = wraps ? 2 * rows : rows;
+    for (int q = lane; q < nrun; q += 32) {
+        const int r = q >= rows ? 1 : 0, rowi = q - r * rows;
+        const int dz = rowi / span - R, dy = rowi % span - R;
+        int rz = cz + dz, ry = cy + dy;
+        int wb = 0;   // wrap flags: 1/2/4 low in x/y/z, 8/16/32 high
+        if (rz < 0) { rz += nc; wb |= 4; }
+        else if (rz >= nc) { rz -= nc; wb |= 32; }
+        if (ry < 0) { ry += nc; wb |= 2; }
+        else if (ry >= nc) { ry -= nc; wb |= 16; }
+        const int32_t *row = P.cell_start + cbase + (rz * nc + ry) * nc;
+        int ca = lo, cb = hi + 1;   // cells [ca, cb) of the row
+        int d0 = -1;
+        if (lo < 0) {           // [0, hi], then [nc + lo, nc) wrapped low
+            ca = r ? nc + lo : 0;
+            cb = r ? nc : hi + 1;
+            if (r) wb |= 1;
+            d0 = r ? -1 : 0;
+        } else if (hi >= nc) {  // [lo, nc), then [0, hi - nc] wrapped high
+            ca = r ? 0 : lo;
+            cb = r ? hi - nc + 1 : nc;
+            if (r) wb |= 8;
+            d0 = r ? 1 : -1;
+        }
+        const int ja = row[ca], jb = row[cb];
+        int bits, b1 = jb;
+        if (CI) {
+            bits = (dy + 2) | ((dz + 2) << 4) | (wb << 8);
+            // first entries of the run's second and third cell (R = 1)
+            b1 = cb - ca > 1 ? row[ca + 1] : jb;
+            const int b2 = cb - ca > 2 ? row[ca + 2] : jb;
+            S.steps[q] = make_int2(b2, d0);
         } else {
-            float q = __fmaf_rn(C.q5, t, C.q4);
-            q = __fmaf_rn(q, t, C.q3);
-            q = __fmaf_rn(q, t, C.q2);
-            q = __fmaf_rn(q, t, C.q1);
-            q = __fmaf_rn(q, t, C.q0);
-            float f = __fmaf_rn(r * r, r, -q);          // t^(-3/2) - P5
-            if (!UM) f *= pj.w;
-            // the cutoff as a predicate on the accumulating FMAs (the paper's
-            // fsel select, without the select): pairs outside never touch the sums
-            const bool use = EPS0 ? (t < C.T && t > 0.0f) : (t < C.T);
-            if (use) {
-                ax[k] = __fmaf_rn(f, dx, ax[k]);
-                ay[k] = __fmaf_rn(f, dy, ay[k]);
-                az[k] = __fmaf_rn(f, dz, az[k]);
-            }
+            // -L on an axis: rows wrapped low, or every row not wrapped high in the moved frame
+            bits = (wb & 7) | (fr & ~(wb >> 3));
         }
-        if (COUNT) cnt += (in && jidx != iself + lpg * k) ? 1u : 0u;   // j != i
-    }
-}
-
-// Entries of a staged tile: up to 32 G entries, plus room for the up to 31
-// that a compaction round carries past a full tile.
-constexpr int kTileCap = 32 * 8 + 32;
-
-// Tile steps per pass of the pair loop (the last tile is padded with far,
-// massless entries to whole passes, so the loop has no remainder).
-template <int K>
-struct Unroll {
-    static constexpr int F = K >= 5 ? 1 : (K >= 3 ? 2 : 4);
-};
-
-// Run the warp's i-particles against the staged entries [0, nj) of buf:
-// group g takes entries g, g+G, g+2G, ... (consecutive float4 addresses
-// across groups: no bank conflicts).  ids (nullable): sorted index of each
-// entry, for the j != i tests of the counting and potential forms.
-template <int K, bool COUNT, bool POT, bool EPS0, bool UM, int U>
-__device__ __forceinline__ void run_tile(const KParams &P, const PairConsts &C, const float4 *buf, const int *ids,
-                                         int nj, int iself, int lg, int grp, const float (&xs)[K],
-                                         const float (&ys)[K], const float (&zs)[K], float (&ax)[K], float (&ay)[K],
-                                         float (&az)[K], unsigned &cnt) {
-    const int G = 1 << lg;
-    const int lpg = 32 >> lg;
-    // entries per group (interleaved); the pointer-stepped loop runs whole passes
-    const int tg = U == 2 ? (nj + G * Unroll<K>::F - 1) / (G * Unroll<K>::F) * Unroll<K>::F : (nj + G - 1) >> lg;
-    constexpr int kUnroll = U == 1 ? (K >= 3 ? 1 : 2) : (K >= 5 ? 1 : (K >= 3 ? 2 : 4));
-    if (U == 2) {
-        // pointer-stepped loop over the group's entries g, g+G, ..., F entries a
-        // pass (the tile holds whole passes: no remainder)
-        constexpr int F = Unroll<K>::F;
-        const float4 *q = buf + grp;
-        int e = grp;
-#pragma unroll 1
-        for (int t = 0; t < tg; t += F) {
-#pragma unroll
-            for (int u = 0; u < F; ++u) {
-                const int jidx = (COUNT || POT) && e + u * G < nj ? ids[e + u * G] : -1;
-                interact<K, COUNT, POT, EPS0, UM>(P, C, q[u * G], jidx, iself, lpg, xs, ys, zs, ax, ay, az, cnt);
-            }
-            q += F * G;
-            e += F * G;
-        }
-    } else {
-        const float4 *bp = buf + grp;
-#pragma unroll kUnroll
-        for (int t = 0; t < tg; ++t) {
-            const int e = grp + (t << lg);
-            const int jidx = (COUNT || POT) && e < nj ? ids[e] : -1;
-            interact<K, COUNT, POT, EPS0, UM>(P, C, bp[t << lg], jidx, iself, lpg, xs, ys, zs, ax, ay, az, cnt);
-        }
-    }
-}
-
-// The neighbour cells of an item as x-runs of consecutive sorted particles:
-// row (dz, dy) of the (2R+1)^2 rows gives run 2*row (cells cx-R..cx+R, or the
-// part of them in [0, nc) when the row wraps in x) and run 2*row+1 (the
-// wrapped part, else empty).  One table per warp in shared memory:
-//   A = (exclusive end of the run in the item's concatenated stream,
-//        offset j - t of its entries, shift bits, unused)
-//   shift bits: 1/2/4 add -L to the staged j's x/y/z, 8/16/32 add -L to
-//   the i side (runs of cells within R of a high face); with in-cell
-//   offsets (CI) bits 0-3 and 4-7 hold dy + 2 and dz + 2 instead, bits 8-13
-//   the same six wrap flags (there they move the i side by +delta for a low
-//   wrap and -delta for a high one), and B = (b1, b2, d0): the x cell step of
-//   entry j is d0 + (j >= b1) + (j >= b2).
-constexpr int kMaxRuns = 64;   // 2 (2R+1)^2 <= 50 for R <= 2
-
-struct RunTable {
-    int4 *A;
-    int4 *B;
-    float4 *bnd;   // [0], [1]: the item's bounds (lx, ly, lz, -), (hx, hy, hz, -); [2], [3]: shifted, keep_r2 in [2].w
-};
-
-
-// Stream the runs [r0, r1) of the table (all with the same i shift tx, ty,
-// tz) through the warp's shared tile.  The warp is split into G = 2^lg lane
-// groups that share the i-particles and split the j.  Staging keeps only the
-// j that can be within the cutoff of some i of the item: farther than r_cut
-// (with a margin far above rounding) from the item's bounding box, a j is
-// outside the cutoff of every i and would add exactly nothing, so dropping it
-// leaves every pair sum unchanged; the kept j are compacted in stream order
-// (ballot + prefix count) into full tiles, which carry over to the next call
-// (fill, warp-uniform) until `last`.  With in-cell offsets (CI) the test runs
-// in the frame of i's cell, where both the bounds and the staged j live.
-// U selects the inner-loop form (the autotuner picks): 0 deep-unrolled and 1
-// light-unrolled indexed loops, 2 pointer-stepped loop; every form visits the
-// same entries in the same order.  (The lane-group count as a compile-time
-// constant, four times the code, measured 2x slower from instruction-cache
-// misses.)
-template <int K, bool COUNT, bool POT, bool EPS0, bool UM, int U, bool CI>
-__device__ __forceinline__ void process_runs(const KParams &P, const RunTable &rt, int r0, int r1, float L, float tx,
-                                             float ty, float tz, int iself, int i_end, int lg, int grp,
-                                             float (&xs)[K], float (&ys)[K], float (&zs)[K],
-                                             float (&ax)[K], float (&ay)[K], float (&az)[K], unsigned &cnt,
-                                             unsigned &jsum, float4 *buf, int *ids, int lane, int &fill, bool last) {
-    const bool ishift = (tx != 0.0f) || (ty != 0.0f) || (tz != 0.0f);
-    const int G = 1 << lg;
-    // the i shift is applied in place and undone by reloading the coordinates
-    // after the runs (no second copy of them in registers)
-    if (ishift) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            xs[k] = __fadd_rn(xs[k], tx);
-            ys[k] = __fadd_rn(ys[k], ty);
-            zs[k] = __fadd_rn(zs[k], tz);
-        }
-    }
-    const PairConsts C{P.eps, P.T, P.q0, P.q1, P.q2, P.q3, P.q4, P.q5};
-    const float4 dummy = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // far away, zero mass
-    const int tile = 32 << lg;
-    // the item's bounds in this frame (monotone rounding keeps them bounds),
-    // held in the warp's shared slots rather than in registers across the tiles
-    if (lane == 0) {
-        const float4 l = rt.bnd[0], h = rt.bnd[1];
-        rt.bnd[2] = make_float4(__fadd_rn(l.x, tx), __fadd_rn(l.y, ty), __fadd_rn(l.z, tz), P.T * 1.001f + 1e-3f);
-        rt.bnd[3] = make_float4(__fadd_rn(h.x, tx), __fadd_rn(h.y, ty), __fadd_rn(h.z, tz), 0.0f);
+        S.runs[q] = make_int4(ja, jb, bits, b1);
     }
     __syncwarp();
-    const unsigned below = (1u << lane) - 1u;
-    const int t_end = rt.A[r1 - 1].x;
-    int t0 = r0 > 0 ? rt.A[r0 - 1].x : 0;
-    int cur = r0;   // this lane's run
-#pragma unroll 1
-    while (true) {
-        // stage 32 candidates at a time until a tile is full or the runs end
-#pragma unroll 1
-        while (fill < tile && t0 < t_end) {
-            const int t = t0 + lane;
-            bool keep = false;
-            float4 v = dummy;
-            int j = -1;
-            if (t < t_end) {
-                while (t >= rt.A[cur].x) ++cur;
-                const int4 a = rt.A[cur];
-                j = t + a.y;
-                v = P.pos[j];
-                if (CI) {
-                    // in-cell offsets: move j into the frame of i's cell by whole
-                    // cell steps of the FP32 width w (the x step depends on which of
-                    // the run's cells j sits in).  For a j within reach of i's cell
-                    // the sum lands in a binade no finer than the offset's, so it is
-                    // exact: a close pair across a face gets its separation with one
-                    // rounding at most, like a pair inside a cell.
-                    const int4 b = rt.B[cur];
-                    const float dlt = (float)(b.z + (j >= b.x) + (j >= b.y));
-                    v.x = __fadd_rn(v.x, dlt * P.w);
-                    v.y = __fadd_rn(v.y, (float)((a.z & 15) - 2) * P.w);
-                    v.z = __fadd_rn(v.z, (float)(((a.z >> 4) & 15) - 2) * P.w);
-                } else if (a.z & 7) {
-                    if (a.z & 1) v.x = __fadd_rn(v.x, -L);
-                    if (a.z & 2) v.y = __fadd_rn(v.y, -L);
-                    if (a.z & 4) v.z = __fadd_rn(v.z, -L);
-                }
-                const float4 lo = rt.bnd[2], hi = rt.bnd[3];
-                const float ex = fmaxf(fmaxf(lo.x - v.x, v.x - hi.x), 0.0f);
-                const float ey = fmaxf(fmaxf(lo.y - v.y, v.y - hi.y), 0.0f);
-                const float ez = fmaxf(fmaxf(lo.z - v.z, v.z - hi.z), 0.0f);
-                keep = __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, ez * ez)) < lo.w;
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int at = fill + __popc(m & below);
-                buf[at] = v;
-                if (COUNT || POT) ids[at] = j;
-            }
-            fill += __popc(m);
-            t0 += 32;
-        }
-        // a partial tile waits for the next call unless this is the last one
-        if (fill < tile && !last) break;
-        const int nj = min(fill, tile);
-        if (nj == 0) break;
-        // a short last tile is padded to whole passes of the pair loop (Unroll<K>::F
-        // entries per lane group) with far, massless entries
-        const int step = G * Unroll<K>::F;
-        const int padded = (nj + step - 1) / step * step;
-        if (nj < tile && lane < padded - nj) buf[nj + lane] = dummy;
-        __syncwarp();
-        run_tile<K, COUNT, POT, EPS0, UM, U>(P, C, buf, ids, nj, iself, lg, grp, xs, ys, zs, ax, ay, az, cnt);
-        __syncwarp();
-        if (COUNT) jsum += nj;
-        // carry the entries past the tile to the front
-        const int rest = fill - nj;
-        float4 cv = dummy;
-        int ci = 0;
-        if (lane < rest) {
-            cv = buf[nj + lane];
-            if (COUNT || POT) ci = ids[nj + lane];
-        }
-        __syncwarp();
-        if (lane < rest) {
-            buf[lane] = cv;
-            if (COUNT || POT) ids[lane] = ci;
-        }
-        fill = rest;
-        if (t0 >= t_end && fill == 0) break;
-    }
-    __syncwarp();
-    if (ishift) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int i = iself + (32 >> lg) * k;
-            const float4 p = i < i_end ? P.pos[i] : make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
-            xs[k] = p.x;
-            ys[k] = p.y;
-            zs[k] = p.z;
-        }
-    }
-}
-
-// Write the run table of cell (cx, cy, cz) (of the box whose cells start at
-// cbase) for stencil radius R, one run per lane; returns the number of runs.
-template <bool CI>
-__device__ __forceinline__ int build_runs(const KParams &P, const RunTable &rt, int cbase, int nc, int cx, int cy,
-                                          int cz, int R, int lane) {
-    const int span = 2 * R + 1;
-    const int nrun = 2 * span * span;
-    int run_end = 0;   // running total of the run lengths written so far
-    for (int q0 = 0; q0 < nrun; q0 += 32) {
-        const int q = q0 + lane;
-        int ja = 0, jb = 0, bits = 0, b1 = 0, b2 = 0, d0 = 0;
-        if (q < nrun) {
-            const int rowi = q >> 1, r = q & 1;
-            const int dz = rowi / span - R, dy = rowi % span - R;
-            int rz = cz + dz, ry = cy + dy;
-            int wb = 0;   // wrap flags: 1/2/4 low in x/y/z, 8/16/32 high
-            if (rz < 0) { rz += nc; wb |= 4; }
-            else if (rz >= nc) { rz -= nc; wb |= 32; }
-            if (ry < 0) { ry += nc; wb |= 2; }
-            else if (ry >= nc) { ry -= nc; wb |= 16; }
-            const int32_t *row = P.cell_start + cbase + (rz * nc + ry) * nc;
-            // cells lo..hi of this row: one run, or two when it wraps in x
-            const int lo = cx - R, hi = cx + R;
-            const bool wraps = lo < 0 || hi >= nc;
-            if (lo < 0) {           // [0, hi], then [nc + lo, nc) with j shifted by -L
-                ja = r ? row[nc + lo] : row[0];
-                jb = r ? row[nc] : row[hi + 1];
-                if (r) wb |= 1;
-                b1 = r ? jb : row[1];
-                d0 = r ? -1 : 0;
-            } else if (hi >= nc) {  // [lo, nc), then [0, hi - nc] with i shifted by -L
-                ja = r ? row[0] : row[lo];
-                jb = r ? row[hi - nc + 1] : row[nc];
-                if (r) wb |= 8;
-                b1 = r ? jb : row[nc - 1];
-                d0 = r ? 1 : -1;
-            } else if (r == 0) {
-                ja = row[lo];
-                jb = row[hi + 1];
-                b1 = row[cx];
-                d0 = -1;
-            }
-            b2 = wraps ? jb : (r == 0 ? row[cx + 1] : 0);
-            bits = CI ? ((dy + 2) | ((dz + 2) << 4) | (wb << 8)) : wb;
-        }
-        // exclusive ends of the runs in the concatenated stream
-        int e = jb - ja;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, e, o);
-            if (lane >= o) e += y;
-        }
-        e += run_end;
-        if (q < nrun) {
-            rt.A[q] = make_int4(e, ja - (e - (jb - ja)), bits, 0);
-            if (CI) rt.B[q] = make_int4(b1, b2, d0, 0);
-        }
-        run_end = __shfl_sync(0xffffffffu, e, 31);
-    }
-    __syncwarp();
-    return nrun;
+    return uniform(nrun);
 }
 
 // Apply the force on sorted particle i (position x, y, z, mass m) as the
@@ -456,237 +264,532 @@ __device__ __forceinline__ void write_result(const KParams &P, int i, float gx, 
     }
 }
 
-template <int K, bool COUNT, bool POT, bool EPS0, bool UM, int U, bool CI>
-__device__ void process_item(const KParams &P, int4 item, float4 *buf, int *ids, const RunTable &rt, int lane,
-                             float m_uniform) {
+// Squared distance of v from the box [lo, hi].  A j is dropped when it reaches
+// a limit that carries a margin far above the rounding of the coordinates: it
+// is outside the cutoff of every i of the box and would have added exactly
+// nothing.
+__device__ __forceinline__ float box_dist2(float4 v, float4 lo, float4 hi) {
+    const float ex = v.x - fminf(fmaxf(v.x, lo.x), hi.x);
+    const float ey = v.y - fminf(fmaxf(v.y, lo.y), hi.y);
+    const float ez = v.z - fminf(fmaxf(v.z, lo.z), hi.z);
+    return __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, ez * ez));
+}
+
+// Compaction of the lanes with d2 < r2 in lane order, as predicated stores
+// (no branch): put4 stores v to entry `at` + prefix of the tile, put3 its
+// coordinates (and mass with M) to the list ring; both return the number of
+// lanes that stored.  Addresses are those of shared memory.
+__device__ __forceinline__ int put4(float d2, float r2, unsigned below, unsigned tile, int at, float4 v) {
+    int n;
+    asm volatile(
+        "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+        "setp.lt.f32 p, %1, %2;\n"
+        "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+        "popc.b32 %0, m;\n"
+        "and.b32 m, m, %3;\n"
+        "popc.b32 a, m;\n"
+        "add.s32 a, a, %5;\n"
+        "mad.lo.u32 a, a, 16, %4;\n"
+        "@p st.shared.v4.f32 [a], {%6, %7, %8, %9};\n}"
+        : "=r"(n)
+        : "f"(d2), "f"(r2), "r"(below), "r"(tile), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+        : "memory");
+    return n;
+}
+
+template <bool M>
+__device__ __forceinline__ int put3(float d2, float r2, unsigned below, unsigned ring, int at, float4 v) {
+    static_assert(kRing == 128, "ring mask and array distances below");
+    int n;
+    if (M)
+        asm volatile(
+            "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+            "setp.lt.f32 p, %1, %2;\n"
+            "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+            "popc.b32 %0, m;\n"
+            "and.b32 m, m, %3;\n"
+            "popc.b32 a, m;\n"
+            "add.s32 a, a, %5;\n"
+            "and.b32 a, a, 127;\n"
+            "mad.lo.u32 a, a, 4, %4;\n"
+            "@p st.shared.f32 [a], %6;\n"
+            "@p st.shared.f32 [a + 512], %7;\n"
+            "@p st.shared.f32 [a + 1024], %8;\n"
+            "@p st.shared.f32 [a + 1536], %9;\n}"
+            : "=r"(n)
+            : "f"(d2), "f"(r2), "r"(below), "r"(ring), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+            : "memory");
+    else
+        asm volatile(
+            "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+            "setp.lt.f32 p, %1, %2;\n"
+            "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+            "popc.b32 %0, m;\n"
+            "and.b32 m, m, %3;\n"
+            "popc.b32 a, m;\n"
+            "add.s32 a, a, %5;\n"
+            "and.b32 a, a, 127;\n"
+            "mad.lo.u32 a, a, 4, %4;\n"
+            "@p st.shared.f32 [a], %6;\n"
+            "@p st.shared.f32 [a + 512], %7;\n"
+            "@p st.shared.f32 [a + 1024], %8;\n}"
+            : "=r"(n)
+            : "f"(d2), "f"(r2), "r"(below), "r"(ring), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z)
+            : "memory");
+    return n;
+}
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ float4 shift4(float4 v, float tx, float ty, float tz) {
+    return make_float4(__fadd_rn(v.x, tx), __fadd_rn(v.y, ty), __fadd_rn(v.z, tz), v.w);
+}
+
+// The pair-force constants, doubled: eps and P5's negated coefficients.
+struct PairConsts {
+    f32x2 eps, c0, c1, c2, c3, c4, c5;
+};
+
+// This lane's two particles: their negated coordinates, doubled, and their
+// sums over the list entries the lane's group took (one sum per half).
+struct Pair {
+    f32x2 nx[2], ny[2], nz[2];
+    f32x2 ax[2], ay[2], az[2];
+};
+
+__device__ __forceinline__ f32x2 lds2(unsigned addr, int off) {
+    f32x2 r;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(r) : "r"(addr + off));
+    return r;
+}
+
+// One step: an entry pair per lane group (x, y, z[, m] of the two entries at
+// `addr` and the following arrays of the list) against the lane's particles.
+template <bool COUNT, bool EPS0, bool UM>
+__device__ __forceinline__ void pair_step(const PairConsts &C, float T, unsigned addr, Pair &A, unsigned &cnt) {
+    const f32x2 X = lds2(addr, 0), Y = lds2(addr, 4 * kRing), Z = lds2(addr, 8 * kRing);
+    f32x2 M = 0ull;
+    if (!UM) M = lds2(addr, 12 * kRing);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const f32x2 dx = add2(X, A.nx[k]), dy = add2(Y, A.ny[k]), dz = add2(Z, A.nz[k]);
+        const f32x2 t2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, C.eps)));
+        float t0, t1;
+        unpack2(t2, t0, t1);
+        const f32x2 r = pack2(rsqrt_approx(t0), rsqrt_approx(t1));
+        f32x2 q = fma2(C.c5, t2, C.c4);   // -P5
+        q = fma2(q, t2, C.c3);
+        q = fma2(q, t2, C.c2);
+        q = fma2(q, t2, C.c1);
+        q = fma2(q, t2, C.c0);
+        f32x2 f = fma2(mul2(r, r), r, q);   // t^(-3/2) - P5
+        if (!UM) f = mul2(f, M);
+        // the cutoff as a select on f (the paper's fsel)
+        const bool in0 = EPS0 ? (t0 < T && t0 > 0.0f) : t0 < T, in1 = EPS0 ? (t1 < T && t1 > 0.0f) : t1 < T;
+        float f0, f1;
+        unpack2(f, f0, f1);
+        f = pack2(in0 ? f0 : 0.0f, in1 ? f1 : 0.0f);
+        if (COUNT) cnt += (t0 < T ? 1u : 0u) + (t1 < T ? 1u : 0u);
+        A.ax[k] = fma2(f, dx, A.ax[k]);
+        A.ay[k] = fma2(f, dy, A.ay[k]);
+        A.az[k] = fma2(f, dz, A.az[k]);
+    }
+}
+
+// The same for the pair potential: phi(s) = -t^(-1/2) - U(t) - phi0 inside
+// the cutoff, U in t = s + eps; A.ax[k] = sum_j m_j phi over j != i.
+template <bool CI, bool POT>
+__device__ __forceinline__ void potential_loop(const KParams &P, const WarpMem<CI, POT> &S, int base, int len, int grp,
+                                               int i, Pair &A) {
+#pragma unroll 1
+    for (int e = base + 2 * grp; e < base + len; e += 16) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float px, py, pz, u, ph[2];
+            unpack2(A.nx[k], px, u);
+            unpack2(A.ny[k], py, u);
+            unpack2(A.nz[k], pz, u);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float dx = S.x[e + h] + px, dy = S.y[e + h] + py, dz = S.z[e + h] + pz;
+                const float t = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, P.eps)));
+                u = __fmaf_rn(P.u6, t, P.u5);
+                u = __fmaf_rn(u, t, P.u4);
+                u = __fmaf_rn(u, t, P.u3);
+                u = __fmaf_rn(u, t, P.u2);
+                u = __fmaf_rn(u, t, P.u1);
+                u = __fmaf_rn(u, t, P.u0);
+                const bool in = t < P.T && S.id[e + h] != i + k;
+                ph[h] = in ? (-rsqrt_approx(t) - u - P.phi0) * S.m[e + h] : 0.0f;
+            }
+            A.ax[k] = add2(A.ax[k], pack2(ph[0], ph[1]));
+        }
+    }
+}
+
+// Run the item's clusters against the `fill` entries of the tile, and add
+// to their sums, with the item moved by (tx, ty, tz) in the cell/offset form.
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
+__device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S, int fill, int i0, int ni, float tx,
+                                           float ty, float tz, float r2, int lane, unsigned &cnt, unsigned &evals) {
+    const float4 far = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // outside everything, massless
+    // whole rounds of 64 entries
+    const int full = uniform((fill + kRound - 1) & ~(kRound - 1));
+    if (fill + lane < full) S.tile[fill + lane] = far;
+    if (fill + 32 + lane < full) S.tile[fill + 32 + lane] = far;
+    __syncwarp();
+    const unsigned below = (1u << lane) - 1u;
+    const int grp = lane >> 2, slot = lane & 3;
+    const unsigned ring = smem_addr(S.x), mine = ring + 8 * grp;   // the list; this group's entry pairs
+    const PairConsts C{keep2(P.eps), keep2(-P.q0), keep2(-P.q1), keep2(-P.q2),
+                       keep2(-P.q3), keep2(-P.q4), keep2(-P.q5)};
+    const float T = keep(P.T);
+#pragma unroll 1
+    for (int c0 = 0; c0 < ni; c0 += kCluster) {
+        float4 lo = S.lo[c0 / kCluster], hi = S.hi[c0 / kCluster];
+        Pair A;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float4 p = S.own[c0 + 2 * slot + k];
+            if (CI) p = shift4(p, tx, ty, tz);
+            A.nx[k] = pack2(-p.x, -p.x);
+            A.ny[k] = pack2(-p.y, -p.y);
+            A.nz[k] = pack2(-p.z, -p.z);
+            A.ax[k] = A.ay[k] = A.az[k] = 0ull;
+        }
+        if (CI) {
+            lo = shift4(lo, tx, ty, tz);
+            hi = shift4(hi, tx, ty, tz);
+        }
+        int at = 0, todo = 0;   // ring position of the next entry; entries waiting
+#pragma unroll 1
+        for (int e0 = 0; e0 < full; e0 += kRound) {
+            const int e = e0 + lane;
+            const float4 v0 = S.tile[e], v1 = S.tile[e + 32];
+            const float d0 = box_dist2(v0, lo, hi), d1 = box_dist2(v1, lo, hi);
+            const int n0 = put3<!UM>(d0, r2, below, ring, at, v0);
+            const int n1 = put3<!UM>(d1, r2, below, ring, at + n0, v1);
+            if (POT) {
+                const unsigned m0 = __ballot_sync(0xffffffffu, d0 < r2), m1 = __ballot_sync(0xffffffffu, d1 < r2);
+                if (d0 < r2) S.id[(at + __popc(m0 & below)) & (kRing - 1)] = S.tile_id[e];
+                if (d1 < r2) S.id[(at + n0 + __popc(m1 & below)) & (kRing - 1)] = S.tile_id[e + 32];
+            }
+            at += n0 + n1;
+            todo = uniform(todo + n0 + n1);
+            if (COUNT) evals += (unsigned)(n0 + n1) * (unsigned)min(kCluster, ni - c0);
+            if (todo >= kChunk) {
+                __syncwarp();
+                const int base = (at - todo) & (kRing - 1);
+                if (POT) {
+                    potential_loop<CI, POT>(P, S, base, kChunk, grp, i0 + c0 + 2 * slot, A);
+                } else {
+#pragma unroll F
+                    for (int t = 0; t < kChunk / 16; ++t)
+                        pair_step<COUNT, EPS0, UM>(C, T, mine + 4 * base + 64 * t, A, cnt);
+                }
+                todo -= kChunk;
+                __syncwarp();
+            }
+        }
+        if (todo) {   // what is left, padded to whole steps
+            const int base = (at - todo) & (kRing - 1), len = (todo + 15) & ~15;
+            if (todo + lane < len) {
+                const int q = base + todo + lane;
+                S.x[q] = S.y[q] = S.z[q] = 1e18f;
+                S.m[q] = 0.0f;
+                if (POT) S.id[q] = -1;
+            }
+            __syncwarp();
+            if (POT) {
+                potential_loop<CI, POT>(P, S, base, len, grp, i0 + c0 + 2 * slot, A);
+            } else {
+                unsigned q = mine + 4 * base;
+#pragma unroll 1
+                for (int t = 0; t < len; t += 16, q += 64) pair_step<COUNT, EPS0, UM>(C, T, q, A, cnt);
+            }
+            __syncwarp();
+        }
+        // sum over the eight groups: the halves of the warp first exchange one
+        // particle each, then lanes of a half add up
+        float s[6];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float u, v;
+            unpack2(A.ax[k], u, v);
+            s[3 * k] = u + v;
+            unpack2(A.ay[k], u, v);
+            s[3 * k + 1] = u + v;
+            unpack2(A.az[k], u, v);
+            s[3 * k + 2] = u + v;
+        }
+        const bool up = lane & 16;
+#pragma unroll
+        for (int k = 0; k < (POT ? 1 : 3); ++k) {
+            const float give = up ? s[k] : s[3 + k];
+            float a = (up ? s[3 + k] : s[k]) + __shfl_xor_sync(0xffffffffu, give, 16);
+            a += __shfl_xor_sync(0xffffffffu, a, 8);
+            a += __shfl_xor_sync(0xffffffffu, a, 4);
+            if ((lane & 12) == 0) S.sum[k][c0 + 2 * slot + (up ? 1 : 0)] += a;
+        }
+    }
+    __syncwarp();
+}
+
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
+__device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMem<CI, POT> &S, int lane,
+                                             float m_uniform) {
     // geometry: the single box of the call, or this item's box of a batch
-    // (the kick and drift factors are read again in the epilogue)
     int nc = P.nc;
     float L = P.L;
     int cbase = 0;
     if (P.boxes) {
-        const BoxDev &bx = P.boxes[item.w >> 8];
-        nc = bx.nc;
+        const BoxDev &bx = P.boxes[item.w];
+        nc = uniform(bx.nc);
         L = bx.L;
-        cbase = bx.cell_base;
+        cbase = uniform(bx.cell_base);
     }
     const int c = item.x - cbase, i0 = item.y, ni = item.z;
-    const int lg = (item.w >> 4) & 15;    // 2^lg lane groups
-    const int lpg = 32 >> lg;             // lanes per group
-    const int grp = lane >> (5 - lg);
-    const int slot = lane & (lpg - 1);
     const int cx = c % nc, cy = (c / nc) % nc, cz = c / (nc * nc);
-
-    // every group holds the same K x lpg particles of the cell (their masses
-    // are read again in the epilogue)
-    float xi[K], yi[K], zi[K];
-    float ax[K], ay[K], az[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        int q = slot + lpg * k;
-        float4 p = q < ni ? P.pos[i0 + q] : make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
-        xi[k] = p.x; yi[k] = p.y; zi[k] = p.z;
-        ax[k] = 0.0f; ay[k] = 0.0f; az[k] = 0.0f;
-    }
-    unsigned cnt = 0, jsum = 0;           // pairs inside the cutoff; j evaluated (counting form)
-    const int iself = i0 + slot;          // sorted index of this lane's k = 0 particle
-    // bounding box of the item's particles (for the j culling of the runs),
-    // kept in the warp's shared slots
+    const int R = P.boxes ? 1 : P.R;
+    // axes on which the item runs in the frame moved by -L
+    const int fr = CI ? 0 : ((cx + R >= nc ? 1 : 0) | (cy + R >= nc ? 2 : 0) | (cz + R >= nc ? 4 : 0));
     {
-        float lx = 1e30f, ly = 1e30f, lz = 1e30f, hx = -1e30f, hy = -1e30f, hz = -1e30f;
+        float4 lo = make_float4(1e30f, 1e30f, 1e30f, 0.0f), hi = make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if (slot + lpg * k < ni) {
-                lx = fminf(lx, xi[k]);
-                hx = fmaxf(hx, xi[k]);
-                ly = fminf(ly, yi[k]);
-                hy = fmaxf(hy, yi[k]);
-                lz = fminf(lz, zi[k]);
-                hz = fmaxf(hz, zi[k]);
+        for (int h = 0; h < kItemMax; h += 32) {
+            if (h >= ni) break;
+            const bool on = h + lane < ni;
+            float4 f = on ? P.pos[i0 + h + lane] : make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
+            f = shift4(f, fr & 1 ? -L : 0.0f, fr & 2 ? -L : 0.0f, fr & 4 ? -L : 0.0f);
+            S.own[h + lane] = f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) S.sum[k][h + lane] = 0.0f;
+            float4 a = on ? f : make_float4(1e30f, 1e30f, 1e30f, 0.0f);
+            float4 b = on ? f : make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
+#pragma unroll
+            for (int o = 1; o < kCluster; o <<= 1) {
+                a.x = fminf(a.x, __shfl_xor_sync(0xffffffffu, a.x, o));
+                b.x = fmaxf(b.x, __shfl_xor_sync(0xffffffffu, b.x, o));
+                a.y = fminf(a.y, __shfl_xor_sync(0xffffffffu, a.y, o));
+                b.y = fmaxf(b.y, __shfl_xor_sync(0xffffffffu, b.y, o));
+                a.z = fminf(a.z, __shfl_xor_sync(0xffffffffu, a.z, o));
+                b.z = fmaxf(b.z, __shfl_xor_sync(0xffffffffu, b.z, o));
             }
+            if ((lane & (kCluster - 1)) == 0) {
+                S.lo[(h + lane) / kCluster] = a;
+                S.hi[(h + lane) / kCluster] = b;
+            }
+            lo = make_float4(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z), 0.0f);
+            hi = make_float4(fmaxf(hi.x, b.x), fmaxf(hi.y, b.y), fmaxf(hi.z, b.z), 0.0f);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
-            hx = fmaxf(hx, __shfl_xor_sync(0xffffffffu, hx, o));
-            ly = fminf(ly, __shfl_xor_sync(0xffffffffu, ly, o));
-            hy = fmaxf(hy, __shfl_xor_sync(0xffffffffu, hy, o));
-            lz = fminf(lz, __shfl_xor_sync(0xffffffffu, lz, o));
-            hz = fmaxf(hz, __shfl_xor_sync(0xffffffffu, hz, o));
-        }
-        if (lane == 0) {
-            rt.bnd[0] = make_float4(lx, ly, lz, 0.0f);
-            rt.bnd[1] = make_float4(hx, hy, hz, 0.0f);
+#pragma unroll
+        for (int o = kCluster; o < 32; o <<= 1) {
+            lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+            hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+            lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+            hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+            lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+            hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
         }
         __syncwarp();
+        // the item's bounds; with no cull, every cluster's as well
+        if (lane == kMaxClusters || (!P.cull && lane < kMaxClusters)) {
+            S.lo[lane] = lo;
+            S.hi[lane] = hi;
+        }
     }
-
-    // neighbour cells cx-R..cx+R (R = 1: 27 cells; R = 2: 125 cells of a mesh twice as fine)
-    const int R = P.boxes ? 1 : P.R;
-    const int nrun = build_runs<CI>(P, rt, cbase, nc, cx, cy, cz, R, lane);
-    // Tiles run on across all runs unless a run shifts the i side (cells
-    // within R of the high faces; with in-cell offsets, cells next to any face
-    // when the mesh has a wrap remainder): then every run ends its own tile.
-    const bool carry = CI ? (P.delta == 0.0f || (cx >= R && cy >= R && cz >= R && cx + R < nc && cy + R < nc &&
-                                                 cz + R < nc))
-                          : (cx + R < nc && cy + R < nc && cz + R < nc);
+    const float r2 = P.T * 1.001f + 1e-3f;
+    const int nrun = build_runs<CI, POT>(P, S, cbase, nc, cx, cy, cz, R, fr, lane);
+    // In the cell/offset form a wrapped neighbour lies the remainder L - nc w
+    // beyond the whole cell steps: moving i by it instead keeps the j side
+    // exact (the shifted i is exact too for any i within reach of the face),
+    // so a change of the shift between runs ends a tile.
+    const bool moves = CI && P.delta != 0.0f &&
+                       !(cx >= R && cy >= R && cz >= R && cx + R < nc && cy + R < nc && cz + R < nc);
+    float tx = 0.0f, ty = 0.0f, tz = 0.0f;
+    unsigned cnt = 0, evals = 0;
+    const unsigned below = (1u << lane) - 1u, tile = smem_addr(S.tile);
     int fill = 0;
-#pragma unroll 1
-    for (int q = 0; q < nrun;) {
-        // all runs at once, or one run with its own i shift
-        const int q1 = carry ? nrun : q + 1;
-        const int bits = carry ? 0 : rt.A[q].z;
-        float tx, ty, tz;
-        if (CI) {
-            // a wrapped neighbour lies L - nc w beyond the whole cell steps:
-            // moving i by it instead keeps the j side exact (the shifted i is
-            // exact too for any i within reach of the face)
-            const int wb = bits >> 8;
-            tx = (wb & 1) ? P.delta : ((wb & 8) ? -P.delta : 0.0f);
-            ty = (wb & 2) ? P.delta : ((wb & 16) ? -P.delta : 0.0f);
-            tz = (wb & 4) ? P.delta : ((wb & 32) ? -P.delta : 0.0f);
-        } else {
-            tx = (bits & 8) ? -L : 0.0f;
-            ty = (bits & 16) ? -L : 0.0f;
-            tz = (bits & 32) ? -L : 0.0f;
-        }
-        if (rt.A[q1 - 1].x > (q > 0 ? rt.A[q - 1].x : 0))   // not empty
-            process_runs<K, COUNT, POT, EPS0, UM, U, CI>(P, rt, q, q1, L, tx, ty, tz, iself, i0 + ni, lg, grp,
-                                                         xi, yi, zi, ax, ay, az, cnt, jsum, buf, ids, lane, fill, true);
-        q = q1;
-    }
-
-    // sum the groups' partial forces (the groups saw disjoint j)
-    for (int o = 16; o >= lpg; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            ax[k] += __shfl_xor_sync(0xffffffffu, ax[k], o);
-            ay[k] += __shfl_xor_sync(0xffffffffu, ay[k], o);
-            az[k] += __shfl_xor_sync(0xffffffffu, az[k], o);
-        }
-    }
-
-    // epilogue (group 0 writes)
-    if (grp == 0) {
-        float h_kick = P.h_kick, h_drift = P.h_drift;
-        if (P.boxes) {
-            const BoxDev &bx = P.boxes[item.w >> 8];
-            h_kick = bx.h;
-            h_drift = bx.post;
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            int q = slot + lpg * k;
-            if (q >= ni) continue;
-            int i = i0 + q;
-            const float mi = P.pos[i].w;
-            if (POT) {
-                P.phi_out[i] = 0.5f * P.G * mi * ax[k];
-                continue;
+    // the stream of rounds: 64 particles of a run (past its end: its last one
+    // again, never kept); the next round's loads are in flight while this one's
+    // are tested
+    int q = -1, j0 = 0, end = 0, bits = 0, b1 = 0;
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f;   // shift of the run's particles
+    auto next = [&]() -> bool {
+        j0 += kRound;
+        while (j0 >= end) {
+            if (++q >= nrun) return false;
+            const int4 run = S.runs[q];
+            j0 = uniform(run.x);
+            end = uniform(run.y);
+            bits = uniform(run.z);
+            b1 = run.w;
+            if (!CI) {
+                sx = (bits & 1) ? -L : 0.0f;
+                sy = (bits & 2) ? -L : 0.0f;
+                sz = (bits & 4) ? -L : 0.0f;
             }
+        }
+        return true;
+    };
+    float4 n0, n1;
+    auto load = [&]() {
+        n0 = P.pos[min(j0 + lane, end - 1)];
+        n1 = P.pos[min(j0 + 32 + lane, end - 1)];
+    };
+    bool more = next();
+    if (more) load();
+#pragma unroll 1
+    while (more) {
+        float4 v[2] = {n0, n1};
+        if (!CI) {
+            v[0] = shift4(v[0], sx, sy, sz);
+            v[1] = shift4(v[1], sx, sy, sz);
+        }
+        const int j = j0 + lane, left = end - j0, run_bits = bits, step1 = b1;
+        int2 st = make_int2(0, 0);
+        if (CI) st = S.steps[q];
+        // no flush after this round?  Then its successor's loads start now, else
+        // after the flush (held across it, they would cost it eight registers)
+        const bool calm = fill <= kTile - 2 * kRound;
+        more = next();
+        if (more && calm) load();
+        if (CI) {
+            sy = (float)((run_bits & 15) - 2) * P.w;
+            sz = (float)(((run_bits >> 4) & 15) - 2) * P.w;
+            if (moves) {
+                const int wb = run_bits >> 8;
+                const float ux = (wb & 1) ? P.delta : ((wb & 8) ? -P.delta : 0.0f);
+                const float uy = (wb & 2) ? P.delta : ((wb & 16) ? -P.delta : 0.0f);
+                const float uz = (wb & 4) ? P.delta : ((wb & 32) ? -P.delta : 0.0f);
+                if (ux != tx || uy != ty || uz != tz) {
+                    if (fill)
+                        flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+                    fill = 0;
+                    tx = ux;
+                    ty = uy;
+                    tz = uz;
+                }
+            }
+        }
+        float4 lo = S.lo[kMaxClusters], hi = S.hi[kMaxClusters];
+        if (CI) {
+            lo = shift4(lo, tx, ty, tz);
+            hi = shift4(hi, tx, ty, tz);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h && left <= 32) break;
+            if (CI) {
+                // whole cell steps of the FP32 width w move j into the frame of i's
+                // cell: exact for a j within reach of i's cell, so a close pair
+                // across a face gets its separation with one rounding at most
+                const int jj = j + 32 * h;
+                const float d = (float)(st.y + (jj >= step1) + (jj >= st.x));
+                v[h] = shift4(v[h], d * P.w, sy, sz);
+            }
+            const float d2 = box_dist2(v[h], lo, hi), lim = lane + 32 * h < left ? r2 : 0.0f;
+            if (POT) {
+                const unsigned m = __ballot_sync(0xffffffffu, d2 < lim);
+                if (d2 < lim) S.tile_id[fill + __popc(m & below)] = j + 32 * h;
+            }
+            fill = uniform(fill + put4(d2, lim, below, tile, fill, v[h]));
+        }
+        if (!calm) {
+            if (fill > kTile - kRound) {
+                flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+                fill = 0;
+            }
+            if (more) load();
+        }
+    }
+    if (fill) flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+
+    // epilogue: a particle per lane
+#pragma unroll
+    for (int h = 0; h < kItemMax / 32; ++h) {
+        if (32 * h + lane >= ni) continue;
+        const int i = i0 + 32 * h + lane;
+        const float4 p = P.pos[i];
+        if (POT) {
+            P.phi_out[i] = 0.5f * P.G * p.w * S.sum[0][32 * h + lane];
+        } else {
             const float gm = UM ? P.G * m_uniform : P.G;
-            write_result(P, i, gm * ax[k], gm * ay[k], gm * az[k], xi[k], yi[k], zi[k], mi, h_kick, h_drift, L);
+            float h_kick = P.h_kick, h_drift = P.h_drift;
+            if (P.boxes) {
+                h_kick = P.boxes[item.w].h;
+                h_drift = P.boxes[item.w].post;
+            }
+            write_result(P, i, gm * S.sum[0][32 * h + lane], gm * S.sum[1][32 * h + lane], gm * S.sum[2][32 * h + lane],
+                         p.x, p.y, p.z, p.w, h_kick, h_drift, L);
         }
     }
     if (COUNT) {
+        // every particle met itself once (t = eps), which is no pair
         unsigned long long c64 = cnt;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c64 += __shfl_down_sync(0xffffffffu, c64, o);
-        if (lane == 0) atomicAdd(P.within, c64);
-        if (lane == 0 && P.evaluated) atomicAdd(P.evaluated, (unsigned long long)jsum * (unsigned long long)ni);
+        if (lane == 0) atomicAdd(P.within, P.eps < P.T ? c64 - (unsigned long long)ni : c64);
+        if (lane == 0 && P.evaluated) atomicAdd(P.evaluated, (unsigned long long)evals);
     }
+    __syncwarp();
 }
 
-template <bool COUNT, bool POT, bool EPS0, bool UM, int U, bool CI = false>
-__device__ __forceinline__ void work_loop(const KParams &P, float4 *buf, int *ids, const RunTable &rt, int lane,
-                                          float m_uniform) {
-    const int n_items = *P.n_items;
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
+__device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S, int lane, float m_uniform) {
+    const int n_items = uniform(*P.n_items);
     while (true) {
         int it = 0;
         if (lane == 0) it = atomicAdd(P.work_counter, 1);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= n_items) break;
         int4 item = P.items[P.order ? P.order[it] : it];
-        switch (item.w & 15) {
-            case 1: process_item<1, COUNT, POT, EPS0, UM, U, CI>(P, item, buf, ids, rt, lane, m_uniform); break;
-            case 2: process_item<2, COUNT, POT, EPS0, UM, U, CI>(P, item, buf, ids, rt, lane, m_uniform); break;
-            case 3: process_item<3, COUNT, POT, EPS0, UM, U, CI>(P, item, buf, ids, rt, lane, m_uniform); break;
-            case 4: process_item<4, COUNT, POT, EPS0, UM, U, CI>(P, item, buf, ids, rt, lane, m_uniform); break;
-            default: process_item<5, COUNT, POT, EPS0, UM, U, CI>(P, item, buf, ids, rt, lane, m_uniform); break;
-        }
+        item.x = uniform(item.x);
+        item.y = uniform(item.y);
+        item.z = uniform(item.z);
+        item.w = uniform(item.w);
+        process_item<COUNT, POT, EPS0, UM, F, CI>(P, item, S, lane, m_uniform);
     }
 }
 
-// MINB: blocks per SM the register allocation must allow (6 -> 80, 8 -> 64,
-// 5 -> 96 registers per thread); U: unroll policy.  The autotuner picks.
-template <bool COUNT, bool POT, bool EPS0, int MINB, int U>
+// MINB: blocks per SM the register allocation must allow; F: steps of the
+// pair loop unrolled.  The autotuner picks.
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI>
 __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
-    __shared__ float4 tiles[kWarps][kTileCap];
-    __shared__ int tile_ids[COUNT || POT ? kWarps : 1][kTileCap];
-    __shared__ int4 runs[kWarps][kMaxRuns];
-    __shared__ float4 bnd[kWarps][4];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float4 *buf = tiles[w];
-    int *ids = tile_ids[COUNT || POT ? w : 0];
-    const RunTable rt{runs[w], nullptr, bnd[w]};
+    extern __shared__ __align__(16) char smem[];
+    WarpMem<CI, POT> *S = reinterpret_cast<WarpMem<CI, POT> *>(smem) + uniform(threadIdx.x >> 5);
+    const int lane = __shfl_xor_sync(0xffffffffu, (threadIdx.x & 31) ^ 1, 1);   // as with uniform(): kept
     // equal masses (flag left 0 by the binning pass): apply the mass once per i
-    if (!POT && P.mass_flag && *P.mass_flag == 0 && *P.n_items > 0)
-        work_loop<COUNT, POT, EPS0, true, U>(P, buf, ids, rt, lane, P.pos[0].w);
+    if (!POT && P.mass_flag && uniform(*P.mass_flag) == 0 && uniform(*P.n_items) > 0)
+        work_loop<COUNT, POT, EPS0, !POT, F, CI>(P, *S, lane, P.pos[0].w);
     else
-        work_loop<COUNT, POT, EPS0, false, U>(P, buf, ids, rt, lane, 0.0f);
+        work_loop<COUNT, POT, EPS0, false, F, CI>(P, *S, lane, 0.0f);
 }
 
-// Positions as (cell, in-cell offset): the precision variant.
-template <bool EPS0>
-__global__ void __launch_bounds__(kThreads, 5) k_sr_force_ci(KParams P) {
-    __shared__ float4 tiles[kWarps][kTileCap];
-    __shared__ int4 runs[kWarps][kMaxRuns];
-    __shared__ int4 steps[kWarps][kMaxRuns];
-    __shared__ float4 bnd[kWarps][4];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float4 *buf = tiles[w];
-    const RunTable rt{runs[w], steps[w], bnd[w]};
-    if (P.mass_flag && *P.mass_flag == 0 && *P.n_items > 0)
-        work_loop<false, false, EPS0, true, 0, true>(P, buf, nullptr, rt, lane, P.pos[0].w);
-    else
-        work_loop<false, false, EPS0, false, 0, true>(P, buf, nullptr, rt, lane, 0.0f);
-}
-
-// Pair potential (diagnostics) of the precision variant.
-template <bool EPS0>
-__global__ void __launch_bounds__(kThreads, 5) k_sr_pot_ci(KParams P) {
-    __shared__ float4 tiles[kWarps][kTileCap];
-    __shared__ int tile_ids[kWarps][kTileCap];
-    __shared__ int4 runs[kWarps][kMaxRuns];
-    __shared__ int4 steps[kWarps][kMaxRuns];
-    __shared__ float4 bnd[kWarps][4];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const RunTable rt{runs[w], steps[w], bnd[w]};
-    work_loop<false, true, EPS0, false, 0, true>(P, tiles[w], tile_ids[w], rt, lane, 0.0f);
-}
-
-template <bool COUNT, bool POT, bool EPS0, int MINB, int U>
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI>
 cudaError_t launch_one(const KParams &P, int num_sms, cudaStream_t s) {
+    auto *k = k_sr_force<COUNT, POT, EPS0, MINB, F, CI>;
+    const size_t bytes = kWarps * sizeof(WarpMem<CI, POT>);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    cudaError_t e =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sr_force<COUNT, POT, EPS0, MINB, U>, kThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, bytes);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_sr_force<COUNT, POT, EPS0, MINB, U><<<num_sms * per_sm, kThreads, 0, s>>>(P);
+    k<<<num_sms * per_sm, kThreads, bytes, s>>>(P);
     note_launch();
     return cudaGetLastError();
 }
 
-// Variants 0..kForceVariants-1: (MINB, U) = (5, 0), (4, 0), (5, 2), (4, 2);
+// Variants 0..kForceVariants-1: (MINB, F) = (5, 4), (4, 4), (5, 2), (4, 2);
 // all give bitwise the same forces.
-// (A blocked tile layout, each group's entries contiguous at a padded stride,
-// measured 5% slower than these and changes the summation order.)
-template <bool COUNT, bool POT, bool EPS0>
+template <bool COUNT, bool EPS0>
 cudaError_t launch_variant(const KParams &P, int variant, int num_sms, cudaStream_t s) {
     switch (variant) {
-        case 1: return launch_one<COUNT, POT, EPS0, 4, 0>(P, num_sms, s);
-        case 2: return launch_one<COUNT, POT, EPS0, 5, 2>(P, num_sms, s);
-        case 3: return launch_one<COUNT, POT, EPS0, 4, 2>(P, num_sms, s);
-        default: return launch_one<COUNT, POT, EPS0, 5, 0>(P, num_sms, s);
+        case 1: return launch_one<COUNT, false, EPS0, 4, 4, false>(P, num_sms, s);
+        case 2: return launch_one<COUNT, false, EPS0, 5, 2, false>(P, num_sms, s);
+        case 3: return launch_one<COUNT, false, EPS0, 4, 2, false>(P, num_sms, s);
+        default: return launch_one<COUNT, false, EPS0, 5, 4, false>(P, num_sms, s);
     }
 }
 
@@ -706,6 +809,7 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     P.work_counter = fl.work_counter;
     P.nc = g.nc;
     P.R = g.R;
+    P.cull = fl.cull ? 1 : 0;
     P.L = g.Lf;
     P.T = fc.T;
     P.eps = fc.eps;
@@ -737,31 +841,19 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     const bool eps0 = !(fc.eps > 0.0f);
     const bool count = fl.within != nullptr;
     const int v = fl.variant;
-    if (fl.cell_offset && pot) {
-        int per_sm = 0;
-        cudaError_t e = eps0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sr_pot_ci<true>, kThreads, 0)
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sr_pot_ci<false>, kThreads, 0);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        if (eps0) k_sr_pot_ci<true><<<num_sms * per_sm, kThreads, 0, s>>>(P);
-        else k_sr_pot_ci<false><<<num_sms * per_sm, kThreads, 0, s>>>(P);
-        note_launch();
-        return cudaGetLastError();
-    }
-    if (fl.cell_offset) {
-        int per_sm = 0;
-        cudaError_t e = eps0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sr_force_ci<true>, kThreads, 0)
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sr_force_ci<false>, kThreads, 0);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        if (eps0) k_sr_force_ci<true><<<num_sms * per_sm, kThreads, 0, s>>>(P);
-        else k_sr_force_ci<false><<<num_sms * per_sm, kThreads, 0, s>>>(P);
-        note_launch();
-        return cudaGetLastError();
-    }
-    if (pot) return eps0 ? launch_one<false, true, true, 5, 0>(P, num_sms, s) : launch_one<false, true, false, 5, 0>(P, num_sms, s);
-    if (count) return eps0 ? launch_variant<true, false, true>(P, v, num_sms, s) : launch_variant<true, false, false>(P, v, num_sms, s);
-    return eps0 ? launch_variant<false, false, true>(P, v, num_sms, s) : launch_variant<false, false, false>(P, v, num_sms, s);
+    if (fl.cell_offset && pot)
+        return eps0 ? launch_one<false, true, true, 4, 1, true>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 1, true>(P, num_sms, s);
+    if (fl.cell_offset)
+        return eps0 ? launch_one<false, false, true, 4, 4, true>(P, num_sms, s)
+                    : launch_one<false, false, false, 4, 4, true>(P, num_sms, s);
+    if (pot)
+        return eps0 ? launch_one<false, true, true, 4, 1, false>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 1, false>(P, num_sms, s);
+    if (count)
+        return eps0 ? launch_one<true, false, true, 4, 1, false>(P, num_sms, s)
+                    : launch_one<true, false, false, 4, 1, false>(P, num_sms, s);
+    return eps0 ? launch_variant<false, true>(P, v, num_sms, s) : launch_variant<false, false>(P, v, num_sms, s);
 }
 
 // ---- FP64 diagnostics ------------------------------------------------------
