@@ -6,11 +6,11 @@
 //   k_key     wrap (after an optional drift), exact cell id, per-cell count
 //             and arrival slot (atomic), [sub-cell]        read 16-32 B, write 8-25 B
 //             (in place without a drift only moved particles are written back)
-//   scan      exclusive scan of (count, work-item count) packed in 64 bits
+//   scan      exclusive scan of (count, work-item count) packed in 64 bits, cell
+//             starts and force work items
 //   k_place   perm_tmp[start[c] + slot] = i, [its sub-cell] read 12-13 B, write 4-5 B
 //   k_order   within each cell, sort perm by input row (stable order) or by
 //             (sub-cell, input row)
-//   k_items   cell starts and force work items
 //   gather    sorted copies of positions / velocities / ids
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -151,23 +151,39 @@ __device__ __forceinline__ uint32_t items_of(uint32_t cnt, ItemRule r) {
     return (clusters_of(cnt) + per - 1) / per;
 }
 
-// Item q of m near-equal runs of the clusters of cnt particles: [a, e).
-__device__ __forceinline__ void item_range(uint32_t cnt, uint32_t m, uint32_t q, uint32_t *a, uint32_t *e) {
-    const uint64_t k = clusters_of(cnt);
-    *a = (uint32_t)(k * q / m) * kCluster;
-    *e = min(cnt, (uint32_t)(k * (q + 1) / m) * kCluster);
-}
+// Items of a cell of cnt particles whose first sorted slot is s: m near-equal
+// runs of its clusters, first(q) .. first(q + 1) (no division per item).
+struct CellItems {
+    uint32_t cnt, m, base, rem;
+    __device__ CellItems(uint32_t cnt_, uint32_t m_) : cnt(cnt_), m(m_) {
+        const uint32_t k = clusters_of(cnt);
+        base = k / m;
+        rem = k - base * m;
+    }
+    __device__ uint32_t first(uint32_t q) const { return min(cnt, (q * base + min(q, rem)) * kCluster); }
+};
 
-__global__ void __launch_bounds__(kBlock) k_pack(int64_t ncell, const uint32_t *__restrict__ count,
-                                                  unsigned long long *__restrict__ packed, ItemRule cap,
-                                                  const BoxDev *__restrict__ boxes, int nbox) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncell) return;
-    uint32_t k = count[c];
-    if (cap.clusters == 0) cap = rule_of_box(cap, boxes[box_of_cell(boxes, nbox, c)]);
-    const uint32_t it = items_of(k, cap);
-    packed[c] = (unsigned long long)k | ((unsigned long long)it << 32);
-}
+// What the scan packs per cell: (particles, work items) in 64 bits.
+struct CellPack {
+    const uint32_t *__restrict__ count;
+    ItemRule rule;
+    const BoxDev *__restrict__ boxes;
+    int nbox;
+    __device__ uint32_t items(int64_t c, uint32_t cnt, int *box) const {
+        ItemRule r = rule;
+        *box = 0;
+        if (boxes) {
+            *box = box_of_cell(boxes, nbox, c);
+            r = rule_of_box(r, boxes[*box]);
+        }
+        return items_of(cnt, r);
+    }
+    __device__ unsigned long long operator()(int64_t c) const {
+        const uint32_t k = count[c];
+        int box;
+        return k ? (unsigned long long)k | ((unsigned long long)items(c, k, &box) << 32) : 0ull;
+    }
+};
 
 // ---- exclusive scan of uint64, reduce-then-scan, 2048 values per block ----
 constexpr int kScanItems = 8;
@@ -201,13 +217,16 @@ __device__ __forceinline__ unsigned long long block_exclusive(unsigned long long
     return r;
 }
 
-__global__ void __launch_bounds__(kBlock) k_scan_reduce(int64_t len, const unsigned long long *__restrict__ in,
+// Sums of scan tiles: of the packed cells (CELLS) or of a level of block sums.
+template <bool CELLS>
+__global__ void __launch_bounds__(kBlock) k_scan_reduce(int64_t len, CellPack cells,
+                                                         const unsigned long long *__restrict__ in,
                                                          unsigned long long *__restrict__ sums) {
     int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     unsigned long long s = 0;
 #pragma unroll
     for (int j = 0; j < kScanItems; ++j)
-        if (base + j < len) s += in[base + j];
+        if (base + j < len) s += CELLS ? cells(base + j) : in[base + j];
     unsigned long long total;
     block_exclusive(s, &total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
@@ -241,11 +260,74 @@ cudaError_t scan_exclusive(unsigned long long *data, int64_t len, unsigned long 
         return cudaGetLastError();
     }
     unsigned long long *sums = tmp;
-    k_scan_reduce<<<(unsigned)nb, kBlock, 0, s>>>(len, data, sums);
+    k_scan_reduce<false><<<(unsigned)nb, kBlock, 0, s>>>(len, CellPack{}, data, sums);
     note_launch();
     cudaError_t e = scan_exclusive(sums, nb, tmp + nb, s);
     if (e != cudaSuccess) return e;
     k_scan_down<<<(unsigned)nb, kBlock, 0, s>>>(len, data, sums);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// The last pass of the scan over the cells: the packing, the cell starts and
+// the force work items as the sums come out (a thread per cell; the cells of a
+// block are taken one row of threads at a time, so that dense cells next to
+// each other meet different threads).  Before, packing and items were kernels
+// of their own that each read the cells again, and divided twice per item (32^3
+// box: 1.7 + 2.4 + 6.0 us, now 7.2; 128^3: 1.7 + 7.5 + 3.5, now 12 with one
+// launch fewer).
+__global__ void __launch_bounds__(kBlock) k_scan_cells(int64_t ncell, int64_t n, CellPack cells,
+                                                        const unsigned long long *__restrict__ offsets,
+                                                        unsigned long long *__restrict__ packed,
+                                                        int32_t *__restrict__ cell_start, int4 *__restrict__ items,
+                                                        int32_t *__restrict__ n_items) {
+    unsigned long long before = offsets ? offsets[blockIdx.x] : 0ull;
+    for (int j = 0; j < kScanItems; ++j) {
+        const int64_t c = (int64_t)blockIdx.x * kScanTile + (int64_t)j * kBlock + threadIdx.x;
+        if ((int64_t)blockIdx.x * kScanTile + (int64_t)j * kBlock >= ncell) break;   // the same for the whole block
+        uint32_t cnt = 0, m = 0;
+        int box = 0;
+        if (c < ncell) {
+            cnt = cells.count[c];
+            if (cnt) m = cells.items(c, cnt, &box);
+        }
+        const unsigned long long v = (unsigned long long)cnt | ((unsigned long long)m << 32);
+        unsigned long long total;
+        const unsigned long long at = before + block_exclusive(v, &total);
+        before += total;
+        if (c >= ncell) continue;
+        const uint32_t s = (uint32_t)at;
+        packed[c] = at;
+        cell_start[c] = (int32_t)s;
+        if (c == ncell - 1) {
+            cell_start[ncell] = (int32_t)n;
+            if (items) *n_items = (int32_t)((at >> 32) + m);
+        }
+        if (!items || !m) continue;
+        const CellItems it(cnt, m);
+        int4 *out = items + (uint32_t)(at >> 32);
+        for (uint32_t q = 0; q < m; ++q) {
+            const uint32_t a = it.first(q);
+            out[q] = make_int4((int)c, (int)(s + a), (int)(it.first(q + 1) - a), box);
+        }
+    }
+}
+
+// Scan of the cells' particle and item counts into packed, cell_start and
+// (make_items) the work items.
+cudaError_t scan_cells(int64_t ncell, int64_t n, const CellPack &cells, const BinBuffers &b, bool make_items,
+                       cudaStream_t s) {
+    const int64_t nb = (ncell + kScanTile - 1) / kScanTile;
+    const unsigned long long *offsets = nullptr;
+    cudaError_t e;
+    if (nb > 1) {
+        k_scan_reduce<true><<<(unsigned)nb, kBlock, 0, s>>>(ncell, cells, nullptr, b.scan_tmp);
+        note_launch();
+        if ((e = scan_exclusive(b.scan_tmp, nb, b.scan_tmp + nb, s)) != cudaSuccess) return e;
+        offsets = b.scan_tmp;
+    }
+    k_scan_cells<<<(unsigned)nb, kBlock, 0, s>>>(ncell, n, cells, offsets, b.packed, b.cell_start,
+                                                 make_items ? b.items : nullptr, b.n_items);
     note_launch();
     return cudaGetLastError();
 }
@@ -451,22 +533,26 @@ __global__ void __launch_bounds__(kBlock) k_order_sub(int64_t ncell, const uint3
     rank_shared(w, cnt, lane, out, RowOf64{});
 }
 
-// The in-cell order, a block per kOrdCells consecutive cells: their slots
-// form one range of the placement array, which the block stages into shared
-// memory with coalesced loads (when it holds at most kOrdCap entries; else
-// the warps read their cells' keys from global memory).  Each warp then ranks
-// one cell at a time; keys are distinct, and the slot of a key is the number
-// of smaller keys of its cell.  A cell of up to 32 keys is ranked in registers
-// by its stretches of consecutive keys when it has few (the key pass's runs),
-// else by a bitonic sort across the warp; a larger row-ordered cell tries
-// the stretch ranking in shared memory, and otherwise a cell of up to 256
-// keys is sorted by a bitonic network over 2, 4 or 8 keys per lane, a larger
-// one ranked by counting with 4 keys per lane on each pass over the cell (up
-// to kBigCell).  The key is the input row (row order), or with SUB the pair
-// (sub-cell code, input row) as one 32-bit key, code << 24 | row (codes below
-// 2^8, rows below 2^24; larger calls take k_order_sub).  Cells above kBigCell
-// are ordered by input row alone, by k_order_big (with SUB their rows are
-// copied to perm_tmp first).
+// The in-cell order, a block per run of up to kOrdCells consecutive cells
+// (fewer in small meshes, so that their few cells spread over the chip): their
+// slots form one range of the placement array, which the block stages into
+// shared memory with coalesced loads (when it holds at most kOrdCap entries;
+// else the warps read their cells' keys from global memory).  Each warp then
+// ranks one cell at a time; keys are distinct, and the slot of a key is the
+// number of smaller keys of its cell.  A cell of up to 32 keys is ranked in
+// registers by its stretches of consecutive keys when it has few (the key
+// pass's runs), else by a bitonic sort across the warp; a larger row-ordered
+// cell tries the stretch ranking in shared memory, and otherwise a cell of up to
+// 256 keys is sorted by a bitonic network over 2, 4 or 8 keys per lane.  Cells
+// of up to kBlockCell keys wait until the warps are through and are then ranked
+// by the whole block, a key per thread counting the smaller ones (by one warp, a
+// cell of 400 keys took 60 us: with the smaller blocks the pass went from 82 to 18
+// us on a 32^3 blob box and from 116 to 51 us on 2 million blob particles).  The key is the input row (row order), or
+// with SUB the pair (sub-cell code, input row) as one 32-bit key, code << 24 |
+// row (codes below 2^8, rows below 2^24; larger calls take k_order_sub).  Cells
+// above kBigCell are ordered by input row alone; those above kBlockCell by
+// k_order_big (with SUB their rows are copied to perm_tmp first).
+constexpr uint32_t kBlockCell = 2048;
 constexpr int kOrdCells = 64;
 constexpr int kOrdCap = 6144;
 constexpr int64_t kOrdSubMaxRows = (int64_t)1 << 24;
@@ -479,29 +565,6 @@ __device__ __forceinline__ uint32_t order_key(const int32_t *perm_tmp, const uns
         return ((uint32_t)(v >> 32) << 24) | (uint32_t)v;
     }
     return (uint32_t)perm_tmp[e];
-}
-
-// Ranks of the keys seg[e0 + lane + 32 k], k < J, among the cnt keys of the
-// cell (one pass over the cell feeds J comparisons per load); writes each
-// row to its slot.
-template <int J, class Seg>
-__device__ __forceinline__ void rank_lanes(const Seg &seg, uint32_t cnt, uint32_t e0, int lane, int32_t *out,
-                                           uint32_t row_mask) {
-    uint32_t v[J], r[J];
-#pragma unroll
-    for (int k = 0; k < J; ++k) {
-        const uint32_t e = e0 + lane + 32 * k;
-        v[k] = e < cnt ? seg(e) : 0xffffffffu;
-        r[k] = 0;
-    }
-    for (uint32_t u = 0; u < cnt; ++u) {
-        const uint32_t x = seg(u);
-#pragma unroll
-        for (int k = 0; k < J; ++k) r[k] += x < v[k] ? 1u : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < J; ++k)
-        if (e0 + lane + 32 * k < cnt) out[r[k]] = (int32_t)(v[k] & row_mask);
 }
 
 // Ranking by stretches.  The key pass gives each run of adjacent lanes with
@@ -580,15 +643,16 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
                                                         int32_t *__restrict__ perm, int32_t *__restrict__ big_list,
                                                         int *__restrict__ big_count,
                                                         const unsigned long long *__restrict__ order_tmp,
-                                                        uint32_t row_below, int stretches) {
-    __shared__ uint32_t keys[kOrdCap];
+                                                        uint32_t row_below, int stretches, int cells) {
+    __shared__ __align__(16) uint32_t keys[kOrdCap];
     __shared__ uint32_t heads[kBlock / 32][3][kHeads];    // a warp's stretch heads: keys, slots, ranks
     __shared__ uint32_t cstart[kOrdCells], ccount[kOrdCells];
     __shared__ int next_cell;   // the warps take the block's cells in turn (cells differ widely in cost)
-    const int64_t c0 = (int64_t)blockIdx.x * kOrdCells;
+    __shared__ int wide[kOrdCells], n_wide;   // cells for the whole block
+    const int64_t c0 = (int64_t)blockIdx.x * cells;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int ncb = ncell - c0 < kOrdCells ? (int)(ncell - c0) : kOrdCells;   // cells of this block (>= 1)
-    if (t == 0) next_cell = 0;
+    const int ncb = ncell - c0 < cells ? (int)(ncell - c0) : cells;   // cells of this block (>= 1)
+    if (t == 0) next_cell = n_wide = 0;
     if (t < kOrdCells) {
         uint32_t cnt = 0, st = 0;
         if (t < ncb) {
@@ -652,11 +716,15 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
         if (by_row && (stretches || cnt <= kStretchTryMax) &&
             rank_stretches(seg, cnt, lane, out, row_mask, heads[w][0], heads[w][1], heads[w][2]))
             continue;
-        if (cnt > kBigCell) {
+        if (cnt > kBlockCell) {
             // to the big-cell sort by row, from perm_tmp
             if (SUB)
                 for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
             if (lane == 0) big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
+            continue;
+        }
+        if (cnt > 256) {
+            if (lane == 0) wide[atomicAdd(&n_wide, 1)] = q;
             continue;
         }
         if (cnt <= 64) {
@@ -667,11 +735,31 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             sort_cell<4>(seg, cnt, lane, out, row_mask);
             continue;
         }
-        if (cnt <= 256) {
-            sort_cell<8>(seg, cnt, lane, out, row_mask);
-            continue;
+        sort_cell<8>(seg, cnt, lane, out, row_mask);
+    }
+    __syncthreads();
+    // the wide cells: their ranks do not depend on the order in which the warps
+    // listed them
+    const int nw = n_wide;
+    for (int k = 0; k < nw; ++k) {
+        const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
+        const uint32_t kmask = !SUB || cnt > kBigCell ? row_mask : 0xffffffffu;
+        int32_t *out = perm + st;
+        const uint32_t *sk = keys + (st - S0);
+        if (!staged) {
+            // a cell at a time through the stage (cnt <= kBlockCell <= kOrdCap)
+            __syncthreads();
+            for (uint32_t e = t; e < cnt; e += kBlock) keys[e] = order_key<SUB>(perm_tmp, order_tmp, st + e);
+            __syncthreads();
+            sk = keys;
         }
-        for (uint32_t e0 = 0; e0 < cnt; e0 += 4 * 32) rank_lanes<4>(seg, cnt, e0, lane, out, row_mask);
+        for (uint32_t e = t; e < cnt; e += kBlock) {
+            const uint32_t v = sk[e] & kmask;
+            uint32_t r = 0;
+#pragma unroll 8
+            for (uint32_t u = 0; u < cnt; ++u) r += (sk[u] & kmask) < v ? 1u : 0u;
+            out[r] = (int32_t)(v & row_mask);
+        }
     }
 }
 
@@ -743,41 +831,6 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
         if (src != B)
             for (int t = tid; t < m; t += kOrderThreads) B[t] = src[t];
         __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(kBlock) k_items(int64_t ncell, int64_t n, const uint32_t *__restrict__ count,
-                                                   const unsigned long long *__restrict__ packed,
-                                                   int32_t *__restrict__ cell_start, int4 *__restrict__ items,
-                                                   int32_t *__restrict__ n_items, int make_items,
-                                                   const BoxDev *__restrict__ boxes, int nbox, ItemRule cap) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c == 0) {
-        cell_start[ncell] = (int32_t)n;
-        if (make_items) {
-            const unsigned long long last = packed[ncell - 1];
-            const ItemRule r = boxes ? rule_of_box(cap, boxes[nbox - 1]) : cap;
-            *n_items = (int32_t)((last >> 32) + items_of(count[ncell - 1], r));
-        }
-    }
-    if (c >= ncell) return;
-    unsigned long long p = packed[c];
-    uint32_t s = (uint32_t)(p & 0xffffffffull);
-    cell_start[c] = (int32_t)s;
-    if (!make_items) return;
-    uint32_t cnt = count[c];
-    uint32_t it = (uint32_t)(p >> 32);
-    if (cnt == 0) return;
-    int box = 0;
-    if (boxes) {
-        box = box_of_cell(boxes, nbox, c);
-        cap = rule_of_box(cap, boxes[box]);
-    }
-    const uint32_t m = items_of(cnt, cap);
-    for (uint32_t q = 0; q < m; ++q) {
-        uint32_t a, e;
-        item_range(cnt, m, q, &a, &e);
-        items[it + q] = make_int4((int)c, (int)(s + a), (int)(e - a), box);
     }
 }
 
@@ -1132,10 +1185,10 @@ __device__ __forceinline__ void emit_run(int64_t c, int32_t lo, int32_t hi, uint
         if (lane == 0) atomicOr(flags, kFlagItems);
         return;
     }
+    const CellItems ci(cnt, m);
     for (uint32_t k = lane; k < m; k += 32) {
-        uint32_t a, e;
-        item_range(cnt, m, k, &a, &e);
-        items[it + k] = make_int4((int)c, (int)(lo + a), (int)(e - a), 0);
+        const uint32_t a = ci.first(k);
+        items[it + k] = make_int4((int)c, (int)(lo + a), (int)(ci.first(k + 1) - a), 0);
     }
 }
 
@@ -1253,10 +1306,15 @@ cudaError_t items_heavy_first(const BinBuffers &b, int64_t max_items, cudaStream
     return cudaGetLastError();
 }
 
+// counters next to the cell counts that one memset clears with them: mass_flag, big_count
+constexpr int kZeroTail = 2;
+
 void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_order) {
     b->key = c.take<int32_t>(n);
     b->rank = c.take<int32_t>(n);
-    b->count = c.take<uint32_t>(ncell);
+    b->count = c.take<uint32_t>(ncell + kZeroTail);   // then the flags that start at zero with the counts
+    b->mass_flag = b->count ? reinterpret_cast<int *>(b->count + ncell) : nullptr;
+    b->big_count = b->count ? reinterpret_cast<int *>(b->count + ncell) + 1 : nullptr;
     b->packed = c.take<unsigned long long>(ncell);
     b->scan_tmp = c.take<unsigned long long>(scan_tmp_elems(ncell));
     b->cell_start = c.take<int32_t>(ncell + 1);
@@ -1267,9 +1325,7 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
     b->order = c.take<int32_t>(max_items(n, ncell, sub_order));
     b->item_cls = c.take<uint32_t>(2 * kItemClasses);
     b->n_items = c.take<int32_t>(1);
-    b->mass_flag = c.take<int>(1);
     b->big_list = c.take<int32_t>(n / (kBigCell + 1) + 1);
-    b->big_count = c.take<int>(1);
     b->sub = sub_order ? c.take<uint8_t>(n) : nullptr;
     b->order_tmp = sub_order ? c.take<unsigned long long>(n) : nullptr;
 }
@@ -1286,39 +1342,35 @@ ItemRule item_rule(int item_cap, int split_max) {
 cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_items, const BoxDev *boxes, int nbox,
                      cudaStream_t s, ItemRule cap = {kItemMax / kCluster, 0xffffffffu}, const uint8_t *sub = nullptr,
                      uint32_t row_below = 0, bool stretches = false) {
-    cudaError_t e;
-    k_pack<<<blocks_for(ncell), kBlock, 0, s>>>(ncell, b.count, b.packed, cap, boxes, nbox);
-    note_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = scan_exclusive(b.packed, ncell, b.scan_tmp, s)) != cudaSuccess) return e;
+    cudaError_t e = scan_cells(ncell, n, CellPack{b.count, cap, boxes, nbox}, b, make_items, s);
+    if (e != cudaSuccess) return e;
     if (n > 0) {
         k_place<<<blocks_for(n), kBlock, 0, s>>>(n, b.key, b.rank, b.packed, b.perm_tmp, sub, b.order_tmp);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(b.big_count, 0, sizeof(int), s)) != cudaSuccess) return e;
+        // cells per block of the ordering: 64, fewer where that leaves SMs without a block
+        const int oc = (int)std::min<int64_t>(kOrdCells, std::max<int64_t>(kBlock / 32, ncell / 512));
         if (sub && n > kOrdSubMaxRows)
             k_order_sub<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                   b.big_list, b.big_count, b.order_tmp, row_below);
         else if (sub)
-            k_order_rows<true><<<blocks_for(ncell, kOrdCells), kBlock, 0, s>>>(
-                ncell, b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count, b.order_tmp, row_below,
-                stretches ? 1 : 0);
+            k_order_rows<true><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
+                                                                       b.big_list, b.big_count, b.order_tmp,
+                                                                       row_below, stretches ? 1 : 0, oc);
         else
-            k_order_rows<false><<<blocks_for(ncell, kOrdCells), kBlock, 0, s>>>(
-                ncell, b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count, nullptr, 0u,
-                stretches ? 1 : 0);
+            k_order_rows<false><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
+                                                                        b.big_list, b.big_count, nullptr, 0u,
+                                                                        stretches ? 1 : 0, oc);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (n > (int64_t)kBigCell) {
+        // k_order_sub lists cells above kBigCell, k_order_rows those above kBlockCell
+        if (n > (int64_t)(sub && n > kOrdSubMaxRows ? kBigCell : kBlockCell)) {
             k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count);
             note_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
-    k_items<<<blocks_for(ncell), kBlock, 0, s>>>(ncell, n, b.count, b.packed, b.cell_start, b.items, b.n_items,
-                                                 make_items ? 1 : 0, boxes, nbox, cap);
-    note_launch();
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 }  // namespace
 
@@ -1328,9 +1380,8 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
     if (item_cap != 0 && (item_cap < kCluster || item_cap > kItemCapMax)) return cudaErrorInvalidValue;
     if (split_max < 1 || ((item_cap || sub_level) && !b.sub)) return cudaErrorInvalidValue;
     uint8_t *sub = (item_cap || sub_level) ? b.sub : nullptr;
-    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * g.ncell, s);
+    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * (g.ncell + kZeroTail), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.mass_flag, 0, sizeof(int), s)) != cudaSuccess) return e;
     if (n > 0) {
         k_key<<<blocks_for(n), kBlock, 0, s>>>(n, src, vel, drift, dst, g.Lf, g.inv_w, g.Ld, g.nc, b.key,
                                                b.rank, b.count, d_flags, b.mass_flag, sub, sub_level);
@@ -1395,9 +1446,8 @@ cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int6
     if (item_cap > 0 && (item_cap < kCluster || item_cap > kItemCapMax)) return cudaErrorInvalidValue;
     if (split_max < 1 || (item_cap && !b.sub)) return cudaErrorInvalidValue;
     uint8_t *sub = item_cap ? b.sub : nullptr;
-    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * ncell_total, s);
+    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * (ncell_total + kZeroTail), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.mass_flag, 0, sizeof(int), s)) != cudaSuccess) return e;
     if (n_total > 0) {
         k_bkey<<<blocks_for(n_total), kBlock, 0, s>>>(n_total, nbox, boxes, pos_pool, vel_pool, dst, id, b.key,
                                                       b.rank, b.count, d_flags, b.mass_flag, sub);
@@ -1411,9 +1461,8 @@ cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int6
 
 cudaError_t bin_build_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
                          float4 *dst, const BinBuffers &b, int *d_flags, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * g.ncell, s);
+    cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * (g.ncell + kZeroTail), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(b.mass_flag, 0, sizeof(int), s)) != cudaSuccess) return e;
     if (n > 0) {
         k_key_ci<<<blocks_for(n), kBlock, 0, s>>>(n, cell, off, vel, drift, g.nc, g.Ld, ci_step(g), 1.0 / ci_step(g),
                                                   dst, b.key, b.rank, b.count, d_flags, b.mass_flag, b.sub);

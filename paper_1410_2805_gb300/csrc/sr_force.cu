@@ -43,7 +43,7 @@
 // Periodic images without rounding error: an item whose cell lies within R of
 // a high face (per axis) runs in the frame moved by -L: its own particles and
 // the neighbours of unwrapped rows get -L (they lie in [L/2, L) for nc >= 4R:
-// exact; for smaller nc only particles half a cutoff or more apart are
+// exact; for smaller nc only those a quarter of a cutoff or more apart are
 // rounded), those of rows that wrap high stay.  Elsewhere the neighbours of
 // rows that wrap low get -L (exact, in [2L/3, L)).  So r_ij = x_j' - x_i'
 // carries only the rounding of one subtraction.

@@ -52,3 +52,33 @@ def test_cell_counts_around_cluster_and_item_sizes(split_params, nc, masses, cap
     rms = np.sqrt((ref ** 2).sum(1).mean())
     assert np.abs(a[:, :3] - ref).max() / rms <= FORCE_TOL
     assert abs(got - within) <= max(2, within // 200000) and got <= cand
+
+
+@pytest.mark.parametrize("nc", [3, 40])
+def test_wide_cells_are_ordered(split_params, nc):
+    # cells at the bounds of the ordering's paths for cells above 256 particles, alone in their block of cells
+    # and crowded together (more keys than a block stages), in a mesh of few and of many cells
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1410_2805_gb300 as hacc
+    rc = np.float32(split_params["r_cut"])
+    L = float(np.float32(nc * 3.2))
+    rng = np.random.default_rng(nc)
+    rows = []
+    for c, n in {0: 256, 1: 257, 2: 512, 3: 513, 4: 2047, 5: 2048, 6: 2049, 9: 300, nc ** 3 - 1: 900}.items():
+        cell = np.array([c % nc, (c // nc) % nc, c // nc ** 2])
+        rows.append((cell + rng.uniform(0.001, 0.999, (n, 3))) * (L / nc))
+    x = np.concatenate(rows)
+    pos = np.ones((len(x), 4), np.float32)
+    pos[:, :3] = x
+    pos = pos[rng.permutation(len(pos))]
+    ctx = hacc.Context()
+    try:
+        p = torch.from_numpy(pos.copy()).cuda()
+        cell, start, perm = (t.cpu().numpy() for t in ctx.bin(hacc.Box(L=L, nc=nc), rc, p))
+    finally:
+        ctx.close()
+    _, cell_o, ok = oracle.wrap_cell(pos, L, nc)
+    _, start_o, perm_o = oracle.bin_cells(cell_o, nc)
+    assert ok and np.array_equal(cell, cell_o) and np.array_equal(start, start_o) and np.array_equal(perm, perm_o)
