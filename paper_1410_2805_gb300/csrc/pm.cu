@@ -7,7 +7,7 @@
 //   k_kspace    phi(k) = 4 pi G G6(k) S(k) rho(k) / ng^3 (Eq. (greenf),
 //               Eq. (filter)) and a_c(k) = -i D_c(k) phi(k), the fourth-order
 //               Super-Lanczos derivative of Eq. (sldiff), for c = x, y, z
-//   cuFFT C2R   x3, one per component
+//   cuFFT C2R   the three components, one batched plan
 //   k_interp    CIC interpolation of (a_x, a_y, a_z) at the particles, then
 //               either a store or a kick v += kick * a
 //
@@ -35,12 +35,14 @@ struct PmState {
     int ng = 0;
     cufftHandle r2c = 0, c2r = 0;
     bool have_plans = false;
+    unsigned long long *mass = nullptr;  // ng^3 fixed-point mass per grid point, then rho: together
+                                         // the three force components in real space, 3 x ng^3 floats
     float *rho = nullptr;        // ng^3
-    unsigned long long *mass = nullptr;  // ng^3 fixed-point mass per grid point
     cufftComplex *rk = nullptr;  // ng*ng*(ng/2+1)
     cufftComplex *ak = nullptr;  // 3 x ng*ng*(ng/2+1)
     float4 *field = nullptr;     // ng^3 (a_x, a_y, a_z, 0): one 16-byte load per CIC corner
     float *tab = nullptr;        // per-axis tables: t[ng], sl[ng], K2[ng]
+    double tab_L = 0.0;          // box side that the tables hold
     size_t bytes = 0;
 };
 
@@ -84,11 +86,25 @@ __global__ void __launch_bounds__(kBlock) k_deposit(int64_t n, const float4 *__r
             }
 }
 
+// rho = mass * scale from the fixed-point mass, scale = sh + sl.  The product
+// is formed from the mass's leading 24 bits and the rest, both exact in FP32, so
+// that it is rounded once and to within 2^-20 of an ulp as an FP64 product would
+// be.  FP64 and the 64-bit conversions run at a fraction of the FP32 rate here:
+// they took three times as long as the 12 bytes per grid point (128^3: 12.4 ->
+// 7 us).
 __global__ void __launch_bounds__(kBlock) k_fix_to_density(int64_t ng3, const unsigned long long *__restrict__ acc,
-                                                            double scale, float *__restrict__ rho) {
+                                                            float sh, float sl, float *__restrict__ rho) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng3) return;
-    rho[g] = (float)((double)(long long)acc[g] * scale);
+    const long long a = (long long)acc[g];
+    const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int cut = max(40 - __clzll((long long)u), 0);   // u >> cut has at most 24 bits
+    const int cut2 = max(cut - 24, 0);
+    const uint32_t top = (uint32_t)(u >> cut), rest = (uint32_t)((u - ((unsigned long long)top << cut)) >> cut2);
+    const float sign = a < 0 ? -1.0f : 1.0f;
+    const float hi = sign * (float)top * __int_as_float((127 + cut) << 23);
+    const float lo = sign * (float)rest * __int_as_float((127 + cut2) << 23);
+    rho[g] = __fmaf_rn(hi, sh, __fmaf_rn(lo, sh, hi * sl));
 }
 
 // Per-axis tables in FP64 (rounded to FP32 once): mode number k of index q is
@@ -198,7 +214,6 @@ void free_state(PmState *st) {
         cufftDestroy(st->r2c);
         cufftDestroy(st->c2r);
     }
-    cudaFree(st->rho);
     cudaFree(st->mass);
     cudaFree(st->rk);
     cudaFree(st->ak);
@@ -220,7 +235,7 @@ hacc_status get_state(hacc_ctx *ctx, int ng, double L, cudaStream_t s, PmState *
         size_t bytes = ng3 * 4 + ng3 * 8 + nm * 8 * 4 + ng3 * 16 + 3 * ng * 4;
         if (ctx->budget && ctx->scratch.cap + bytes > ctx->budget)
             return set_error(ctx, HACC_ENOMEM, "PM grid exceeds the context budget");
-        if (cudaMalloc(&st->rho, ng3 * 4) != cudaSuccess || cudaMalloc(&st->mass, ng3 * 8) != cudaSuccess ||
+        if (cudaMalloc(&st->mass, ng3 * 12) != cudaSuccess ||
             cudaMalloc(&st->rk, nm * 8) != cudaSuccess ||
             cudaMalloc(&st->ak, 3 * nm * 8) != cudaSuccess || cudaMalloc(&st->field, ng3 * 16) != cudaSuccess ||
             cudaMalloc(&st->tab, 3 * ng * 4) != cudaSuccess) {
@@ -228,11 +243,14 @@ hacc_status get_state(hacc_ctx *ctx, int ng, double L, cudaStream_t s, PmState *
             free_state(st);
             return set_error(ctx, HACC_ENOMEM, "cudaMalloc of the PM grid failed");
         }
+        st->rho = reinterpret_cast<float *>(st->mass + ng3);
         if (cufftPlan3d(&st->r2c, ng, ng, ng, CUFFT_R2C) != CUFFT_SUCCESS) {
             free_state(st);
             return set_error(ctx, HACC_ECUDA, "cufftPlan3d R2C failed");
         }
-        if (cufftPlan3d(&st->c2r, ng, ng, ng, CUFFT_C2R) != CUFFT_SUCCESS) {
+        // the three components in one plan: a third of the launches
+        int dims[3] = {ng, ng, ng};
+        if (cufftPlanMany(&st->c2r, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3) != CUFFT_SUCCESS) {
             cufftDestroy(st->r2c);
             free_state(st);
             return set_error(ctx, HACC_ECUDA, "cufftPlan3d C2R failed");
@@ -311,25 +329,32 @@ hacc_status pm_accel(hacc_ctx *ctx, const hacc_box *box, const hacc_pm *pm, doub
             if ((e = cudaEventRecord(io->ev[c], io->copy)) != cudaSuccess) return check_cuda(ctx, e, "cudaEventRecord");
         }
     }
-    k_fix_to_density<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, st->mass, 1.0 / (kFix * D * D * D),
-                                                                   st->rho);
+    const double scale = 1.0 / (kFix * D * D * D);
+    k_fix_to_density<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, st->mass, (float)scale,
+                                                                   (float)(scale - (double)(float)scale), st->rho);
     note_launch();
-    k_tables<<<(ng + 127) / 128, 128, 0, s>>>(ng, L, st->tab);
-    note_launch();
+    // the tables depend on the box side alone: kept until it changes (8 us of FP64
+    // a call), but not on the word of a launch that is only being captured
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return check_cuda(ctx, e, "cudaStreamIsCapturing");
+    if (st->tab_L != L || cap != cudaStreamCaptureStatusNone) {
+        k_tables<<<(ng + 127) / 128, 128, 0, s>>>(ng, L, st->tab);
+        note_launch();
+        st->tab_L = cap == cudaStreamCaptureStatusNone ? L : 0.0;
+    }
     if (cufftSetStream(st->r2c, s) != CUFFT_SUCCESS || cufftSetStream(st->c2r, s) != CUFFT_SUCCESS)
         return set_error(ctx, HACC_ECUDA, "cufftSetStream failed");
     if (cufftExecR2C(st->r2c, st->rho, st->rk) != CUFFT_SUCCESS) return set_error(ctx, HACC_ECUDA, "cufftExecR2C failed");
     const float pref = (float)(4.0 * 3.14159265358979323846 * G / (double)ng3);
     k_kspace<<<blocks_for(nm), kBlock, 0, s>>>(ng, (float)D, pm->sigma, pm->ns, pref, st->tab, st->rk, st->ak);
     note_launch();
-    // the components back to real space into arrays free at this point (the
-    // density, and the fixed-point mass grid as two real arrays), then
-    // interleaved into the field grid in one pass
-    float *comp[3] = {st->rho, reinterpret_cast<float *>(st->mass), reinterpret_cast<float *>(st->mass) + ng3};
-    for (int c = 0; c < 3; ++c)
-        if (cufftExecC2R(st->c2r, st->ak + c * nm, comp[c]) != CUFFT_SUCCESS)
-            return set_error(ctx, HACC_ECUDA, "cufftExecC2R failed");
-    k_pack_components<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, comp[0], comp[1], comp[2], st->field);
+    // the components back to real space into the arrays free at this point (the
+    // fixed-point mass grid and the density behind it), then interleaved into the
+    // field grid in one pass
+    float *comp = reinterpret_cast<float *>(st->mass);
+    if (cufftExecC2R(st->c2r, st->ak, comp) != CUFFT_SUCCESS) return set_error(ctx, HACC_ECUDA, "cufftExecC2R failed");
+    k_pack_components<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, comp, comp + ng3, comp + 2 * ng3,
+                                                                    st->field);
     note_launch();
     if (before_kick && (e = cudaStreamWaitEvent(s, before_kick, 0)) != cudaSuccess)
         return check_cuda(ctx, e, "cudaStreamWaitEvent");
