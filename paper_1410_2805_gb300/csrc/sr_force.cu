@@ -16,29 +16,32 @@
 //           row wraps), 64 at a time; those within reach of the item's bounds
 //           go to a per-warp shared tile (ballot + prefix count).
 //   select  Per cluster, the tile's entries within reach of the cluster's own
-//           bounds are compacted into a list (a lane per entry).
+//           bounds are compacted into a list (two entries a lane).
 //   pairs   Four lanes hold the cluster's 8 particles, two each, and eight
 //           lane groups share the list, two entries a step: four pairs per
 //           lane and step, as two packed FP32 chains (fma.rn.f32x2), the two
 //           entries in the two halves.
-// What bounds it: the FP32 pipe and the issue slots together.  A pair of the
-// pair loop alone takes 21-22 cycles a warp and scheduler, with any number of
-// warps: 16 FMA-pipe cycles (an f32x2 operation holds the pipe two cycles, three
-// when its three operands are different registers), the rsqrt, and the select.
-// Scalar arithmetic takes 24-25.  Of a launch on 128^3 Zel'dovich particles
-// (0.91 ms), the pairs take 0.50 ms, selecting and staging 0.34 ms, the rest
-// 0.07 ms.  So every pair not evaluated counts:
+// What bounds it: issue slots and the FP32 pipe together.  On 128^3 Zel'dovich
+// particles (0.84 ms) a scheduler issues in 70% of its cycles and the FP32 pipe
+// is held in 54% (an f32x2 operation takes two of its cycles, three when its
+// operands are three different registers); scalar arithmetic for the
+// polynomial or the sums, which needs fewer pipe cycles and more slots, is
+// 3-7% slower.  The pairs are half of the instructions, the selecting and
+// staging most of the rest.  So every pair not evaluated counts:
 // Why clusters of 8: per particle of a Zel'dovich box, 970 candidates lie in
 // the 27 cells, 655 within reach of a cell's bounds, 390 of an 8-cluster's and
-// 285 of a 4-cluster's, 154 inside the cutoff.  A select test costs 40 warp
-// instructions per 32 entries and cluster, so 4-clusters would pay in tests
-// what they save in pairs.  Items of 64 share one staging among 8 clusters
-// (256^3 box: 6.9 ms a launch against 7.3 with items of 32, 8.6 with 16);
-// smaller calls take smaller items to spread over the chip (auto_item_cap).
+// 285 of a 4-cluster's, 154 inside the cutoff (a bounding sphere instead of the
+// bounds keeps 18% more).  4-clusters would pay in tests what they save in
+// pairs; a last cluster of up to 4 on half the lanes costs more in the loop's
+// variable strides than the 5% of pairs that it saves.  Items of 64 share one
+// staging among 8 clusters (256^3 box: 6.9 ms a launch against 7.3 with items of
+// 32, 8.6 with 16); smaller calls take smaller items to spread over the chip
+// (auto_item_cap).
 // Against one warp per cell-wide item whose lanes evaluate all that is within
 // reach of the cell (scalar, 5 particles a lane): 256^3 launch 9.3 -> 6.9 ms,
-// 128^3 1.19 -> 0.91 ms, 32^3 122 -> 57 us; 256^3 full step 53.3 -> 40.6
-// ms, 24 boxes x 4 sub-cycles 26.7 -> 19.1 ms, 32^3 force call 194 -> 141 us.
+// 128^3 1.19 -> 0.91 ms, 32^3 122 -> 57 us; with the constants as parameters,
+// the packed selection, the longer tile and the unrolled last steps 256^3 6.5 ms,
+// 128^3 0.84 ms.
 //
 // Periodic images without rounding error: an item whose cell lies within R of
 // a high face (per axis) runs in the frame moved by -L: its own particles and
@@ -50,6 +53,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstring>
+
 #include "hacc_internal.cuh"
 
 namespace hacc {
@@ -57,6 +62,20 @@ namespace {
 
 constexpr int kWarps = 4;
 constexpr int kThreads = kWarps * 32;
+
+// Two FP32 values in one 64-bit register pair; each operation rounds its
+// halves as the scalar one does.
+typedef unsigned long long f32x2;
+
+// The pair-force constants, each in both halves: eps and P5's negated
+// coefficients.  Doubled on the host, they reach the packed operations as
+// operands from the parameter bank.  In registers of their own they made each
+// step of the polynomial one of three different registers, which holds the FMA
+// pipe three cycles instead of two, and took fourteen registers (128^3
+// Zel'dovich launch 900 -> 879 us, 256^3 6.91 -> 6.76 ms).
+struct PairConsts {
+    f32x2 eps, c0, c1, c2, c3, c4, c5;
+};
 
 struct KParams {
     const float4 *__restrict__ pos;
@@ -70,7 +89,6 @@ struct KParams {
     int cull;         // 1: select per cluster; 0: by the item's bounds alone
     float L;
     float T, eps, G;
-    float q0, q1, q2, q3, q4, q5;
     float u0, u1, u2, u3, u4, u5, u6, phi0;
     int mode;
     float4 *out;
@@ -90,6 +108,7 @@ struct KParams {
     float4 *pos_pool;
     float4 *vel_pool;
     int *flags;
+    PairConsts pair;
 };
 
 __device__ __forceinline__ float rsqrt_approx(float x) {
@@ -98,9 +117,6 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     return y;
 }
 
-// Two FP32 values in one 64-bit register pair; each operation rounds its
-// halves as the scalar one does.
-typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
     f32x2 r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -113,10 +129,6 @@ __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, 
 // like any other result of a shuffle, where a constant would be loaded and
 // doubled again in every round of the pair loop.
 __device__ __forceinline__ float keep(float v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
-__device__ __forceinline__ f32x2 keep2(float v) {
-    v = keep(v);
-    return pack2(v, v);
-}
 __device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
@@ -136,12 +148,27 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     return r;
 }
 
-constexpr int kTile = 384;                // staged entries of a warp at most
 constexpr int kRound = 64;                // candidates staged per round
 constexpr int kRing = 128;                // list entries held: two chunks
 constexpr int kChunk = 64;                // list entries per call of the pair loop
 constexpr int kMaxClusters = kItemMax / kCluster;
 constexpr int kMaxRuns = 50;              // 2 (2R+1)^2 for R = 2
+
+// The staged entries of a warp (the tile) and the list selected for a cluster,
+// as arrays of x, y, z and, with M (masses differ), m.  The tile takes what five
+// blocks of an SM leave: each flush of it ends every cluster's list with a
+// part-filled step and a sum over the warp (256^3 launch 6.76 ms with 384
+// entries, 6.57 with 512; six blocks with 384: 6.65).
+template <bool M>
+struct WarpBuf {
+    static constexpr int kArrays = M ? 4 : 3;
+    static constexpr int kTile = M ? 384 : 576;   // staged entries at most, whole rounds
+    float tile[kArrays][kTile];
+    float list[kArrays][kRing];
+};
+constexpr int kBufBytes = sizeof(WarpBuf<false>);
+static_assert(sizeof(WarpBuf<true>) <= kBufBytes && WarpBuf<false>::kTile % kRound == 0 &&
+                  WarpBuf<true>::kTile % kRound == 0, "one buffer for both forms");
 
 // A warp's shared memory.  Runs: (first, end, bits, b1) of the sorted
 // particles of each x-run, with (b2, d0) for the cell/offset form; bits 1/2/4:
@@ -150,15 +177,18 @@ constexpr int kMaxRuns = 50;              // 2 (2R+1)^2 for R = 2
 // high), and the x cell step of entry j is d0 + (j >= b1) + (j >= b2).
 template <bool CI, bool POT>
 struct WarpMem {
-    float4 tile[kTile];
-    float x[kRing], y[kRing], z[kRing], m[kRing];   // the list
+    char buf[kBufBytes];                  // a WarpBuf
     float4 own[kItemMax];                 // the item's particles in its frame
     float sum[3][kItemMax];               // and their sums
     float4 lo[kMaxClusters + 1], hi[kMaxClusters + 1];   // bounds of its clusters, and its own (last)
     int4 runs[kMaxRuns];
     int2 steps[CI ? kMaxRuns : 1];
-    int tile_id[POT ? kTile : 1];         // sorted index of each entry (the j != i test of the potential)
+    int tile_id[POT ? WarpBuf<true>::kTile : 1];         // sorted index of each entry (the j != i test of the potential)
     int id[POT ? kRing : 1];
+    template <bool M>
+    __device__ __forceinline__ WarpBuf<M> &as() {
+        return *reinterpret_cast<WarpBuf<M> *>(buf);
+    }
 };
 
 // The item's neighbour cells as x-runs of consecutive sorted particles, one
@@ -265,9 +295,9 @@ __device__ __forceinline__ void write_result(const KParams &P, int i, float gx, 
 }
 
 // Squared distance of v from the box [lo, hi].  A j is dropped when it reaches
-// a limit that carries a margin far above the rounding of the coordinates: it
+// a limit that carries a margin far above the rounding of the distance: it
 // is outside the cutoff of every i of the box and would have added exactly
-// nothing.
+// nothing.  A NaN is dropped too.
 __device__ __forceinline__ float box_dist2(float4 v, float4 lo, float4 hi) {
     const float ex = v.x - fminf(fmaxf(v.x, lo.x), hi.x);
     const float ey = v.y - fminf(fmaxf(v.y, lo.y), hi.y);
@@ -275,25 +305,80 @@ __device__ __forceinline__ float box_dist2(float4 v, float4 lo, float4 hi) {
     return __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, ez * ez));
 }
 
+// A cluster's bounds in units of the reach 1/s, as centre c and negated half
+// widths nh (s times them): the distance from them along an axis is
+// s |v - c| + nh, cut to [0, 1] by the saturation of the FMA itself.  Axes past
+// the reach saturate at 1, so a j is within reach when the squares sum to less
+// than 1.  v - c and c - lo are differences of FP32 values, so the test is off
+// by a few ulp of the distance, whatever the side of the box.  Against clamping
+// v to [lo, hi], half the instructions: no minimum and maximum, which run at
+// half the rate, and the subtraction and the squares packed.
+struct Reach {
+    float cx, cy, cz, nhx, nhy, nhz, s;
+};
+
+__device__ __forceinline__ Reach reach_of(float4 lo, float4 hi, float s) {
+    Reach b;
+    b.s = s;
+    b.cx = 0.5f * lo.x + 0.5f * hi.x;
+    b.cy = 0.5f * lo.y + 0.5f * hi.y;
+    b.cz = 0.5f * lo.z + 0.5f * hi.z;
+    b.nhx = -s * fmaxf(hi.x - b.cx, b.cx - lo.x);
+    b.nhy = -s * fmaxf(hi.y - b.cy, b.cy - lo.y);
+    b.nhz = -s * fmaxf(hi.z - b.cz, b.cz - lo.z);
+    return b;
+}
+
+// The distances along an axis of two entries, in units of the reach.
+__device__ __forceinline__ f32x2 axis_reach(f32x2 v, float c, float nh, float s) {
+    float d0, d1;
+    unpack2(add2(v, pack2(-c, -c)), d0, d1);
+    return pack2(__saturatef(__fmaf_rn(fabsf(d0), s, nh)), __saturatef(__fmaf_rn(fabsf(d1), s, nh)));
+}
+
 // Compaction of the lanes with d2 < r2 in lane order, as predicated stores
-// (no branch): put4 stores v to entry `at` + prefix of the tile, put3 its
-// coordinates (and mass with M) to the list ring; both return the number of
-// lanes that stored.  Addresses are those of shared memory.
-__device__ __forceinline__ int put4(float d2, float r2, unsigned below, unsigned tile, int at, float4 v) {
+// (no branch) of the coordinates (and mass with M) to the arrays of the tile or
+// of the list, `at` + prefix count; returns the number of lanes that stored.
+// Addresses are those of shared memory.
+template <bool M>
+__device__ __forceinline__ int put_tile(float d2, float r2, unsigned below, unsigned tile, int at, float4 v) {
+    constexpr int kStep = 4 * WarpBuf<M>::kTile;   // bytes from one array to the next
     int n;
-    asm volatile(
-        "{\n.reg .pred p;\n.reg .b32 m, a;\n"
-        "setp.lt.f32 p, %1, %2;\n"
-        "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
-        "popc.b32 %0, m;\n"
-        "and.b32 m, m, %3;\n"
-        "popc.b32 a, m;\n"
-        "add.s32 a, a, %5;\n"
-        "mad.lo.u32 a, a, 16, %4;\n"
-        "@p st.shared.v4.f32 [a], {%6, %7, %8, %9};\n}"
-        : "=r"(n)
-        : "f"(d2), "f"(r2), "r"(below), "r"(tile), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-        : "memory");
+    if (M)
+        asm volatile(
+            "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+            "setp.lt.f32 p, %1, %2;\n"
+            "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+            "popc.b32 %0, m;\n"
+            "and.b32 m, m, %3;\n"
+            "popc.b32 a, m;\n"
+            "add.s32 a, a, %5;\n"
+            "mad.lo.u32 a, a, 4, %4;\n"
+            "@p st.shared.f32 [a], %6;\n"
+            "@p st.shared.f32 [a + %10], %7;\n"
+            "@p st.shared.f32 [a + %11], %8;\n"
+            "@p st.shared.f32 [a + %12], %9;\n}"
+            : "=r"(n)
+            : "f"(d2), "f"(r2), "r"(below), "r"(tile), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "n"(kStep),
+              "n"(2 * kStep), "n"(3 * kStep)
+            : "memory");
+    else
+        asm volatile(
+            "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+            "setp.lt.f32 p, %1, %2;\n"
+            "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+            "popc.b32 %0, m;\n"
+            "and.b32 m, m, %3;\n"
+            "popc.b32 a, m;\n"
+            "add.s32 a, a, %5;\n"
+            "mad.lo.u32 a, a, 4, %4;\n"
+            "@p st.shared.f32 [a], %6;\n"
+            "@p st.shared.f32 [a + %9], %7;\n"
+            "@p st.shared.f32 [a + %10], %8;\n}"
+            : "=r"(n)
+            : "f"(d2), "f"(r2), "r"(below), "r"(tile), "r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "n"(kStep),
+              "n"(2 * kStep)
+            : "memory");
     return n;
 }
 
@@ -345,11 +430,6 @@ __device__ __forceinline__ float4 shift4(float4 v, float tx, float ty, float tz)
     return make_float4(__fadd_rn(v.x, tx), __fadd_rn(v.y, ty), __fadd_rn(v.z, tz), v.w);
 }
 
-// The pair-force constants, doubled: eps and P5's negated coefficients.
-struct PairConsts {
-    f32x2 eps, c0, c1, c2, c3, c4, c5;
-};
-
 // This lane's two particles: their negated coordinates, doubled, and their
 // sums over the list entries the lane's group took (one sum per half).
 struct Pair {
@@ -399,8 +479,9 @@ __device__ __forceinline__ void pair_step(const PairConsts &C, float T, unsigned
 // The same for the pair potential: phi(s) = -t^(-1/2) - U(t) - phi0 inside
 // the cutoff, U in t = s + eps; A.ax[k] = sum_j m_j phi over j != i.
 template <bool CI, bool POT>
-__device__ __forceinline__ void potential_loop(const KParams &P, const WarpMem<CI, POT> &S, int base, int len, int grp,
+__device__ __forceinline__ void potential_loop(const KParams &P, WarpMem<CI, POT> &S, int base, int len, int grp,
                                                int i, Pair &A) {
+    const auto &list = S.template as<true>().list;
 #pragma unroll 1
     for (int e = base + 2 * grp; e < base + len; e += 16) {
 #pragma unroll
@@ -411,7 +492,7 @@ __device__ __forceinline__ void potential_loop(const KParams &P, const WarpMem<C
             unpack2(A.nz[k], pz, u);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const float dx = S.x[e + h] + px, dy = S.y[e + h] + py, dz = S.z[e + h] + pz;
+                const float dx = list[0][e + h] + px, dy = list[1][e + h] + py, dz = list[2][e + h] + pz;
                 const float t = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, P.eps)));
                 u = __fmaf_rn(P.u6, t, P.u5);
                 u = __fmaf_rn(u, t, P.u4);
@@ -420,7 +501,7 @@ __device__ __forceinline__ void potential_loop(const KParams &P, const WarpMem<C
                 u = __fmaf_rn(u, t, P.u1);
                 u = __fmaf_rn(u, t, P.u0);
                 const bool in = t < P.T && S.id[e + h] != i + k;
-                ph[h] = in ? (-rsqrt_approx(t) - u - P.phi0) * S.m[e + h] : 0.0f;
+                ph[h] = in ? (-rsqrt_approx(t) - u - P.phi0) * list[3][e + h] : 0.0f;
             }
             A.ax[k] = add2(A.ax[k], pack2(ph[0], ph[1]));
         }
@@ -432,18 +513,21 @@ __device__ __forceinline__ void potential_loop(const KParams &P, const WarpMem<C
 template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
 __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S, int fill, int i0, int ni, float tx,
                                            float ty, float tz, float r2, int lane, unsigned &cnt, unsigned &evals) {
-    const float4 far = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // outside everything, massless
-    // whole rounds of 64 entries
+    constexpr int kTile = WarpBuf<!UM>::kTile;
+    WarpBuf<!UM> &buf = S.template as<!UM>();
+    // whole rounds of 64 entries: outside everything, massless
     const int full = uniform((fill + kRound - 1) & ~(kRound - 1));
-    if (fill + lane < full) S.tile[fill + lane] = far;
-    if (fill + 32 + lane < full) S.tile[fill + 32 + lane] = far;
+#pragma unroll
+    for (int h = 0; h < kRound; h += 32)
+        if (fill + h + lane < full) {
+#pragma unroll
+            for (int a = 0; a < WarpBuf<!UM>::kArrays; ++a) buf.tile[a][fill + h + lane] = a < 3 ? 1e18f : 0.0f;
+        }
     __syncwarp();
     const unsigned below = (1u << lane) - 1u;
     const int grp = lane >> 2, slot = lane & 3;
-    const unsigned ring = smem_addr(S.x), mine = ring + 8 * grp;   // the list; this group's entry pairs
-    const PairConsts C{keep2(P.eps), keep2(-P.q0), keep2(-P.q1), keep2(-P.q2),
-                       keep2(-P.q3), keep2(-P.q4), keep2(-P.q5)};
-    const float T = keep(P.T);
+    const unsigned tile = smem_addr(buf.tile), ring = smem_addr(buf.list), mine = ring + 8 * grp;   // the list; this group's entry pairs
+    const float T = keep(P.T), s_reach = rsqrtf(r2);
 #pragma unroll 1
     for (int c0 = 0; c0 < ni; c0 += kCluster) {
         float4 lo = S.lo[c0 / kCluster], hi = S.hi[c0 / kCluster];
@@ -461,18 +545,29 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
             lo = shift4(lo, tx, ty, tz);
             hi = shift4(hi, tx, ty, tz);
         }
+        const Reach B = reach_of(lo, hi, s_reach);
         int at = 0, todo = 0;   // ring position of the next entry; entries waiting
 #pragma unroll 1
         for (int e0 = 0; e0 < full; e0 += kRound) {
-            const int e = e0 + lane;
-            const float4 v0 = S.tile[e], v1 = S.tile[e + 32];
-            const float d0 = box_dist2(v0, lo, hi), d1 = box_dist2(v1, lo, hi);
-            const int n0 = put3<!UM>(d0, r2, below, ring, at, v0);
-            const int n1 = put3<!UM>(d1, r2, below, ring, at + n0, v1);
+            // entries e and e + 1 of the tile
+            const int e = e0 + 2 * lane;
+            const unsigned te = tile + 4 * e;
+            const f32x2 X = lds2(te, 0), Y = lds2(te, 4 * kTile), Z = lds2(te, 8 * kTile);
+            float4 v0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), v1 = v0;
+            unpack2(X, v0.x, v1.x);
+            unpack2(Y, v0.y, v1.y);
+            unpack2(Z, v0.z, v1.z);
+            if (!UM) unpack2(lds2(te, 12 * kTile), v0.w, v1.w);
+            const f32x2 ex = axis_reach(X, B.cx, B.nhx, B.s), ey = axis_reach(Y, B.cy, B.nhy, B.s),
+                        ez = axis_reach(Z, B.cz, B.nhz, B.s);
+            float d0, d1;
+            unpack2(fma2(ex, ex, fma2(ey, ey, mul2(ez, ez))), d0, d1);
+            const int n0 = put3<!UM>(d0, 1.0f, below, ring, at, v0);
+            const int n1 = put3<!UM>(d1, 1.0f, below, ring, at + n0, v1);
             if (POT) {
-                const unsigned m0 = __ballot_sync(0xffffffffu, d0 < r2), m1 = __ballot_sync(0xffffffffu, d1 < r2);
-                if (d0 < r2) S.id[(at + __popc(m0 & below)) & (kRing - 1)] = S.tile_id[e];
-                if (d1 < r2) S.id[(at + n0 + __popc(m1 & below)) & (kRing - 1)] = S.tile_id[e + 32];
+                const unsigned m0 = __ballot_sync(0xffffffffu, d0 < 1.0f), m1 = __ballot_sync(0xffffffffu, d1 < 1.0f);
+                if (d0 < 1.0f) S.id[(at + __popc(m0 & below)) & (kRing - 1)] = S.tile_id[e];
+                if (d1 < 1.0f) S.id[(at + n0 + __popc(m1 & below)) & (kRing - 1)] = S.tile_id[e + 1];
             }
             at += n0 + n1;
             todo = uniform(todo + n0 + n1);
@@ -485,7 +580,7 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
                 } else {
 #pragma unroll F
                     for (int t = 0; t < kChunk / 16; ++t)
-                        pair_step<COUNT, EPS0, UM>(C, T, mine + 4 * base + 64 * t, A, cnt);
+                        pair_step<COUNT, EPS0, UM>(P.pair, T, mine + 4 * base + 64 * t, A, cnt);
                 }
                 todo -= kChunk;
                 __syncwarp();
@@ -495,17 +590,23 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
             const int base = (at - todo) & (kRing - 1), len = (todo + 15) & ~15;
             if (todo + lane < len) {
                 const int q = base + todo + lane;
-                S.x[q] = S.y[q] = S.z[q] = 1e18f;
-                S.m[q] = 0.0f;
+#pragma unroll
+                for (int a = 0; a < WarpBuf<!UM>::kArrays; ++a) buf.list[a][q] = a < 3 ? 1e18f : 0.0f;
                 if (POT) S.id[q] = -1;
             }
             __syncwarp();
             if (POT) {
                 potential_loop<CI, POT>(P, S, base, len, grp, i0 + c0 + 2 * slot, A);
             } else {
+                // 1 to 4 steps, without the loop's overhead
                 unsigned q = mine + 4 * base;
-#pragma unroll 1
-                for (int t = 0; t < len; t += 16, q += 64) pair_step<COUNT, EPS0, UM>(C, T, q, A, cnt);
+                if (len > 32) {
+                    pair_step<COUNT, EPS0, UM>(P.pair, T, q, A, cnt);
+                    pair_step<COUNT, EPS0, UM>(P.pair, T, q + 64, A, cnt);
+                    q += 128;
+                }
+                pair_step<COUNT, EPS0, UM>(P.pair, T, q, A, cnt);
+                if (!(len & 16)) pair_step<COUNT, EPS0, UM>(P.pair, T, q + 64, A, cnt);
             }
             __syncwarp();
         }
@@ -608,7 +709,8 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
                        !(cx >= R && cy >= R && cz >= R && cx + R < nc && cy + R < nc && cz + R < nc);
     float tx = 0.0f, ty = 0.0f, tz = 0.0f;
     unsigned cnt = 0, evals = 0;
-    const unsigned below = (1u << lane) - 1u, tile = smem_addr(S.tile);
+    constexpr int kTile = WarpBuf<!UM>::kTile;
+    const unsigned below = (1u << lane) - 1u, tile = smem_addr(S.buf);
     int fill = 0;
     // the stream of rounds: 64 particles of a run (past its end: its last one
     // again, never kept); the next round's loads are in flight while this one's
@@ -693,7 +795,7 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
                 const unsigned m = __ballot_sync(0xffffffffu, d2 < lim);
                 if (d2 < lim) S.tile_id[fill + __popc(m & below)] = j + 32 * h;
             }
-            fill = uniform(fill + put4(d2, lim, below, tile, fill, v[h]));
+            fill = uniform(fill + put_tile<!UM>(d2, lim, below, tile, fill, v[h]));
         }
         if (!calm) {
             if (fill > kTile - kRound) {
@@ -781,6 +883,12 @@ cudaError_t launch_one(const KParams &P, int num_sms, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+f32x2 doubled(float v) {
+    uint32_t u;
+    std::memcpy(&u, &v, sizeof u);
+    return ((f32x2)u << 32) | u;
+}
+
 // Variants 0..kForceVariants-1: (MINB, F) = (5, 4), (4, 4), (5, 2), (4, 2);
 // all give bitwise the same forces.
 template <bool COUNT, bool EPS0>
@@ -814,7 +922,8 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     P.T = fc.T;
     P.eps = fc.eps;
     P.G = fc.G;
-    P.q0 = fc.q[0]; P.q1 = fc.q[1]; P.q2 = fc.q[2]; P.q3 = fc.q[3]; P.q4 = fc.q[4]; P.q5 = fc.q[5];
+    P.pair = PairConsts{doubled(fc.eps),   doubled(-fc.q[0]), doubled(-fc.q[1]), doubled(-fc.q[2]),
+                        doubled(-fc.q[3]), doubled(-fc.q[4]), doubled(-fc.q[5])};
     P.u0 = fc.u[0]; P.u1 = fc.u[1]; P.u2 = fc.u[2]; P.u3 = fc.u[3]; P.u4 = fc.u[4]; P.u5 = fc.u[5];
     P.u6 = fc.u[6];
     P.phi0 = fc.phi0;
