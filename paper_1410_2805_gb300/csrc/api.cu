@@ -283,6 +283,8 @@ hacc_status run_sorted_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts
     fl.mass_flag = w->b.mass_flag;
     fl.variant = ctx->variant;
     fl.cull = item_cap_for(ctx, n) != 0;
+    if (ctx->item_cap < 0 && ctx->split_max == kDefaultSplitMax && shared_items(n) && mode != kModePotential)
+        fl.sharing = kByBlock;
     if (ctx->counting && mode != kModePotential && !within) {
         HACC_CUDA(candidate_count(g, w->b.cell_start, ctx->d_pairs, s), "candidate count");
         fl.within = ctx->d_pairs + 1;

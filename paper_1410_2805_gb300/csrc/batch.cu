@@ -169,6 +169,9 @@ hacc_status run_tick(hacc_ctx *ctx, const ForceConsts &fc, const Plan &pl, const
     fl.mass_flag = w.b.mass_flag;
     fl.variant = sh.variant;
     fl.cull = sh.cap != 0;
+    if (sh.cap < 0 && ctx->split_max == kDefaultSplitMax)
+        for (const BoxDev &d : pl.base)
+            if (shared_items(d.n)) fl.sharing = kByParts;
     if (sh.order && pl.n_total >= kHeavyFirstMinN) {
         HACC_CUDA_RETURN(items_heavy_first(w.b, max_items(pl.n_total, pl.ncell_total), s), "item order");
         fl.order = w.b.order;

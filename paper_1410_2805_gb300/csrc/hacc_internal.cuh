@@ -87,12 +87,20 @@ struct hacc_ctx {
 };
 
 namespace hacc {
+// Single-box calls of few particles let the four warps of a block share each
+// item, a quarter of its neighbours each: with an item per warp, the densest
+// cells' items set the launch's time while most warps have none (blob boxes, us
+// of the launch with an item per warp and shared: 4099 particles 33 and 18,
+// 16384 43 and 27, 32768 47 and 36, 65536 65 and 57, 131072 100 and 103).
+__host__ __device__ inline bool shared_items(int64_t n) { return n <= (1 << 16); }
 // Automatic item cap of a box of n particles: smaller items for smaller boxes,
-// so that their few items spread over the chip.  A box of a batch follows its
+// so that their few items spread over the chip.  A shared item costs a block
+// its staging, so it is larger where there are enough items (32768 particles:
+// 37 us with 32, 41 with 16; 9001: 27 and 21).  A box of a batch follows its
 // own size, so that its sums are the same alone, in any mix and in a call of
 // its own.
 __host__ __device__ inline int auto_item_cap(int64_t n) {
-    return n <= (1 << 13) ? 8 : (n <= (1 << 16) ? 16 : (n <= (1 << 20) ? 32 : kItemMax));
+    return n <= (1 << 13) ? 8 : (n <= (3 << 12) ? 16 : (n <= (1 << 20) ? 32 : kItemMax));
 }
 // Item cap of a force call over n particles (hacc_set_item_cap): the set
 // value, or the automatic one.
@@ -350,6 +358,11 @@ enum ForceMode : int {
     kModeKickLevels = 5  // kick by the table entry of the particle's kick count (multi-level)
 };
 
+// How an item is shared (shared_items()): one warp takes it whole; the warps of a
+// block take a part of its neighbours each; or one warp, of a batch, takes the
+// items of small boxes in the same parts one after the other.
+enum Sharing : int { kWhole = 0, kByBlock = 1, kByParts = 2 };
+
 struct ForceLaunch {
     const float4 *pos;          // sorted, wrapped
     const int4 *items;
@@ -385,6 +398,7 @@ struct ForceLaunch {
     float w = 0.0f;
     float delta = 0.0f;
     int variant = 0;            // pair-kernel variant (autotuned), 0..kForceVariants-1
+    Sharing sharing = kWhole;   // of work items (automatic item caps only)
     const int32_t *order = nullptr;   // non-null: the queue takes items[order[k]] (items_heavy_first)
 };
 

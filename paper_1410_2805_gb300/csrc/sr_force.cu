@@ -36,7 +36,7 @@
 // variable strides than the 5% of pairs that it saves.  Items of 64 share one
 // staging among 8 clusters (256^3 box: 6.9 ms a launch against 7.3 with items of
 // 32, 8.6 with 16); smaller calls take smaller items to spread over the chip
-// (auto_item_cap).
+// (auto_item_cap), the smallest share each item in a block (shared_items).
 // Against one warp per cell-wide item whose lanes evaluate all that is within
 // reach of the cell (scalar, 5 particles a lane): 256^3 launch 9.3 -> 6.9 ms,
 // 128^3 1.19 -> 0.91 ms, 32^3 122 -> 57 us; with the constants as parameters,
@@ -636,15 +636,16 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
     __syncwarp();
 }
 
-template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
 __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMem<CI, POT> &S, int lane,
-                                             float m_uniform) {
+                                             float m_uniform, int warp) {
     // geometry: the single box of the call, or this item's box of a batch
     int nc = P.nc;
     float L = P.L;
-    int cbase = 0;
+    int cbase = 0, parts = 1;
     if (P.boxes) {
         const BoxDev &bx = P.boxes[item.w];
+        if (SH == kByParts && shared_items(bx.n)) parts = kWarps;
         nc = uniform(bx.nc);
         L = bx.L;
         cbase = uniform(bx.cell_base);
@@ -712,17 +713,24 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
     constexpr int kTile = WarpBuf<!UM>::kTile;
     const unsigned below = (1u << lane) - 1u, tile = smem_addr(S.buf);
     int fill = 0;
+    // The rounds of a shared item go to its warps in turn, each run starting with
+    // another warp: most runs are one full round and a part.  The warp of a batch
+    // goes through the parts of a small box's item one after the other, so that
+    // its sums are those of the box in a call of its own.
+    int part = SH == kByBlock ? warp : 0;
+    if (SH == kByBlock) parts = kWarps;
     // the stream of rounds: 64 particles of a run (past its end: its last one
     // again, never kept); the next round's loads are in flight while this one's
     // are tested
     int q = -1, j0 = 0, end = 0, bits = 0, b1 = 0;
     float sx = 0.0f, sy = 0.0f, sz = 0.0f;   // shift of the run's particles
     auto next = [&]() -> bool {
-        j0 += kRound;
+        j0 += SH == kWhole ? kRound : kRound * parts;
         while (j0 >= end) {
             if (++q >= nrun) return false;
             const int4 run = S.runs[q];
             j0 = uniform(run.x);
+            if (SH != kWhole) j0 += kRound * ((part - q) & (parts - 1));
             end = uniform(run.y);
             bits = uniform(run.z);
             b1 = run.w;
@@ -739,82 +747,111 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
         n0 = P.pos[min(j0 + lane, end - 1)];
         n1 = P.pos[min(j0 + 32 + lane, end - 1)];
     };
-    bool more = next();
-    if (more) load();
 #pragma unroll 1
-    while (more) {
-        float4 v[2] = {n0, n1};
-        if (!CI) {
-            v[0] = shift4(v[0], sx, sy, sz);
-            v[1] = shift4(v[1], sx, sy, sz);
-        }
-        const int j = j0 + lane, left = end - j0, run_bits = bits, step1 = b1;
-        int2 st = make_int2(0, 0);
-        if (CI) st = S.steps[q];
-        // no flush after this round?  Then its successor's loads start now, else
-        // after the flush (held across it, they would cost it eight registers)
-        const bool calm = fill <= kTile - 2 * kRound;
-        more = next();
-        if (more && calm) load();
-        if (CI) {
-            sy = (float)((run_bits & 15) - 2) * P.w;
-            sz = (float)(((run_bits >> 4) & 15) - 2) * P.w;
-            if (moves) {
-                const int wb = run_bits >> 8;
-                const float ux = (wb & 1) ? P.delta : ((wb & 8) ? -P.delta : 0.0f);
-                const float uy = (wb & 2) ? P.delta : ((wb & 16) ? -P.delta : 0.0f);
-                const float uz = (wb & 4) ? P.delta : ((wb & 32) ? -P.delta : 0.0f);
-                if (ux != tx || uy != ty || uz != tz) {
-                    if (fill)
-                        flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
-                    fill = 0;
-                    tx = ux;
-                    ty = uy;
-                    tz = uz;
+    for (;;) {
+        bool more = next();
+        if (more) load();
+#pragma unroll 1
+        while (more) {
+            float4 v[2] = {n0, n1};
+            if (!CI) {
+                v[0] = shift4(v[0], sx, sy, sz);
+                v[1] = shift4(v[1], sx, sy, sz);
+            }
+            const int j = j0 + lane, left = end - j0, run_bits = bits, step1 = b1;
+            int2 st = make_int2(0, 0);
+            if (CI) st = S.steps[q];
+            // no flush after this round?  Then its successor's loads start now, else
+            // after the flush (held across it, they would cost it eight registers)
+            const bool calm = fill <= kTile - 2 * kRound;
+            more = next();
+            if (more && calm) load();
+            if (CI) {
+                sy = (float)((run_bits & 15) - 2) * P.w;
+                sz = (float)(((run_bits >> 4) & 15) - 2) * P.w;
+                if (moves) {
+                    const int wb = run_bits >> 8;
+                    const float ux = (wb & 1) ? P.delta : ((wb & 8) ? -P.delta : 0.0f);
+                    const float uy = (wb & 2) ? P.delta : ((wb & 16) ? -P.delta : 0.0f);
+                    const float uz = (wb & 4) ? P.delta : ((wb & 32) ? -P.delta : 0.0f);
+                    if (ux != tx || uy != ty || uz != tz) {
+                        if (fill)
+                            flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+                        fill = 0;
+                        tx = ux;
+                        ty = uy;
+                        tz = uz;
+                    }
                 }
             }
-        }
-        float4 lo = S.lo[kMaxClusters], hi = S.hi[kMaxClusters];
-        if (CI) {
-            lo = shift4(lo, tx, ty, tz);
-            hi = shift4(hi, tx, ty, tz);
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (h && left <= 32) break;
+            float4 lo = S.lo[kMaxClusters], hi = S.hi[kMaxClusters];
             if (CI) {
-                // whole cell steps of the FP32 width w move j into the frame of i's
-                // cell: exact for a j within reach of i's cell, so a close pair
-                // across a face gets its separation with one rounding at most
-                const int jj = j + 32 * h;
-                const float d = (float)(st.y + (jj >= step1) + (jj >= st.x));
-                v[h] = shift4(v[h], d * P.w, sy, sz);
+                lo = shift4(lo, tx, ty, tz);
+                hi = shift4(hi, tx, ty, tz);
             }
-            const float d2 = box_dist2(v[h], lo, hi), lim = lane + 32 * h < left ? r2 : 0.0f;
-            if (POT) {
-                const unsigned m = __ballot_sync(0xffffffffu, d2 < lim);
-                if (d2 < lim) S.tile_id[fill + __popc(m & below)] = j + 32 * h;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h && left <= 32) break;
+                if (CI) {
+                    // whole cell steps of the FP32 width w move j into the frame of i's
+                    // cell: exact for a j within reach of i's cell, so a close pair
+                    // across a face gets its separation with one rounding at most
+                    const int jj = j + 32 * h;
+                    const float d = (float)(st.y + (jj >= step1) + (jj >= st.x));
+                    v[h] = shift4(v[h], d * P.w, sy, sz);
+                }
+                const float d2 = box_dist2(v[h], lo, hi), lim = lane + 32 * h < left ? r2 : 0.0f;
+                if (POT) {
+                    const unsigned m = __ballot_sync(0xffffffffu, d2 < lim);
+                    if (d2 < lim) S.tile_id[fill + __popc(m & below)] = j + 32 * h;
+                }
+                fill = uniform(fill + put_tile<!UM>(d2, lim, below, tile, fill, v[h]));
             }
-            fill = uniform(fill + put_tile<!UM>(d2, lim, below, tile, fill, v[h]));
+            if (!calm) {
+                if (fill > kTile - kRound) {
+                    flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+                    fill = 0;
+                }
+                if (more) load();
+            }
         }
-        if (!calm) {
-            if (fill > kTile - kRound) {
-                flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
-                fill = 0;
+        if (fill) flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+        if (SH != kByParts || parts == 1) break;
+        if constexpr (SH == kByParts) {
+            // the parts' sums are added in order (items of a small box hold at most 32 particles)
+            for (int k = 0; k < (POT ? 1 : 3); ++k) {
+                const float a = S.sum[k][lane];
+                S.sum[k][32 + lane] = part ? S.sum[k][32 + lane] + a : a;
+                S.sum[k][lane] = 0.0f;
             }
-            if (more) load();
+            __syncwarp();
+            if (++part == parts) break;
+            fill = 0;
+            q = -1;
+            j0 = end = 0;
         }
     }
-    if (fill) flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
 
-    // epilogue: a particle per lane
+    // epilogue: a particle per lane, or per thread of the block that shares the item
+    if (SH == kByBlock) __syncthreads();
 #pragma unroll
-    for (int h = 0; h < kItemMax / 32; ++h) {
-        if (32 * h + lane >= ni) continue;
-        const int i = i0 + 32 * h + lane;
+    for (int h = 0; h < kItemMax; h += 32) {
+        const int e = h + lane;
+        if (e >= ni || (SH == kByBlock && h != 32 * warp)) continue;
+        float sum[3];
+#pragma unroll
+        for (int k = 0; k < (POT ? 1 : 3); ++k) {
+            if (SH == kByBlock) {
+                const WarpMem<CI, POT> *w = &S - warp;
+                sum[k] = ((w[0].sum[k][e] + w[1].sum[k][e]) + w[2].sum[k][e]) + w[3].sum[k][e];
+            } else {
+                sum[k] = S.sum[k][SH != kByParts || parts == 1 ? e : 32 + lane];
+            }
+        }
+        const int i = i0 + e;
         const float4 p = P.pos[i];
         if (POT) {
-            P.phi_out[i] = 0.5f * P.G * p.w * S.sum[0][32 * h + lane];
+            P.phi_out[i] = 0.5f * P.G * p.w * sum[0];
         } else {
             const float gm = UM ? P.G * m_uniform : P.G;
             float h_kick = P.h_kick, h_drift = P.h_drift;
@@ -822,8 +859,7 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
                 h_kick = P.boxes[item.w].h;
                 h_drift = P.boxes[item.w].post;
             }
-            write_result(P, i, gm * S.sum[0][32 * h + lane], gm * S.sum[1][32 * h + lane], gm * S.sum[2][32 * h + lane],
-                         p.x, p.y, p.z, p.w, h_kick, h_drift, L);
+            write_result(P, i, gm * sum[0], gm * sum[1], gm * sum[2], p.x, p.y, p.z, p.w, h_kick, h_drift, L);
         }
     }
     if (COUNT) {
@@ -831,46 +867,56 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
         unsigned long long c64 = cnt;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c64 += __shfl_down_sync(0xffffffffu, c64, o);
-        if (lane == 0) atomicAdd(P.within, P.eps < P.T ? c64 - (unsigned long long)ni : c64);
+        if (lane == 0) atomicAdd(P.within, P.eps < P.T && warp == 0 ? c64 - (unsigned long long)ni : c64);
         if (lane == 0 && P.evaluated) atomicAdd(P.evaluated, (unsigned long long)evals);
     }
     __syncwarp();
 }
 
-template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI>
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
 __device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S, int lane, float m_uniform) {
     const int n_items = uniform(*P.n_items);
+    const int warp = SH == kByBlock ? uniform(threadIdx.x >> 5) : 0;
+    __shared__ int claimed;
     while (true) {
         int it = 0;
-        if (lane == 0) it = atomicAdd(P.work_counter, 1);
-        it = __shfl_sync(0xffffffffu, it, 0);
+        if (SH == kByBlock) {
+            __syncthreads();   // the sums of the item before are read
+            if (threadIdx.x == 0) claimed = atomicAdd(P.work_counter, 1);
+            __syncthreads();
+            it = uniform(claimed);
+        } else {
+            if (lane == 0) it = atomicAdd(P.work_counter, 1);
+            it = __shfl_sync(0xffffffffu, it, 0);
+        }
         if (it >= n_items) break;
         int4 item = P.items[P.order ? P.order[it] : it];
         item.x = uniform(item.x);
         item.y = uniform(item.y);
         item.z = uniform(item.z);
         item.w = uniform(item.w);
-        process_item<COUNT, POT, EPS0, UM, F, CI>(P, item, S, lane, m_uniform);
+        process_item<COUNT, POT, EPS0, UM, F, CI, SH>(P, item, S, lane, m_uniform, warp);
     }
 }
 
 // MINB: blocks per SM the register allocation must allow; F: steps of the
-// pair loop unrolled.  The autotuner picks.
-template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI>
+// pair loop unrolled.  The autotuner picks.  SH: the warps of a block share each
+// item (calls of few items, see shared_items).
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH>
 __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
     extern __shared__ __align__(16) char smem[];
     WarpMem<CI, POT> *S = reinterpret_cast<WarpMem<CI, POT> *>(smem) + uniform(threadIdx.x >> 5);
     const int lane = __shfl_xor_sync(0xffffffffu, (threadIdx.x & 31) ^ 1, 1);   // as with uniform(): kept
     // equal masses (flag left 0 by the binning pass): apply the mass once per i
     if (!POT && P.mass_flag && uniform(*P.mass_flag) == 0 && uniform(*P.n_items) > 0)
-        work_loop<COUNT, POT, EPS0, !POT, F, CI>(P, *S, lane, P.pos[0].w);
+        work_loop<COUNT, POT, EPS0, !POT, F, CI, SH>(P, *S, lane, P.pos[0].w);
     else
-        work_loop<COUNT, POT, EPS0, false, F, CI>(P, *S, lane, 0.0f);
+        work_loop<COUNT, POT, EPS0, false, F, CI, SH>(P, *S, lane, 0.0f);
 }
 
-template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI>
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH = kWhole>
 cudaError_t launch_one(const KParams &P, int num_sms, cudaStream_t s) {
-    auto *k = k_sr_force<COUNT, POT, EPS0, MINB, F, CI>;
+    auto *k = k_sr_force<COUNT, POT, EPS0, MINB, F, CI, SH>;
     const size_t bytes = kWarps * sizeof(WarpMem<CI, POT>);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
@@ -899,6 +945,16 @@ cudaError_t launch_variant(const KParams &P, int variant, int num_sms, cudaStrea
         case 3: return launch_one<COUNT, false, EPS0, 4, 2, false>(P, num_sms, s);
         default: return launch_one<COUNT, false, EPS0, 5, 4, false>(P, num_sms, s);
     }
+}
+
+// Shared items: one variant each, bitwise the same forces.
+template <Sharing SH>
+cudaError_t launch_shared(const KParams &P, bool eps0, bool count, int num_sms, cudaStream_t s) {
+    if (count)
+        return eps0 ? launch_one<true, false, true, 4, 1, false, SH>(P, num_sms, s)
+                    : launch_one<true, false, false, 4, 1, false, SH>(P, num_sms, s);
+    return eps0 ? launch_one<false, false, true, 5, 4, false, SH>(P, num_sms, s)
+                : launch_one<false, false, false, 5, 4, false, SH>(P, num_sms, s);
 }
 
 }  // namespace
@@ -959,6 +1015,8 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     if (pot)
         return eps0 ? launch_one<false, true, true, 4, 1, false>(P, num_sms, s)
                     : launch_one<false, true, false, 4, 1, false>(P, num_sms, s);
+    if (fl.sharing == kByBlock) return launch_shared<kByBlock>(P, eps0, count, num_sms, s);
+    if (fl.sharing == kByParts) return launch_shared<kByParts>(P, eps0, count, num_sms, s);
     if (count)
         return eps0 ? launch_one<true, false, true, 4, 1, false>(P, num_sms, s)
                     : launch_one<true, false, false, 4, 1, false>(P, num_sms, s);
