@@ -217,15 +217,16 @@ __device__ __forceinline__ unsigned long long block_exclusive(unsigned long long
     return r;
 }
 
-// Sums of scan tiles: of the packed cells (CELLS) or of a level of block sums.
-template <bool CELLS>
+// Sums of scan tiles: of the packed cells (CELLS) or of a level of block sums;
+// ROWS values per thread.
+template <bool CELLS, int ROWS>
 __global__ void __launch_bounds__(kBlock) k_scan_reduce(int64_t len, CellPack cells,
                                                          const unsigned long long *__restrict__ in,
                                                          unsigned long long *__restrict__ sums) {
-    int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    int64_t base = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * ROWS;
     unsigned long long s = 0;
 #pragma unroll
-    for (int j = 0; j < kScanItems; ++j)
+    for (int j = 0; j < ROWS; ++j)
         if (base + j < len) s += CELLS ? cells(base + j) : in[base + j];
     unsigned long long total;
     block_exclusive(s, &total);
@@ -260,7 +261,7 @@ cudaError_t scan_exclusive(unsigned long long *data, int64_t len, unsigned long 
         return cudaGetLastError();
     }
     unsigned long long *sums = tmp;
-    k_scan_reduce<false><<<(unsigned)nb, kBlock, 0, s>>>(len, CellPack{}, data, sums);
+    k_scan_reduce<false, kScanItems><<<(unsigned)nb, kBlock, 0, s>>>(len, CellPack{}, data, sums);
     note_launch();
     cudaError_t e = scan_exclusive(sums, nb, tmp + nb, s);
     if (e != cudaSuccess) return e;
@@ -272,19 +273,34 @@ cudaError_t scan_exclusive(unsigned long long *data, int64_t len, unsigned long 
 // The last pass of the scan over the cells: the packing, the cell starts and
 // the force work items as the sums come out (a thread per cell; the cells of a
 // block are taken one row of threads at a time, so that dense cells next to
-// each other meet different threads).  Before, packing and items were kernels
-// of their own that each read the cells again, and divided twice per item (32^3
-// box: 1.7 + 2.4 + 6.0 us, now 7.2; 128^3: 1.7 + 7.5 + 3.5, now 12 with one
-// launch fewer).
+// each other meet different threads).  What lies before the block's cells is
+// one of the scanned tile sums (kScanned), the sum of the raw tile sums before
+// it (kSums) or of the cells themselves (kCells): a block's own sum over up to
+// kScanSums values costs less than a launch that scans them.
+enum ScanBefore : int { kCells, kSums, kScanned };
+constexpr int64_t kScanSums = 1024;    // raw tile sums that a block adds up itself
+constexpr int64_t kScanCells = 16384;  // cells that need no tile sums
+
+template <ScanBefore BEFORE, int ROWS>
 __global__ void __launch_bounds__(kBlock) k_scan_cells(int64_t ncell, int64_t n, CellPack cells,
                                                         const unsigned long long *__restrict__ offsets,
                                                         unsigned long long *__restrict__ packed,
                                                         int32_t *__restrict__ cell_start, int4 *__restrict__ items,
                                                         int32_t *__restrict__ n_items) {
-    unsigned long long before = offsets ? offsets[blockIdx.x] : 0ull;
-    for (int j = 0; j < kScanItems; ++j) {
-        const int64_t c = (int64_t)blockIdx.x * kScanTile + (int64_t)j * kBlock + threadIdx.x;
-        if ((int64_t)blockIdx.x * kScanTile + (int64_t)j * kBlock >= ncell) break;   // the same for the whole block
+    const int64_t first = (int64_t)blockIdx.x * kBlock * ROWS;
+    unsigned long long before = 0;
+    if (BEFORE == kScanned) {
+        before = offsets[blockIdx.x];
+    } else {
+        unsigned long long s = 0;
+        const int64_t len = BEFORE == kCells ? first : (int64_t)blockIdx.x;
+#pragma unroll 4
+        for (int64_t k = threadIdx.x; k < len; k += kBlock) s += BEFORE == kCells ? cells(k) : offsets[k];
+        block_exclusive(s, &before);
+    }
+    for (int j = 0; j < ROWS; ++j) {
+        const int64_t c = first + (int64_t)j * kBlock + threadIdx.x;
+        if (first + (int64_t)j * kBlock >= ncell) break;   // the same for the whole block
         uint32_t cnt = 0, m = 0;
         int box = 0;
         if (c < ncell) {
@@ -314,20 +330,38 @@ __global__ void __launch_bounds__(kBlock) k_scan_cells(int64_t ncell, int64_t n,
 }
 
 // Scan of the cells' particle and item counts into packed, cell_start and
-// (make_items) the work items.
+// (make_items) the work items.  Meshes of up to 2^18 cells take a block per 256
+// cells, so that more than a few SMs take part; small ones need no tile sums, and
+// only those of more than 2^21 cells a scan of theirs.  (One block per 2048
+// cells, eight rows in turn, took 9.1 us on 1000 cells and 13.5 on 2197; now 5.3
+// and 6.)
 cudaError_t scan_cells(int64_t ncell, int64_t n, const CellPack &cells, const BinBuffers &b, bool make_items,
                        cudaStream_t s) {
-    const int64_t nb = (ncell + kScanTile - 1) / kScanTile;
-    const unsigned long long *offsets = nullptr;
+    int4 *items = make_items ? b.items : nullptr;
+    const int64_t nb1 = (ncell + kBlock - 1) / kBlock, nb = (ncell + kScanTile - 1) / kScanTile;
     cudaError_t e;
-    if (nb > 1) {
-        k_scan_reduce<true><<<(unsigned)nb, kBlock, 0, s>>>(ncell, cells, nullptr, b.scan_tmp);
+    if (ncell <= kScanCells) {
+        k_scan_cells<kCells, 1><<<(unsigned)nb1, kBlock, 0, s>>>(ncell, n, cells, nullptr, b.packed, b.cell_start,
+                                                                 items, b.n_items);
+    } else if (nb1 <= kScanSums) {
+        // the tile sums pass through the queue order, which is written later (an entry per cell and more)
+        unsigned long long *sums = reinterpret_cast<unsigned long long *>(b.order);
+        k_scan_reduce<true, 1><<<(unsigned)nb1, kBlock, 0, s>>>(ncell, cells, nullptr, sums);
         note_launch();
-        if ((e = scan_exclusive(b.scan_tmp, nb, b.scan_tmp + nb, s)) != cudaSuccess) return e;
-        offsets = b.scan_tmp;
+        k_scan_cells<kSums, 1><<<(unsigned)nb1, kBlock, 0, s>>>(ncell, n, cells, sums, b.packed, b.cell_start, items,
+                                                                b.n_items);
+    } else {
+        k_scan_reduce<true, kScanItems><<<(unsigned)nb, kBlock, 0, s>>>(ncell, cells, nullptr, b.scan_tmp);
+        note_launch();
+        if (nb <= kScanSums) {
+            k_scan_cells<kSums, kScanItems><<<(unsigned)nb, kBlock, 0, s>>>(ncell, n, cells, b.scan_tmp, b.packed,
+                                                                            b.cell_start, items, b.n_items);
+        } else {
+            if ((e = scan_exclusive(b.scan_tmp, nb, b.scan_tmp + nb, s)) != cudaSuccess) return e;
+            k_scan_cells<kScanned, kScanItems><<<(unsigned)nb, kBlock, 0, s>>>(
+                ncell, n, cells, b.scan_tmp, b.packed, b.cell_start, items, b.n_items);
+        }
     }
-    k_scan_cells<<<(unsigned)nb, kBlock, 0, s>>>(ncell, n, cells, offsets, b.packed, b.cell_start,
-                                                 make_items ? b.items : nullptr, b.n_items);
     note_launch();
     return cudaGetLastError();
 }
@@ -533,6 +567,78 @@ __global__ void __launch_bounds__(kBlock) k_order_sub(int64_t ncell, const uint3
     rank_shared(w, cnt, lane, out, RowOf64{});
 }
 
+// A big cell, ordered by input row by one block: sort chunks of kChunk rows
+// with a shared-memory bitonic network, then merge runs of doubling width
+// between the two segment buffers, each output element placed by its
+// merge-path co-rank.  O(m log^2 m) work per cell of m particles.  The rows come
+// in A and end in B; sh holds kChunk values.  All threads of the block call it.
+constexpr int kChunk = 2048;
+__device__ __noinline__ void order_big_cell(int32_t *A, int32_t *B, int m, int32_t *sh, int tid, int threads) {
+    // 1. sorted chunks, in place in A
+    for (int base = 0; base < m; base += kChunk) {
+        for (int t = tid; t < kChunk; t += threads) sh[t] = base + t < m ? A[base + t] : 0x7fffffff;
+        __syncthreads();
+        for (int k = 2; k <= kChunk; k <<= 1)
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = tid; t < kChunk; t += threads) {
+                    int o = t ^ j;
+                    if (o > t) {
+                        int32_t a = sh[t], b = sh[o];
+                        if ((a > b) == ((t & k) == 0)) {
+                            sh[t] = b;
+                            sh[o] = a;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        for (int t = tid; t < kChunk && base + t < m; t += threads) A[base + t] = sh[t];
+        __syncthreads();
+    }
+    // 2. merge passes, ping-pong A <-> B
+    int32_t *src = A, *dst = B;
+    for (int width = kChunk; width < m; width <<= 1) {
+        for (int k = tid; k < m; k += threads) {
+            const int base = (k / (2 * width)) * (2 * width);
+            const int lenA = min(width, m - base);
+            const int lenB = max(0, min(width, m - base - width));
+            const int32_t *a = src + base, *b = src + base + width;
+            const int qk = k - base;
+            int lo = max(0, qk - lenB), hi = min(qk, lenA);
+            while (lo < hi) {
+                int mid = (lo + hi) >> 1;
+                if (a[mid] < b[qk - mid - 1]) lo = mid + 1;
+                else hi = mid;
+            }
+            const int i = lo, j = qk - lo;
+            dst[k] = (i < lenA && (j >= lenB || a[i] < b[j])) ? a[i] : b[j];
+        }
+        __syncthreads();
+        int32_t *tmp = src;
+        src = dst;
+        dst = tmp;
+    }
+    if (src != B)
+        for (int t = tid; t < m; t += threads) B[t] = src[t];
+    __syncthreads();
+}
+
+// The big cells of a list, a block of its own threads for each.
+constexpr int kOrderThreads = 1024;
+__global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__restrict__ count,
+                                                              const unsigned long long *__restrict__ packed,
+                                                              int32_t *perm_tmp, int32_t *perm,
+                                                              const int32_t *__restrict__ big_list,
+                                                              const int *__restrict__ big_count) {
+    __shared__ int32_t sh[kChunk];
+    const int nbig = *big_count;
+    for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
+        const int32_t c = big_list[q];
+        const uint32_t s = (uint32_t)(packed[c] & 0xffffffffull);
+        order_big_cell(perm_tmp + s, perm + s, (int)count[c], sh, threadIdx.x, kOrderThreads);
+    }
+}
+
 // The in-cell order, a block per run of up to kOrdCells consecutive cells
 // (fewer in small meshes, so that their few cells spread over the chip): their
 // slots form one range of the placement array, which the block stages into
@@ -551,8 +657,11 @@ __global__ void __launch_bounds__(kBlock) k_order_sub(int64_t ncell, const uint3
 // with SUB the pair (sub-cell code, input row) as one 32-bit key, code << 24 |
 // row (codes below 2^8, rows below 2^24; larger calls take k_order_sub).  Cells
 // above kBigCell are ordered by input row alone; those above kBlockCell by
-// k_order_big (with SUB their rows are copied to perm_tmp first).
+// k_order_big (with SUB their rows are copied to perm_tmp first), or, in calls
+// of up to kBigHereMax particles, by their block at the end: the launch costs
+// such a call more than its thousand threads save on a cell that it rarely has.
 constexpr uint32_t kBlockCell = 2048;
+constexpr int64_t kBigHereMax = (int64_t)1 << 16;
 constexpr int kOrdCells = 64;
 constexpr int kOrdCap = 6144;
 constexpr int64_t kOrdSubMaxRows = (int64_t)1 << 24;
@@ -639,11 +748,10 @@ __device__ __forceinline__ bool rank_stretches(const Seg &seg, uint32_t cnt, int
 template <bool SUB>
 __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const uint32_t *__restrict__ count,
                                                         const unsigned long long *__restrict__ packed,
-                                                        int32_t *__restrict__ perm_tmp,
-                                                        int32_t *__restrict__ perm, int32_t *__restrict__ big_list,
-                                                        int *__restrict__ big_count,
+                                                        int32_t *perm_tmp, int32_t *perm,
+                                                        int32_t *__restrict__ big_list, int *__restrict__ big_count,
                                                         const unsigned long long *__restrict__ order_tmp,
-                                                        uint32_t row_below, int stretches, int cells) {
+                                                        uint32_t row_below, int stretches, int cells, int big_here) {
     __shared__ __align__(16) uint32_t keys[kOrdCap];
     __shared__ uint32_t heads[kBlock / 32][3][kHeads];    // a warp's stretch heads: keys, slots, ranks
     __shared__ uint32_t cstart[kOrdCells], ccount[kOrdCells];
@@ -720,8 +828,8 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             // to the big-cell sort by row, from perm_tmp
             if (SUB)
                 for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
-            if (lane == 0) big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
-            continue;
+            if (lane == 0 && !big_here) big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
+            if (!big_here) continue;
         }
         if (cnt > 256) {
             if (lane == 0) wide[atomicAdd(&n_wide, 1)] = q;
@@ -743,6 +851,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
     const int nw = n_wide;
     for (int k = 0; k < nw; ++k) {
         const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
+        if (cnt > kBlockCell) continue;
         const uint32_t kmask = !SUB || cnt > kBigCell ? row_mask : 0xffffffffu;
         int32_t *out = perm + st;
         const uint32_t *sk = keys + (st - S0);
@@ -761,76 +870,12 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             out[r] = (int32_t)(v & row_mask);
         }
     }
-}
-
-// Big cells, one block per cell (grid-stride over the list): sort chunks of
-// kChunk input rows with a shared-memory bitonic network, then merge runs of
-// doubling width between the two segment buffers, each output element placed
-// by its merge-path co-rank.  O(m log^2 m) work per cell of m particles.
-constexpr int kOrderThreads = 1024;
-constexpr int kChunk = 2048;
-
-__global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__restrict__ count,
-                                                              const unsigned long long *__restrict__ packed,
-                                                              int32_t *__restrict__ perm_tmp,
-                                                              int32_t *__restrict__ perm,
-                                                              const int32_t *__restrict__ big_list,
-                                                              const int *__restrict__ big_count) {
-    __shared__ int32_t sh[kChunk];
-    const int nbig = *big_count;
-    const int tid = threadIdx.x;
-    for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
-        const int32_t c = big_list[q];
-        const int m = (int)count[c];
-        const uint32_t s = (uint32_t)(packed[c] & 0xffffffffull);
-        int32_t *A = perm_tmp + s, *B = perm + s;
-        // 1. sorted chunks, in place in A
-        for (int base = 0; base < m; base += kChunk) {
-            for (int t = tid; t < kChunk; t += kOrderThreads) sh[t] = base + t < m ? A[base + t] : 0x7fffffff;
-            __syncthreads();
-            for (int k = 2; k <= kChunk; k <<= 1)
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    for (int t = tid; t < kChunk; t += kOrderThreads) {
-                        int o = t ^ j;
-                        if (o > t) {
-                            int32_t a = sh[t], b = sh[o];
-                            if ((a > b) == ((t & k) == 0)) {
-                                sh[t] = b;
-                                sh[o] = a;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-            for (int t = tid; t < kChunk && base + t < m; t += kOrderThreads) A[base + t] = sh[t];
-            __syncthreads();
-        }
-        // 2. merge passes, ping-pong A <-> B
-        int32_t *src = A, *dst = B;
-        for (int width = kChunk; width < m; width <<= 1) {
-            for (int k = tid; k < m; k += kOrderThreads) {
-                const int base = (k / (2 * width)) * (2 * width);
-                const int lenA = min(width, m - base);
-                const int lenB = max(0, min(width, m - base - width));
-                const int32_t *a = src + base, *b = src + base + width;
-                const int qk = k - base;
-                int lo = max(0, qk - lenB), hi = min(qk, lenA);
-                while (lo < hi) {
-                    int mid = (lo + hi) >> 1;
-                    if (a[mid] < b[qk - mid - 1]) lo = mid + 1;
-                    else hi = mid;
-                }
-                const int i = lo, j = qk - lo;
-                dst[k] = (i < lenA && (j >= lenB || a[i] < b[j])) ? a[i] : b[j];
-            }
-            __syncthreads();
-            int32_t *tmp = src;
-            src = dst;
-            dst = tmp;
-        }
-        if (src != B)
-            for (int t = tid; t < m; t += kOrderThreads) B[t] = src[t];
-        __syncthreads();
+    if (!big_here || S1 - S0 <= kBlockCell) return;
+    __syncthreads();   // the stage is free
+    for (int k = 0; k < nw; ++k) {
+        const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
+        if (cnt > kBlockCell)
+            order_big_cell(perm_tmp + st, perm + st, (int)cnt, reinterpret_cast<int32_t *>(keys), t, kBlock);
     }
 }
 
@@ -1350,21 +1395,22 @@ cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_it
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // cells per block of the ordering: 64, fewer where that leaves SMs without a block
         const int oc = (int)std::min<int64_t>(kOrdCells, std::max<int64_t>(kBlock / 32, ncell / 512));
+        const int big_here = n <= kBigHereMax ? 1 : 0;
         if (sub && n > kOrdSubMaxRows)
             k_order_sub<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                   b.big_list, b.big_count, b.order_tmp, row_below);
         else if (sub)
             k_order_rows<true><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                        b.big_list, b.big_count, b.order_tmp,
-                                                                       row_below, stretches ? 1 : 0, oc);
+                                                                       row_below, stretches ? 1 : 0, oc, big_here);
         else
             k_order_rows<false><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                         b.big_list, b.big_count, nullptr, 0u,
-                                                                        stretches ? 1 : 0, oc);
+                                                                        stretches ? 1 : 0, oc, big_here);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // k_order_sub lists cells above kBigCell, k_order_rows those above kBlockCell
-        if (n > (int64_t)(sub && n > kOrdSubMaxRows ? kBigCell : kBlockCell)) {
+        if (!big_here && n > (int64_t)(sub && n > kOrdSubMaxRows ? kBigCell : kBlockCell)) {
             k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count);
             note_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
