@@ -257,7 +257,8 @@ hacc_status check_particles(hacc_ctx *ctx, int64_t n, const void *a, const void 
 hacc_status launch_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts &fc, const ForceLaunch &fl, bool counted,
                          cudaStream_t s);
 
-// The short-range force on sorted positions (w->Ps, cell starts and items in w->b).
+// The short-range force on sorted positions (w->Ps, cell starts and items in
+// w->b), once after each binning.
 hacc_status run_sorted_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts &fc, Work *w, int mode,
                              float4 *out, const int32_t *perm, float4 *vel, float4 *pos_next, float hk, float hd,
                              unsigned long long *within, cudaStream_t s, int64_t n = 0) {
@@ -270,7 +271,8 @@ hacc_status run_sorted_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts
     fl.items = w->b.items;
     fl.n_items = w->b.n_items;
     fl.cell_start = w->b.cell_start;
-    fl.work_counter = w->counter;
+    fl.work_counter = w->b.work_counter;
+    fl.counter_clear = true;
     fl.mode = mode;
     fl.out = out;
     fl.perm = perm;
@@ -484,9 +486,8 @@ hacc_status hacc_tune(hacc_ctx *ctx, const hacc_box *box, const hacc_split *spli
     // one sub-cycle's chaining-mesh build and pair-kernel launch (kick + stream)
     auto subcycle_work = [&](int cap, bool first) -> hacc_status {
         HACC_CUDA(bin_build(g, n, first ? src : w.P, nullptr, 0.0f, w.P, w.b, ctx->d_flags, true, s, cap,
-                            ctx->split_max, nullptr, !first),
+                            ctx->split_max, nullptr, !first, Gather{w.P, w.Ps, w.V, w.Vs, nullptr, w.IDs}),
                   "tuner binning");
-        HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, w.V, w.Vs, nullptr, w.IDs, s), "tuner gather");
         return run_sorted_force(ctx, g, fc, &w, kModeKickDrift, nullptr, nullptr, w.Vs, w.P, h, h, nullptr, s, n);
     };
     for (int k = 0; k < kTuneSettings && st == HACC_OK; ++k) {
@@ -614,9 +615,8 @@ hacc_status hacc_sr_force(hacc_ctx *ctx, const hacc_box *box, const hacc_split *
     HACC_TRY(prepare_work(ctx, n, g, false, s, &w));
     const float4 *src = reinterpret_cast<const float4 *>(pos_m);
     HACC_CUDA(bin_build(g, n, src, nullptr, 0.0f, w.P, w.b, ctx->d_flags, true, s, item_cap_for(ctx, n),
-                        ctx->split_max),
+                        ctx->split_max, nullptr, false, Gather{w.P, w.Ps}),
               "binning");
-    HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, nullptr, nullptr, nullptr, nullptr, s), "gather");
     unsigned long long *within = nullptr;
     if (pair_counts) {
         unsigned long long *pc = reinterpret_cast<unsigned long long *>(pair_counts);
@@ -657,11 +657,9 @@ hacc_status hacc_subcycle(hacc_ctx *ctx, const hacc_box *box, const hacc_split *
         std::pair<cudaEvent_t, cudaEvent_t> ev;
         HACC_TRY(timing_begin(ctx, s, &ev));
         HACC_CUDA(bin_build(g, n, first ? pos_in : w.P, first ? vel_in : nullptr, h2, w.P, w.b, ctx->d_flags, true,
-                            s, item_cap_for(ctx, n), ctx->split_max, nullptr, !first),
+                            s, item_cap_for(ctx, n), ctx->split_max, nullptr, !first,
+                            Gather{w.P, w.Ps, first ? vel_in : w.V, w.Vs, first ? nullptr : w.ID, w.IDs}),
                   "binning");
-        HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, first ? vel_in : w.V, w.Vs, first ? nullptr : w.ID, w.IDs,
-                                s),
-                  "gather");
         HACC_TRY(timing_end(ctx, s, ev, 1));
         // kick h, then stream h (fused halves) or h/2 (closing the last sub-cycle);
         // positions of this sub-cycle's sorted order go to w.P
@@ -709,7 +707,8 @@ hacc_status ci_force(hacc_ctx *ctx, const Geometry &g, const ForceConsts &fc, Wo
     fl.items = w->b.items;
     fl.n_items = w->b.n_items;
     fl.cell_start = w->b.cell_start;
-    fl.work_counter = w->counter;
+    fl.work_counter = w->b.work_counter;
+    fl.counter_clear = true;
     fl.mode = mode;
     fl.out = out;
     fl.perm = w->b.perm;
@@ -748,9 +747,8 @@ hacc_status hacc_sr_force_ci(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
     HACC_TRY(prepare_work(ctx, n, g, false, s, &w));
     // no stream: the cell ids are the keys as stored (cell and off_m are not written)
     HACC_CUDA(bin_build_ci(g, n, const_cast<int32_t *>(cell), reinterpret_cast<float4 *>(const_cast<float *>(off_m)),
-                           nullptr, 0.0, w.P, w.b, ctx->d_flags, s),
+                           nullptr, 0.0, w.P, w.b, ctx->d_flags, s, Gather{w.P, w.Ps}),
               "binning");
-    HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, nullptr, nullptr, nullptr, nullptr, s), "gather");
     return ci_force(ctx, g, fc, &w, kModeForce, reinterpret_cast<float4 *>(acc), nullptr, 0.f, s);
 }
 
@@ -771,10 +769,9 @@ hacc_status hacc_diagnostics_ci(hacc_ctx *ctx, const hacc_box *box, const hacc_s
     Work w;
     HACC_TRY(prepare_work(ctx, n, g, true, s, &w));
     HACC_CUDA(bin_build_ci(g, n, const_cast<int32_t *>(cell), reinterpret_cast<float4 *>(const_cast<float *>(off_m)),
-                           nullptr, 0.0, w.P, w.b, ctx->d_flags, s),
+                           nullptr, 0.0, w.P, w.b, ctx->d_flags, s,
+                           Gather{w.P, w.Ps, reinterpret_cast<const float4 *>(vel), w.Vs}),
               "binning");
-    HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, reinterpret_cast<const float4 *>(vel), w.Vs, nullptr, nullptr, s),
-              "gather");
     ForceLaunch fl;
     fl.pos = w.Ps;
     fl.items = w.b.items;
@@ -822,8 +819,9 @@ hacc_status hacc_subcycle_ci(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
     const double h = dt / n_sub;
     for (int k = 0; k < n_sub; ++k) {
         // stream (FP64 on the global position: h/2 opening, then h fusing two halves), rebin
-        HACC_CUDA(bin_build_ci(g, n, cell, off, v, k == 0 ? 0.5 * h : h, w.P, w.b, ctx->d_flags, s), "binning");
-        HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, v, w.Vs, nullptr, nullptr, s), "gather");
+        HACC_CUDA(bin_build_ci(g, n, cell, off, v, k == 0 ? 0.5 * h : h, w.P, w.b, ctx->d_flags, s,
+                               Gather{w.P, w.Ps, v, w.Vs}),
+                  "binning");
         // kick h (FP32), velocities back to input order
         HACC_TRY(ci_force(ctx, g, fc, &w, kModeKick, nullptr, v, (float)h, s));
     }
@@ -1185,10 +1183,9 @@ hacc_status hacc_diagnostics(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
     }
     const float4 *src = reinterpret_cast<const float4 *>(pos_m);
     HACC_CUDA(bin_build(g, n, src, nullptr, 0.0f, w.P, w.b, ctx->d_flags, true, s, item_cap_for(ctx, n),
-                        ctx->split_max),
+                        ctx->split_max, nullptr, false,
+                        Gather{w.P, w.Ps, reinterpret_cast<const float4 *>(vel), w.Vs}),
               "binning");
-    HACC_CUDA(gather_sorted(n, w.b.perm, w.P, w.Ps, reinterpret_cast<const float4 *>(vel), w.Vs, nullptr, nullptr, s),
-              "gather");
     HACC_TRY(run_sorted_force(ctx, g, fc, &w, kModePotential, nullptr, nullptr, nullptr, nullptr, 0.f, 0.f, nullptr,
                               s));
     HACC_CUDA(diag_reduce(n, w.Ps, w.Vs, w.phi, out, s), "diagnostics");

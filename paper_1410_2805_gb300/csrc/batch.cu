@@ -145,17 +145,16 @@ hacc_status run_tick(hacc_ctx *ctx, const ForceConsts &fc, const Plan &pl, const
                      float4 *vel_pool, const BatchWork &w, cudaStream_t s) {
     const Shape sh = batch_shape(ctx, pl);
     HACC_CUDA_RETURN(bin_build_batch(pl.nbox, tab, pl.n_total, pl.ncell_total, pos_pool, vel_pool, w.P, w.ID, w.b,
-                                     ctx->d_flags, s, sh.cap, ctx->split_max),
+                                     ctx->d_flags, s, sh.cap, ctx->split_max,
+                                     Gather{w.P, w.Ps, vel_pool, w.Vs, w.ID, w.IDs, true}),
                      "batched binning");
-    HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.b.perm, w.P, w.Ps, nullptr, nullptr, w.ID, w.IDs, s), "gather");
-    HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.IDs, vel_pool, w.Vs, nullptr, nullptr, nullptr, nullptr, s),
-                     "gather velocities");
     ForceLaunch fl;
     fl.pos = w.Ps;
     fl.items = w.b.items;
     fl.n_items = w.b.n_items;
     fl.cell_start = w.b.cell_start;
-    fl.work_counter = w.counter;
+    fl.work_counter = w.b.work_counter;
+    fl.counter_clear = true;
     fl.mode = kModeBatch;
     fl.out = nullptr;
     fl.perm = nullptr;
@@ -436,11 +435,9 @@ extern "C" hacc_status hacc_batch_diagnostics(hacc_ctx *ctx, const hacc_split *s
     float4 *vp = const_cast<float4 *>(reinterpret_cast<const float4 *>(vel_pool));
     // the pools are only read: the binning writes wrapped copies to scratch
     HACC_CUDA_RETURN(bin_build_batch(pl.nbox, w.tables, pl.n_total, pl.ncell_total, pp, vp, w.P, w.ID, w.b,
-                                     ctx->d_flags, s, ctx->item_cap, ctx->split_max),
+                                     ctx->d_flags, s, ctx->item_cap, ctx->split_max,
+                                     Gather{w.P, w.Ps, vp, w.Vs, w.ID, w.IDs, true}),
                      "batched binning");
-    HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.b.perm, w.P, w.Ps, nullptr, nullptr, w.ID, w.IDs, s), "gather");
-    HACC_CUDA_RETURN(gather_sorted(pl.n_total, w.IDs, vp, w.Vs, nullptr, nullptr, nullptr, nullptr, s),
-                     "gather velocities");
     ForceLaunch fl;
     fl.pos = w.Ps;
     fl.items = w.b.items;

@@ -11,7 +11,8 @@
 //   k_place   perm_tmp[start[c] + slot] = i, [its sub-cell] read 12-13 B, write 4-5 B
 //   k_order   within each cell, sort perm by input row (stable order) or by
 //             (sub-cell, input row)
-//   gather    sorted copies of positions / velocities / ids
+//   gather    sorted copies of positions / velocities / ids (calls of up to 2^20
+//             particles: in the blocks of k_order)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -279,7 +280,7 @@ cudaError_t scan_exclusive(unsigned long long *data, int64_t len, unsigned long 
 // kScanSums values costs less than a launch that scans them.
 enum ScanBefore : int { kCells, kSums, kScanned };
 constexpr int64_t kScanSums = 1024;    // raw tile sums that a block adds up itself
-constexpr int64_t kScanCells = 16384;  // cells that need no tile sums
+constexpr int64_t kScanCells = 4096;   // cells that need no tile sums
 
 template <ScanBefore BEFORE, int ROWS>
 __global__ void __launch_bounds__(kBlock) k_scan_cells(int64_t ncell, int64_t n, CellPack cells,
@@ -380,6 +381,14 @@ __global__ void __launch_bounds__(kBlock) k_place(int64_t n, const int32_t *__re
     // scattered write, as for the row alone)
     if (sub) order_tmp[at] = ((unsigned long long)sub[i] << 32) | (uint32_t)i;
     else perm_tmp[at] = (int32_t)i;
+}
+
+// Sorted copies of input row i in slot k.
+__device__ __forceinline__ void gather_row(const Gather &g, int64_t k, int32_t i) {
+    g.p_out[k] = g.p_in[i];
+    const int32_t id = g.id_in ? g.id_in[i] : i;
+    if (g.v_out) g.v_out[k] = g.v_in[g.v_by_id ? id : i];
+    if (g.id_out) g.id_out[k] = id;
 }
 
 // The arrival order from the atomics is arbitrary, so each element's final
@@ -629,13 +638,16 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
                                                               const unsigned long long *__restrict__ packed,
                                                               int32_t *perm_tmp, int32_t *perm,
                                                               const int32_t *__restrict__ big_list,
-                                                              const int *__restrict__ big_count) {
+                                                              const int *__restrict__ big_count, Gather gather) {
     __shared__ int32_t sh[kChunk];
     const int nbig = *big_count;
     for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
         const int32_t c = big_list[q];
         const uint32_t s = (uint32_t)(packed[c] & 0xffffffffull);
-        order_big_cell(perm_tmp + s, perm + s, (int)count[c], sh, threadIdx.x, kOrderThreads);
+        const uint32_t m = count[c];
+        order_big_cell(perm_tmp + s, perm + s, (int)m, sh, threadIdx.x, kOrderThreads);
+        if (gather.p_out)
+            for (uint32_t e = s + threadIdx.x; e < s + m; e += kOrderThreads) gather_row(gather, e, perm[e]);
     }
 }
 
@@ -651,9 +663,10 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
 // cell tries the stretch ranking in shared memory, and otherwise a cell of up to
 // 256 keys is sorted by a bitonic network over 2, 4 or 8 keys per lane.  Cells
 // of up to kBlockCell keys wait until the warps are through and are then ranked
-// by the whole block, a key per thread counting the smaller ones (by one warp, a
-// cell of 400 keys took 60 us: with the smaller blocks the pass went from 82 to 18
-// us on a 32^3 blob box and from 116 to 51 us on 2 million blob particles).  The key is the input row (row order), or
+// by the whole block: the keys go to 256 buckets of equal width, and a thread
+// counts the smaller ones in its key's bucket (by one warp, a cell of 400 keys
+// took 60 us; with every smaller key of the cell counted, 4099 blob particles
+// took 11 us, 2 million 50, now 34).  The key is the input row (row order), or
 // with SUB the pair (sub-cell code, input row) as one 32-bit key, code << 24 |
 // row (codes below 2^8, rows below 2^24; larger calls take k_order_sub).  Cells
 // above kBigCell are ordered by input row alone; those above kBlockCell by
@@ -662,6 +675,11 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
 // such a call more than its thousand threads save on a cell that it rarely has.
 constexpr uint32_t kBlockCell = 2048;
 constexpr int64_t kBigHereMax = (int64_t)1 << 16;
+// Calls of up to this many particles gather in the ordering's blocks: a launch
+// fewer (250 thousand particles: call 205.5 -> 202 us).  Larger ones hide more
+// latency with a thread per particle (6 served boxes, 3.6 million: 2038 us a
+// tick in the blocks, 2001 on their own).
+constexpr int64_t kGatherHereMax = (int64_t)1 << 20;
 constexpr int kOrdCells = 64;
 constexpr int kOrdCap = 6144;
 constexpr int64_t kOrdSubMaxRows = (int64_t)1 << 24;
@@ -751,16 +769,19 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
                                                         int32_t *perm_tmp, int32_t *perm,
                                                         int32_t *__restrict__ big_list, int *__restrict__ big_count,
                                                         const unsigned long long *__restrict__ order_tmp,
-                                                        uint32_t row_below, int stretches, int cells, int big_here) {
+                                                        uint32_t row_below, int stretches, int cells, int big_here,
+                                                        Gather gather) {
     __shared__ __align__(16) uint32_t keys[kOrdCap];
     __shared__ uint32_t heads[kBlock / 32][3][kHeads];    // a warp's stretch heads: keys, slots, ranks
+    static_assert(sizeof heads >= sizeof(uint32_t) * (kBlockCell + kBlock), "a wide cell's buckets take their place");
     __shared__ uint32_t cstart[kOrdCells], ccount[kOrdCells];
     __shared__ int next_cell;   // the warps take the block's cells in turn (cells differ widely in cost)
     __shared__ int wide[kOrdCells], n_wide;   // cells for the whole block
+    __shared__ int n_later;                   // set: cells for k_order_big
     const int64_t c0 = (int64_t)blockIdx.x * cells;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int ncb = ncell - c0 < cells ? (int)(ncell - c0) : cells;   // cells of this block (>= 1)
-    if (t == 0) next_cell = n_wide = 0;
+    if (t == 0) next_cell = n_wide = n_later = 0;
     if (t < kOrdCells) {
         uint32_t cnt = 0, st = 0;
         if (t < ncb) {
@@ -828,7 +849,10 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             // to the big-cell sort by row, from perm_tmp
             if (SUB)
                 for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
-            if (lane == 0 && !big_here) big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
+            if (lane == 0 && !big_here) {
+                big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
+                n_later = 1;
+            }
             if (!big_here) continue;
         }
         if (cnt > 256) {
@@ -849,11 +873,11 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
     // the wide cells: their ranks do not depend on the order in which the warps
     // listed them
     const int nw = n_wide;
+    uint32_t *slots = &heads[0][0][0], *first = slots + kBlockCell;
     for (int k = 0; k < nw; ++k) {
         const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
         if (cnt > kBlockCell) continue;
         const uint32_t kmask = !SUB || cnt > kBigCell ? row_mask : 0xffffffffu;
-        int32_t *out = perm + st;
         const uint32_t *sk = keys + (st - S0);
         if (!staged) {
             // a cell at a time through the stage (cnt <= kBlockCell <= kOrdCap)
@@ -862,20 +886,56 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             __syncthreads();
             sk = keys;
         }
+        // the cell's lowest and highest key
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (uint32_t e = lane; e < cnt; e += 32) {
+            lo = min(lo, sk[e] & kmask);
+            hi = max(hi, sk[e] & kmask);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        // its keys in kBlock buckets, by their distance from the lowest
+        const int shift = max(0, 24 - __clz(hi - lo));
+        first[t] = 0;
+        __syncthreads();
+        for (uint32_t e = t; e < cnt; e += kBlock) atomicAdd(&first[((sk[e] & kmask) - lo) >> shift], 1u);
+        __syncthreads();
+        const uint32_t own = first[t], at = (uint32_t)block_exclusive(own, nullptr);
+        first[t] = at;
+        __syncthreads();
+        // the buckets' keys, each bucket's in any order; first[b] moves on to its end
         for (uint32_t e = t; e < cnt; e += kBlock) {
             const uint32_t v = sk[e] & kmask;
-            uint32_t r = 0;
-#pragma unroll 8
-            for (uint32_t u = 0; u < cnt; ++u) r += (sk[u] & kmask) < v ? 1u : 0u;
+            slots[atomicAdd(&first[(v - lo) >> shift], 1u)] = v;
+        }
+        __syncthreads();
+        int32_t *out = perm + st;
+        for (uint32_t e = t; e < cnt; e += kBlock) {
+            const uint32_t v = slots[e], b = (v - lo) >> shift;
+            const uint32_t a = b ? first[b - 1] : 0u, z = first[b];
+            uint32_t r = a;
+#pragma unroll 4
+            for (uint32_t u = a; u < z; ++u) r += slots[u] < v ? 1u : 0u;
             out[r] = (int32_t)(v & row_mask);
         }
+        __syncthreads();   // slots and first are free
     }
-    if (!big_here || S1 - S0 <= kBlockCell) return;
-    __syncthreads();   // the stage is free
-    for (int k = 0; k < nw; ++k) {
-        const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
-        if (cnt > kBlockCell)
-            order_big_cell(perm_tmp + st, perm + st, (int)cnt, reinterpret_cast<int32_t *>(keys), t, kBlock);
+    if (big_here && S1 - S0 > kBlockCell) {
+        __syncthreads();   // the stage is free
+        for (int k = 0; k < nw; ++k) {
+            const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
+            if (cnt > kBlockCell)
+                order_big_cell(perm_tmp + st, perm + st, (int)cnt, reinterpret_cast<int32_t *>(keys), t, kBlock);
+        }
+    }
+    if (!gather.p_out) return;
+    __syncthreads();
+    const bool some_later = n_later;   // cells that k_order_big orders and gathers
+    for (uint32_t e = S0 + t; e < S1; e += kBlock) {
+        bool later = false;
+        if (some_later)
+            for (int q = 0; q < ncb; ++q) later |= ccount[q] > kBlockCell && e - cstart[q] < ccount[q];
+        if (!later) gather_row(gather, e, perm[e]);
     }
 }
 
@@ -923,16 +983,9 @@ __global__ void __launch_bounds__(kBlock) k_bkey(int64_t n_total, int nbox, cons
     if (t < n_total) rank[t] = (int32_t)slot;
 }
 
-__global__ void __launch_bounds__(kBlock) k_gather(int64_t n, const int32_t *__restrict__ perm,
-                                                    const float4 *__restrict__ p_in, float4 *__restrict__ p_out,
-                                                    const float4 *__restrict__ v_in, float4 *__restrict__ v_out,
-                                                    const int32_t *__restrict__ id_in, int32_t *__restrict__ id_out) {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    int32_t i = perm[k];
-    p_out[k] = p_in[i];
-    if (v_out) v_out[k] = v_in[i];
-    if (id_out) id_out[k] = id_in ? id_in[i] : i;
+__global__ void __launch_bounds__(kBlock) k_gather(int64_t n, const int32_t *__restrict__ perm, Gather g) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) gather_row(g, k, perm[k]);
 }
 
 // Multi-level rebinning: gather positions (and a copy, the binned reference),
@@ -1351,8 +1404,9 @@ cudaError_t items_heavy_first(const BinBuffers &b, int64_t max_items, cudaStream
     return cudaGetLastError();
 }
 
-// counters next to the cell counts that one memset clears with them: mass_flag, big_count
-constexpr int kZeroTail = 2;
+// counters next to the cell counts that one memset clears with them: mass_flag,
+// big_count, work_counter (a memset of its own costs a small call 2 us)
+constexpr int kZeroTail = 3;
 
 void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_order) {
     b->key = c.take<int32_t>(n);
@@ -1360,6 +1414,7 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
     b->count = c.take<uint32_t>(ncell + kZeroTail);   // then the flags that start at zero with the counts
     b->mass_flag = b->count ? reinterpret_cast<int *>(b->count + ncell) : nullptr;
     b->big_count = b->count ? reinterpret_cast<int *>(b->count + ncell) + 1 : nullptr;
+    b->work_counter = b->count ? reinterpret_cast<int *>(b->count + ncell) + 2 : nullptr;
     b->packed = c.take<unsigned long long>(ncell);
     b->scan_tmp = c.take<unsigned long long>(scan_tmp_elems(ncell));
     b->cell_start = c.take<int32_t>(ncell + 1);
@@ -1385,8 +1440,8 @@ ItemRule item_rule(int item_cap, int split_max) {
 
 // Counting sort by key and work items, shared by the single-box and batched passes.
 cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_items, const BoxDev *boxes, int nbox,
-                     cudaStream_t s, ItemRule cap = {kItemMax / kCluster, 0xffffffffu}, const uint8_t *sub = nullptr,
-                     uint32_t row_below = 0, bool stretches = false) {
+                     cudaStream_t s, ItemRule cap, const uint8_t *sub,
+                     uint32_t row_below, bool stretches, const Gather &gather) {
     cudaError_t e = scan_cells(ncell, n, CellPack{b.count, cap, boxes, nbox}, b, make_items, s);
     if (e != cudaSuccess) return e;
     if (n > 0) {
@@ -1396,22 +1451,30 @@ cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_it
         // cells per block of the ordering: 64, fewer where that leaves SMs without a block
         const int oc = (int)std::min<int64_t>(kOrdCells, std::max<int64_t>(kBlock / 32, ncell / 512));
         const int big_here = n <= kBigHereMax ? 1 : 0;
-        if (sub && n > kOrdSubMaxRows)
+        const bool by_row = !(sub && n > kOrdSubMaxRows);   // in k_order_rows
+        const Gather here = by_row && n <= kGatherHereMax ? gather : Gather{};
+        if (!by_row)
             k_order_sub<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                   b.big_list, b.big_count, b.order_tmp, row_below);
         else if (sub)
             k_order_rows<true><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                        b.big_list, b.big_count, b.order_tmp,
-                                                                       row_below, stretches ? 1 : 0, oc, big_here);
+                                                                       row_below, stretches ? 1 : 0, oc, big_here, here);
         else
             k_order_rows<false><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
                                                                         b.big_list, b.big_count, nullptr, 0u,
-                                                                        stretches ? 1 : 0, oc, big_here);
+                                                                        stretches ? 1 : 0, oc, big_here, here);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // k_order_sub lists cells above kBigCell, k_order_rows those above kBlockCell
-        if (!big_here && n > (int64_t)(sub && n > kOrdSubMaxRows ? kBigCell : kBlockCell)) {
-            k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count);
+        if (!big_here && n > (int64_t)(by_row ? kBlockCell : kBigCell)) {
+            k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count,
+                                                      here);
+            note_launch();
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        if (!here.p_out && gather.p_out) {
+            k_gather<<<blocks_for(n), kBlock, 0, s>>>(n, b.perm, gather);
             note_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
@@ -1422,7 +1485,7 @@ cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_it
 
 cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const float4 *vel, float drift,
                       float4 *dst, const BinBuffers &b, int *d_flags, bool make_items, cudaStream_t s,
-                      int item_cap, int split_max, const int32_t *sub_level, bool sorted_input) {
+                      int item_cap, int split_max, const int32_t *sub_level, bool sorted_input, const Gather &gather) {
     if (item_cap != 0 && (item_cap < kCluster || item_cap > kItemCapMax)) return cudaErrorInvalidValue;
     if (split_max < 1 || ((item_cap || sub_level) && !b.sub)) return cudaErrorInvalidValue;
     uint8_t *sub = (item_cap || sub_level) ? b.sub : nullptr;
@@ -1438,7 +1501,7 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
     // order an event's items rely on)
     const uint32_t row_below = (item_cap && !sub_level) ? (uint32_t)kCluster : 0u;
     return bin_sort(n, g.ncell, b, make_items, nullptr, 1, s, item_rule(item_cap, split_max), sub, row_below,
-                    sorted_input);
+                    sorted_input, gather);
 }
 
 cudaError_t ml_levels(const Geometry &g, int64_t n, const BinBuffers &b, int d, int lmin, int lmax, int32_t *level,
@@ -1488,7 +1551,8 @@ cudaError_t items_kicked(int64_t ncell, const BinBuffers &b, const int32_t *leve
 
 cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int64_t ncell_total,
                             const float4 *pos_pool, const float4 *vel_pool, float4 *dst, int32_t *id,
-                            const BinBuffers &b, int *d_flags, cudaStream_t s, int item_cap, int split_max) {
+                            const BinBuffers &b, int *d_flags, cudaStream_t s, int item_cap, int split_max,
+                            const Gather &gather) {
     if (item_cap > 0 && (item_cap < kCluster || item_cap > kItemCapMax)) return cudaErrorInvalidValue;
     if (split_max < 1 || (item_cap && !b.sub)) return cudaErrorInvalidValue;
     uint8_t *sub = item_cap ? b.sub : nullptr;
@@ -1502,11 +1566,11 @@ cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int6
     }
     // as bin_build: a cell of a single cluster keeps row order
     return bin_sort(n_total, ncell_total, b, true, boxes, nbox, s, item_rule(item_cap, split_max), sub,
-                    item_cap ? (uint32_t)kCluster : 0u, false);
+                    item_cap ? (uint32_t)kCluster : 0u, false, gather);
 }
 
 cudaError_t bin_build_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
-                         float4 *dst, const BinBuffers &b, int *d_flags, cudaStream_t s) {
+                         float4 *dst, const BinBuffers &b, int *d_flags, cudaStream_t s, const Gather &gather) {
     cudaError_t e = cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * (g.ncell + kZeroTail), s);
     if (e != cudaSuccess) return e;
     if (n > 0) {
@@ -1515,7 +1579,8 @@ cudaError_t bin_build_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *of
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    return bin_sort(n, g.ncell, b, true, nullptr, 1, s, item_rule(kItemMax, kDefaultSplitMax), b.sub, kCluster);
+    return bin_sort(n, g.ncell, b, true, nullptr, 1, s, item_rule(kItemMax, kDefaultSplitMax), b.sub, kCluster,
+                    false, gather);
 }
 
 cudaError_t drift_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
@@ -1540,14 +1605,6 @@ cudaError_t ci_to_f64(const Geometry &g, int64_t n, const int32_t *cell, const f
                       cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     k_ci_to_f64<<<blocks_for(n), kBlock, 0, s>>>(n, cell, off, g.nc, ci_step(g), x64);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t gather_sorted(int64_t n, const int32_t *perm, const float4 *p_in, float4 *p_out, const float4 *v_in,
-                          float4 *v_out, const int32_t *id_in, int32_t *id_out, cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    k_gather<<<blocks_for(n), kBlock, 0, s>>>(n, perm, p_in, p_out, v_in, v_out, id_in, id_out);
     note_launch();
     return cudaGetLastError();
 }

@@ -243,8 +243,22 @@ struct BinBuffers {
     int *mass_flag;        // [1] device: nonzero if some mass differs from the first
     int32_t *big_list;     // cells too large for the warp-level ordering
     int *big_count;
+    int *work_counter;     // [1] device: cleared by each binning (the force launch that follows it)
     uint8_t *sub;                  // [n] Morton sub-cell of each input row (item_cap > 0), or null
     unsigned long long *order_tmp; // [n] (sub-cell << 32 | row) in the slots of perm_tmp, or null
+};
+
+// Sorted copies that a binning makes on its way (p_out null: none): slot k gets
+// the position, velocity (of row i, or with v_by_id of row id) and id (id_in
+// null: i itself) of input row i = perm[k].
+struct Gather {
+    const float4 *p_in = nullptr;
+    float4 *p_out = nullptr;
+    const float4 *v_in = nullptr;
+    float4 *v_out = nullptr;
+    const int32_t *id_in = nullptr;
+    int32_t *id_out = nullptr;
+    bool v_by_id = false;
 };
 
 size_t scan_tmp_elems(int64_t len);
@@ -278,7 +292,7 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
 cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const float4 *vel, float drift,
                       float4 *dst, const BinBuffers &b, int *d_flags, bool make_items, cudaStream_t s,
                       int item_cap = 0, int split_max = kDefaultSplitMax, const int32_t *sub_level = nullptr,
-                      bool sorted_input = false);
+                      bool sorted_input = false, const Gather &gather = {});
 
 // Batched binning of nbox boxes (table `boxes` on the device, ascending
 // part_base and cell_base): for every tick-scratch index t the particle at
@@ -290,7 +304,7 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
 cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int64_t ncell_total,
                             const float4 *pos_pool, const float4 *vel_pool, float4 *dst, int32_t *id,
                             const BinBuffers &b, int *d_flags, cudaStream_t s, int item_cap = 0,
-                            int split_max = kDefaultSplitMax);
+                            int split_max = kDefaultSplitMax, const Gather &gather = {});
 
 // Multi-level stepping: kick counts from the cell densities of the last
 // binning (keys/counts in b; present[l] += particles with l kicks); in-place stream of
@@ -323,18 +337,13 @@ cudaError_t items_kicked(int64_t ncell, const BinBuffers &b, const int32_t *leve
 // Precision variant: positions as (cell id, FP32 in-cell offset, mass).
 // bin_build_ci optionally streams (FP64 on the global position) first.
 cudaError_t bin_build_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
-                         float4 *dst, const BinBuffers &b, int *d_flags, cudaStream_t s);
+                         float4 *dst, const BinBuffers &b, int *d_flags, cudaStream_t s, const Gather &gather = {});
 cudaError_t drift_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
                      int *d_flags, cudaStream_t s);
 cudaError_t ci_from_f64(const Geometry &g, int64_t n, const double *x64, const float *mass, int32_t *cell,
                         float4 *off, int *d_flags, cudaStream_t s);
 cudaError_t ci_to_f64(const Geometry &g, int64_t n, const int32_t *cell, const float4 *off, double *x64,
                       cudaStream_t s);
-
-// Gather rows into sorted order: out[k] = in[perm[k]] for float4, int ids.
-cudaError_t gather_sorted(int64_t n, const int32_t *perm, const float4 *p_in, float4 *p_out,
-                          const float4 *v_in, float4 *v_out, const int32_t *id_in, int32_t *id_out,
-                          cudaStream_t s);
 
 // Scatter rows back to input order: out[id[k]] = in[k]; positions are
 // wrapped into [0, L) on the way (flagging coordinates outside [-L, 2L)).
@@ -368,7 +377,8 @@ struct ForceLaunch {
     const int4 *items;
     const int32_t *n_items;     // device count
     const int32_t *cell_start;
-    int *work_counter;          // zeroed before launch
+    int *work_counter;          // zeroed before launch,
+    bool counter_clear = false; // or by the binning just before it
     bool cull = true;           // select the neighbours per cluster, else by the item's bounds alone
     int mode;
     // kModeForce: out[perm[i]] (perm null: out[i])

@@ -65,12 +65,11 @@ cudaError_t setup_device(int dev, DeviceSetup **out) {
 }
 
 // Layout of the fixed scratch for one call (same carving as the context path).
-size_t carve_noalloc(char *base, int64_t n, int64_t ncell, float4 **P, float4 **Ps, int **counter, int **flags,
+size_t carve_noalloc(char *base, int64_t n, int64_t ncell, float4 **P, float4 **Ps, int **flags,
                      BinBuffers *b) {
     Carver c(base);
     *P = c.take<float4>(n);
     *Ps = c.take<float4>(n);
-    *counter = c.take<int>(1);
     *flags = c.take<int>(4);
     carve_bin(c, n, ncell, b, false);
     return c.off;
@@ -95,10 +94,10 @@ extern "C" hacc_status hacc_sr_force_noalloc(const hacc_box *box, const hacc_spl
     st = make_force_consts(nullptr, split, g, &fc);
     if (st != HACC_OK) return st;
     float4 *P, *Ps;
-    int *counter, *flags;
+    int *flags;
     BinBuffers b;
     // sizes beyond the fixed array are refused before anything is enqueued
-    if (carve_noalloc(nullptr, n, g.ncell, &P, &Ps, &counter, &flags, &b) > kNoAllocScratchBytes)
+    if (carve_noalloc(nullptr, n, g.ncell, &P, &Ps, &flags, &b) > kNoAllocScratchBytes)
         return HACC_ENOMEM;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return HACC_ECUDA;
@@ -112,20 +111,22 @@ extern "C" hacc_status hacc_sr_force_noalloc(const hacc_box *box, const hacc_spl
     if (stream_dev != dev) return HACC_EINVAL;
     DeviceSetup *ds = nullptr;
     if (setup_device(dev, &ds) != cudaSuccess) return HACC_ECUDA;
-    carve_noalloc(ds->base, n, g.ncell, &P, &Ps, &counter, &flags, &b);
+    carve_noalloc(ds->base, n, g.ncell, &P, &Ps, &flags, &b);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // the flags word keeps the previous call's value: start it at zero
     if (cudaMemsetAsync(flags, 0, 4 * sizeof(int), s) != cudaSuccess) return HACC_ECUDA;
     const float4 *src = reinterpret_cast<const float4 *>(pos_m);
-    if (bin_build(g, n, src, nullptr, 0.0f, P, b, flags, true, s) != cudaSuccess) return HACC_ECUDA;
+    if (bin_build(g, n, src, nullptr, 0.0f, P, b, flags, true, s, 0, kDefaultSplitMax, nullptr, false,
+                  Gather{P, Ps}) != cudaSuccess)
+        return HACC_ECUDA;
     if (n == 0) return HACC_OK;
-    if (gather_sorted(n, b.perm, P, Ps, nullptr, nullptr, nullptr, nullptr, s) != cudaSuccess) return HACC_ECUDA;
     ForceLaunch fl;
     fl.pos = Ps;
     fl.items = b.items;
     fl.n_items = b.n_items;
     fl.cell_start = b.cell_start;
-    fl.work_counter = counter;
+    fl.work_counter = b.work_counter;
+    fl.counter_clear = true;
     fl.mode = kModeForce;
     fl.out = reinterpret_cast<float4 *>(acc);
     fl.perm = b.perm;

@@ -962,8 +962,10 @@ cudaError_t launch_shared(const KParams &P, bool eps0, bool count, int num_sms, 
 cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const ForceLaunch &fl, int num_sms,
                             cudaStream_t s) {
     const bool pot = fl.mode == kModePotential;
-    cudaError_t e = cudaMemsetAsync(fl.work_counter, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
+    if (!fl.counter_clear) {
+        const cudaError_t e = cudaMemsetAsync(fl.work_counter, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
     KParams P;
     P.pos = fl.pos;
     P.items = fl.items;
