@@ -835,6 +835,7 @@ namespace {
 struct MlEvent {
     double t;
     KickTable kt;
+    Sharing sharing = kWhole;   // of its work items
 };
 
 // Events (2k+1)/(2l) dt, k < l, over the kick counts l that occur, in time
@@ -891,7 +892,7 @@ struct MlLoop {
     float half_lim;
 };
 
-ForceLaunch ml_force(hacc_ctx *ctx, Work &w, const MlLoop &m, const KickTable &kt) {
+ForceLaunch ml_force(hacc_ctx *ctx, Work &w, const MlLoop &m, const MlEvent &e) {
     ForceLaunch fl;
     fl.pos = m.Ps;
     fl.items = w.ml_items;
@@ -913,7 +914,8 @@ ForceLaunch ml_force(hacc_ctx *ctx, Work &w, const MlLoop &m, const KickTable &k
     fl.ids = nullptr;
     fl.vel_pool = nullptr;
     fl.levels = m.lev_s;
-    fl.kick = kt;
+    fl.kick = e.kt;
+    fl.sharing = e.sharing;
     fl.flags = ctx->d_flags;
     return fl;
 }
@@ -984,7 +986,7 @@ cudaError_t ml_capture(hacc_ctx *ctx, const Geometry &g, const ForceConsts &fc, 
         if ((e = items_kicked(g.ncell, w.b, m.lev_s, ev[k].kt, caps[k], w.ml_items, (int32_t)(m.n + 1),
                               ctx->d_flags, cs)) != cudaSuccess)
             break;
-        if ((e = sr_force_launch(g, fc, ml_force(ctx, w, m, ev[k].kt), ctx->num_sms, cs)) != cudaSuccess) break;
+        if ((e = sr_force_launch(g, fc, ml_force(ctx, w, m, ev[k]), ctx->num_sms, cs)) != cudaSuccess) break;
         ctx->force_launches++;
     }
     if (e == cudaSuccess) e = stream_sorted(m.n, m.Ps, m.Vs, (float)(dt - t_prev), nullptr, nullptr, cs);
@@ -1071,7 +1073,7 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
     int present[kMaxLevels + 1];
     HACC_CUDA(cudaMemcpyAsync(present, w.present, sizeof present, cudaMemcpyDeviceToHost, s), "levels present");
     HACC_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-    const std::vector<MlEvent> ev = ml_schedule(present, lmax, dt);
+    std::vector<MlEvent> ev = ml_schedule(present, lmax, dt);
     const float half_lim = (float)(half * (1.0 - 1e-5));
     // particles kicked at each event; a small launch splits its cells into
     // smaller items (down to one lane per particle) so that enough warps share it
@@ -1083,6 +1085,10 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
         const int64_t per_item = kicked / ((int64_t)ctx->num_sms * 64);
         caps[k] = (int)std::max<int64_t>(kCluster, std::min<int64_t>(kItemMax, per_item / kCluster * kCluster));
         if (icap) caps[k] = std::min(caps[k], icap);
+        if (ctx->item_cap < 0 && ctx->split_max == kDefaultSplitMax && shared_items(kicked)) {
+            ev[k].sharing = kByBlock;
+            caps[k] = auto_item_cap(kicked);
+        }
     }
 
     // Without timing or counting the event loop runs as one cached CUDA graph
@@ -1101,6 +1107,7 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
             key = mixk(key, tb);
             for (int l = 0; l <= kMaxLevels; ++l) key = mixk(key, fbits(ev[k].kt.h[l]));
             key = mixk(key, (uint64_t)caps[k]);
+            key = mixk(key, (uint64_t)ev[k].sharing);
         }
         key = mixk(key, (uint64_t)ctx->item_cap);
         key = mixk(key, (uint64_t)ctx->split_max);
@@ -1156,7 +1163,7 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
         HACC_CUDA(items_kicked(g.ncell, w.b, lev_s, e.kt, caps[k], w.ml_items, (int32_t)(n + 1), ctx->d_flags, s),
                   "work items");
         const MlLoop m{n, Ps, Vs, Vt, Ref, pos_in, V, lev_s, lev_t, id_s, id_t, disp_bits, half_lim};
-        HACC_TRY(launch_force(ctx, g, fc, ml_force(ctx, w, m, e.kt), true, s));
+        HACC_TRY(launch_force(ctx, g, fc, ml_force(ctx, w, m, e), true, s));
     }
     // last stream, then wrapped positions and velocities back to input order
     HACC_CUDA(stream_sorted(n, Ps, Vs, (float)(dt - t_prev), nullptr, nullptr, s), "closing stream");

@@ -1194,21 +1194,29 @@ __global__ void __launch_bounds__(kBlock) k_ci_to_f64(int64_t n, const int32_t *
 __global__ void __launch_bounds__(kBlock) k_levels(int64_t n, int64_t ncell, const int32_t *__restrict__ key,
                                                     const uint32_t *__restrict__ count, int d, int lmin, int lmax,
                                                     int32_t *__restrict__ level, int *__restrict__ present) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int l = 0;   // 0: no particle on this lane
-    if (i < n) {
-        int64_t q = lmax;
-        if (d > 0) {
-            const int64_t ratio = (int64_t)count[key[i]] * ncell / n;
-            q = ratio / d + 1;
-            if (q > lmax) q = lmax;
+    __shared__ int here[kMaxLevels + 1];
+    if (threadIdx.x <= kMaxLevels) here[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * kBlock;
+    for (int64_t at = (int64_t)blockIdx.x * kBlock; at < n; at += step) {
+        const int64_t i = at + threadIdx.x;
+        int l = 0;   // 0: no particle on this lane
+        if (i < n) {
+            int64_t q = lmax;
+            if (d > 0) {
+                const int64_t ratio = (int64_t)count[key[i]] * ncell / n;
+                q = ratio / d + 1;
+                if (q > lmax) q = lmax;
+            }
+            l = (int)(q < lmin ? lmin : q);
+            level[i] = l;
         }
-        l = (int)(q < lmin ? lmin : q);
-        level[i] = l;
+        // particles per kick count: one addition per distinct count in the warp
+        const unsigned peers = __match_any_sync(0xffffffffu, l);
+        if (l > 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&here[l], __popc(peers));
     }
-    // particles per kick count, one atomic per distinct count in the warp
-    const unsigned peers = __match_any_sync(0xffffffffu, l);
-    if (l > 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&present[l], __popc(peers));
+    __syncthreads();
+    if (threadIdx.x <= kMaxLevels && here[threadIdx.x]) atomicAdd(&present[threadIdx.x], here[threadIdx.x]);
 }
 
 // Stream sorted positions in place, without wrapping (inside one multi-level
@@ -1233,8 +1241,17 @@ __global__ void __launch_bounds__(kBlock) k_stream(int64_t n, float4 *__restrict
         }
     }
     if (!p0) return;
+    // the block's largest, and an atomic only where it exceeds what is there (one
+    // per warp took 41 of the 54 us that 2 million particles took)
+    __shared__ float largest[kBlock / 32];
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(disp, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) largest[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kBlock / 32; ++w) m = fmaxf(m, largest[w]);
+        const unsigned bits = __float_as_uint(m);
+        if (m > 0.0f && bits > *(volatile unsigned *)disp) atomicMax(disp, bits);
+    }
 }
 
 __global__ void k_ml_decide(const unsigned *disp_bits, float half_lim, cudaGraphConditionalHandle handle,
@@ -1272,6 +1289,7 @@ __global__ void __launch_bounds__(kBlock) k_ml_commit(int64_t n, const float4 *_
 // finds the runs in the ballot of kicked lanes, and cuts each run into
 // ceil(run / cap) items of near-equal size.  Items are appended through
 // n_items (their order only changes which warp takes which item, not any sum).
+// Bit l of `kicked` is set when particles with l kicks are kicked now.
 __device__ __forceinline__ void emit_run(int64_t c, int32_t lo, int32_t hi, uint32_t cap, int lane, int4 *items,
                                          int32_t *n_items, int32_t max_items, int *flags) {
     const uint32_t cnt = (uint32_t)(hi - lo);
@@ -1291,7 +1309,7 @@ __device__ __forceinline__ void emit_run(int64_t c, int32_t lo, int32_t hi, uint
 }
 
 __global__ void __launch_bounds__(kBlock) k_items_kicked(int64_t ncell, const int32_t *__restrict__ cell_start,
-                                                          const int32_t *__restrict__ level, KickTable kt,
+                                                          const int32_t *__restrict__ level, uint32_t kicked,
                                                           uint32_t cap, int4 *__restrict__ items,
                                                           int32_t *__restrict__ n_items, int32_t max_items,
                                                           int *flags) {
@@ -1302,7 +1320,7 @@ __global__ void __launch_bounds__(kBlock) k_items_kicked(int64_t ncell, const in
     int32_t open = -1;   // start of the run in progress
     for (int32_t base = a; base < b; base += 32) {
         const int32_t q = base + lane;
-        const unsigned m = __ballot_sync(0xffffffffu, q < b && kt.h[level[q]] != 0.0f);
+        const unsigned m = __ballot_sync(0xffffffffu, q < b && ((kicked >> level[q]) & 1u));
         const int len = min(32, b - base);
         int pos = 0;
         while (pos < len) {
@@ -1507,7 +1525,9 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
 cudaError_t ml_levels(const Geometry &g, int64_t n, const BinBuffers &b, int d, int lmin, int lmax, int32_t *level,
                       int *present, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_levels<<<blocks_for(n), kBlock, 0, s>>>(n, g.ncell, b.key, b.count, d, lmin, lmax, level, present);
+    // few blocks: each adds to the same few words at its end (with every warp
+    // adding to them, 45 us of atomics on 2 million particles)
+    k_levels<<<std::min(blocks_for(n), 1024u), kBlock, 0, s>>>(n, g.ncell, b.key, b.count, d, lmin, lmax, level, present);
     note_launch();
     return cudaGetLastError();
 }
@@ -1542,7 +1562,9 @@ cudaError_t items_kicked(int64_t ncell, const BinBuffers &b, const int32_t *leve
     if (cap < kCluster || cap > kItemMax) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(b.n_items, 0, sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
-    k_items_kicked<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.cell_start, level, kt, (uint32_t)cap, items,
+    uint32_t kicked = 0;
+    for (int l = 0; l <= kMaxLevels; ++l) kicked |= kt.h[l] != 0.0f ? 1u << l : 0u;
+    k_items_kicked<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.cell_start, level, kicked, (uint32_t)cap, items,
                                                              b.n_items, max_items, d_flags);
     note_launch();
     return cudaGetLastError();
