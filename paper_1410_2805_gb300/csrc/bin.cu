@@ -394,7 +394,7 @@ __device__ __forceinline__ void gather_row(const Gather &g, int64_t k, int32_t i
 // The arrival order from the atomics is arbitrary, so each element's final
 // slot is the number of smaller keys in its cell.  The key is the input row
 // (distinct), which gives ascending input row within the cell, or the pair
-// (Morton sub-cell, input row), which groups the cell's particles by sub-cell.
+// (sub-cell code, input row), which groups the cell's particles by sub-cell.
 // k_order_rows serves calls of up to 2^24 rows (the pair as one 32-bit key,
 // code << 24 | row); k_order_sub, one warp per cell, larger ones: a cell that
 // becomes one work item by row, the others by the pair with the row taken

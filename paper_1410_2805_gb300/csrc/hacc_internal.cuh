@@ -244,7 +244,7 @@ struct BinBuffers {
     int32_t *big_list;     // cells too large for the warp-level ordering
     int *big_count;
     int *work_counter;     // [1] device: cleared by each binning (the force launch that follows it)
-    uint8_t *sub;                  // [n] Morton sub-cell of each input row (item_cap > 0), or null
+    uint8_t *sub;                  // [n] sub-cell code of each input row (item_cap > 0), or null
     unsigned long long *order_tmp; // [n] (sub-cell << 32 | row) in the slots of perm_tmp, or null
 };
 
