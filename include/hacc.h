@@ -471,8 +471,10 @@ hacc_status hacc_set_stencil(hacc_ctx *ctx, int32_t cells_per_rcut);
  * cap = 0: input row order within cells, items of up to 64 particles, and
  * neighbours skipped by the item's bounds alone.
  * cap = -1 (default): by the box's size, 8 particles up to 2^13, 16 up to
- * 2^16, 32 up to 2^20, 64 above (small boxes have few items to spread over the
- * chip); a box of a batch follows its own size.  The cell/offset paths use 64,
+ * 3*2^12, 32 up to 2^20, 64 above (small boxes have few items to spread over the
+ * chip), and up to 2^16 particles the neighbours of an item are summed in four
+ * parts, by the four warps of a block; a box of a batch follows its own size, its
+ * parts one after the other.  The cell/offset paths use 64,
  * hacc_sr_force_noalloc row order with items of 64 skipped per cluster.
  * Forces differ between settings only by the order of FP32 sums.  Errors: cap
  * outside {-1, 0} and [16, 160] or split_max < 0. */
