@@ -777,11 +777,12 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
     __shared__ uint32_t cstart[kOrdCells], ccount[kOrdCells];
     __shared__ int next_cell;   // the warps take the block's cells in turn (cells differ widely in cost)
     __shared__ int wide[kOrdCells], n_wide;   // cells for the whole block
-    __shared__ int n_later;                   // set: cells for k_order_big
+    __shared__ unsigned later[kOrdCells / 32];   // a bit per cell: listed for k_order_big
     const int64_t c0 = (int64_t)blockIdx.x * cells;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int ncb = ncell - c0 < cells ? (int)(ncell - c0) : cells;   // cells of this block (>= 1)
-    if (t == 0) next_cell = n_wide = n_later = 0;
+    if (t == 0) next_cell = n_wide = 0;
+    if (t < kOrdCells / 32) later[t] = 0u;
     if (t < kOrdCells) {
         uint32_t cnt = 0, st = 0;
         if (t < ncb) {
@@ -851,7 +852,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
                 for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
             if (lane == 0 && !big_here) {
                 big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
-                n_later = 1;
+                atomicOr(&later[q >> 5], 1u << (q & 31));
             }
             if (!big_here) continue;
         }
@@ -930,12 +931,16 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
     }
     if (!gather.p_out) return;
     __syncthreads();
-    const bool some_later = n_later;   // cells that k_order_big orders and gathers
+    // k_order_big gathers the cells that it orders: those listed above, and not
+    // every cell as large as they are (the ranking by stretches orders some here)
     for (uint32_t e = S0 + t; e < S1; e += kBlock) {
-        bool later = false;
-        if (some_later)
-            for (int q = 0; q < ncb; ++q) later |= ccount[q] > kBlockCell && e - cstart[q] < ccount[q];
-        if (!later) gather_row(gather, e, perm[e]);
+        bool here = true;
+        for (int h = 0; h < kOrdCells / 32; ++h)
+            for (unsigned m = later[h]; m; m &= m - 1u) {
+                const int q = 32 * h + __ffs(m) - 1;
+                here &= e - cstart[q] >= ccount[q];
+            }
+        if (here) gather_row(gather, e, perm[e]);
     }
 }
 
