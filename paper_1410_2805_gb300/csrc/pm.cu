@@ -334,19 +334,24 @@ hacc_status pm_accel(hacc_ctx *ctx, const hacc_box *box, const hacc_pm *pm, doub
                                                                    (float)(scale - (double)(float)scale), st->rho);
     note_launch();
     // the tables depend on the box side alone: kept until it changes (8 us of FP64
-    // a call), but not on the word of a launch that is only being captured
+    // a call).  A captured call makes its own at every replay, in the field grid
+    // (free until the transforms below), so that no replay changes the kept ones.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return check_cuda(ctx, e, "cudaStreamIsCapturing");
-    if (st->tab_L != L || cap != cudaStreamCaptureStatusNone) {
-        k_tables<<<(ng + 127) / 128, 128, 0, s>>>(ng, L, st->tab);
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    float *tab = captured ? reinterpret_cast<float *>(st->field) : st->tab;
+    if (captured || st->tab_L != L) {
+        if (!captured) st->tab_L = 0.0;
+        k_tables<<<(ng + 127) / 128, 128, 0, s>>>(ng, L, tab);
         note_launch();
-        st->tab_L = cap == cudaStreamCaptureStatusNone ? L : 0.0;
+        if ((e = cudaGetLastError()) != cudaSuccess) return check_cuda(ctx, e, "PM tables");
+        if (!captured) st->tab_L = L;
     }
     if (cufftSetStream(st->r2c, s) != CUFFT_SUCCESS || cufftSetStream(st->c2r, s) != CUFFT_SUCCESS)
         return set_error(ctx, HACC_ECUDA, "cufftSetStream failed");
     if (cufftExecR2C(st->r2c, st->rho, st->rk) != CUFFT_SUCCESS) return set_error(ctx, HACC_ECUDA, "cufftExecR2C failed");
     const float pref = (float)(4.0 * 3.14159265358979323846 * G / (double)ng3);
-    k_kspace<<<blocks_for(nm), kBlock, 0, s>>>(ng, (float)D, pm->sigma, pm->ns, pref, st->tab, st->rk, st->ak);
+    k_kspace<<<blocks_for(nm), kBlock, 0, s>>>(ng, (float)D, pm->sigma, pm->ns, pref, tab, st->rk, st->ak);
     note_launch();
     // the components back to real space into the arrays free at this point (the
     // fixed-point mass grid and the density behind it), then interleaved into the
