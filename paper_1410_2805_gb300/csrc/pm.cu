@@ -86,14 +86,17 @@ __global__ void __launch_bounds__(kBlock) k_deposit(int64_t n, const float4 *__r
             }
 }
 
-// rho = mass * scale from the fixed-point mass, scale = sh + sl.  The product
-// is formed from the mass's leading 24 bits and the rest, both exact in FP32, so
-// that it is rounded once and to within 2^-20 of an ulp as an FP64 product would
-// be.  FP64 and the 64-bit conversions run at a fraction of the FP32 rate here:
-// they took three times as long as the 12 bytes per grid point (128^3: 12.4 ->
-// 7 us).
+// rho = mass * scale from the fixed-point mass, scale = (sh + sl) e1 e2 with
+// sh + sl in [1/2, 1) and e1, e2 powers of two.  The product of sh + sl is formed
+// from the mass's leading 24 bits and the next 24, all exact in FP32, so that it
+// is rounded once and to within 2^-20 of an ulp as an FP64 product would be; the
+// powers of two then change no bit of a rho that is a normal FP32 value, at any
+// grid spacing.  FP64 and the 64-bit conversions run at a fraction of the FP32
+// rate here: they took three times as long as the 12 bytes per grid point
+// (128^3: 12.4 -> 7 us).
 __global__ void __launch_bounds__(kBlock) k_fix_to_density(int64_t ng3, const unsigned long long *__restrict__ acc,
-                                                            float sh, float sl, float *__restrict__ rho) {
+                                                            float sh, float sl, float e1, float e2,
+                                                            float *__restrict__ rho) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng3) return;
     const long long a = (long long)acc[g];
@@ -104,7 +107,7 @@ __global__ void __launch_bounds__(kBlock) k_fix_to_density(int64_t ng3, const un
     const float sign = a < 0 ? -1.0f : 1.0f;
     const float hi = sign * (float)top * __int_as_float((127 + cut) << 23);
     const float lo = sign * (float)rest * __int_as_float((127 + cut2) << 23);
-    rho[g] = __fmaf_rn(hi, sh, __fmaf_rn(lo, sh, hi * sl));
+    rho[g] = __fmaf_rn(hi, sh, __fmaf_rn(lo, sh, hi * sl)) * e1 * e2;
 }
 
 // Per-axis tables in FP64 (rounded to FP32 once): mode number k of index q is
@@ -329,9 +332,14 @@ hacc_status pm_accel(hacc_ctx *ctx, const hacc_box *box, const hacc_pm *pm, doub
             if ((e = cudaEventRecord(io->ev[c], io->copy)) != cudaSuccess) return check_cuda(ctx, e, "cudaEventRecord");
         }
     }
-    const double scale = 1.0 / (kFix * D * D * D);
-    k_fix_to_density<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, st->mass, (float)scale,
-                                                                   (float)(scale - (double)(float)scale), st->rho);
+    // 1 / (2^32 D^3) as a fraction and a power of two in two factors (past 2^+-252 the
+    // density is beyond FP32 for every mass)
+    int exponent = 0;
+    const double frac = std::frexp(1.0 / (kFix * D * D * D), &exponent);
+    exponent = std::max(-252, std::min(252, exponent));
+    k_fix_to_density<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>(
+        (int64_t)ng3, st->mass, (float)frac, (float)(frac - (double)(float)frac), std::ldexp(1.0f, exponent / 2),
+        std::ldexp(1.0f, exponent - exponent / 2), st->rho);
     note_launch();
     // the tables depend on the box side alone: kept until it changes (8 us of FP64
     // a call).  A captured call makes its own at every replay, in the field grid

@@ -53,3 +53,24 @@ def test_replays_of_another_side_leave_a_call_alone(env):
         ref = opm.pm_accel(pos[k][0][:, :3].astype(np.float64), pos[k][0][:, 3].astype(np.float64), L, ng)
         rms = np.sqrt((ref ** 2).sum(1).mean())
         assert np.abs(alone[k].cpu().numpy()[:, :3] - ref).max() / rms <= 1e-4
+
+
+@pytest.mark.parametrize("exponent", [-30, 31, 36, 38])
+def test_force_scales_with_the_unit_of_length(env, exponent):
+    # the same box in units 2^-exponent as long (grid spacings of 8e-10 to 2e11): the acceleration is
+    # m / length^2, and every step of the solve scales by a power of two.  Densities below 2^-126, which a
+    # transform may take for zero, are at most 2^-12 of the mean at the largest spacing: the bar of every force
+    # comparison covers them.
+    torch, hacc = env
+    ng, L = 24, 20.0
+    _, p = _box(torch, 4000, L, 7)
+    q = p.clone()
+    q[:, :3] *= 2.0 ** exponent
+    ctx = hacc.Context()
+    try:
+        a = ctx.pm_force(hacc.Box(L=L, ng=ng), hacc.PM(), p).double()
+        b = ctx.pm_force(hacc.Box(L=L * 2.0 ** exponent, ng=ng), hacc.PM(), q).double() * 4.0 ** exponent
+    finally:
+        ctx.close()
+    rms = (a ** 2).sum(1).mean().sqrt()
+    assert float((b - a).abs().max() / rms) <= 1e-4
