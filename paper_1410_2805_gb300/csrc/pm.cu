@@ -7,7 +7,7 @@
 //   k_kspace    phi(k) = 4 pi G G6(k) S(k) rho(k) / ng^3 (Eq. (greenf),
 //               Eq. (filter)) and a_c(k) = -i D_c(k) phi(k), the fourth-order
 //               Super-Lanczos derivative of Eq. (sldiff), for c = x, y, z
-//   cuFFT C2R   the three components, one batched plan
+//   cuFFT C2R   the three components, in one plan on grids of up to 256^3 points
 //   k_interp    CIC interpolation of (a_x, a_y, a_z) at the particles, then
 //               either a store or a kick v += kick * a
 //
@@ -30,10 +30,12 @@ namespace hacc {
 namespace {
 
 constexpr int kBlock = 256;
+constexpr int kBatchedMax = 256;   // grid points per side up to which the inverse transforms are one plan
 
 struct PmState {
     int ng = 0;
     cufftHandle r2c = 0, c2r = 0;
+    int c2r_batch = 3;           // transforms that one execution of c2r does: 3 or 1
     bool have_plans = false;
     unsigned long long *mass = nullptr;  // ng^3 fixed-point mass per grid point, then rho: together
                                          // the three force components in real space, 3 x ng^3 floats
@@ -251,12 +253,24 @@ hacc_status get_state(hacc_ctx *ctx, int ng, double L, cudaStream_t s, PmState *
             free_state(st);
             return set_error(ctx, HACC_ECUDA, "cufftPlan3d R2C failed");
         }
-        // the three components in one plan: a third of the launches
+        // The three components in one plan up to kBatchedMax: fewer launches (us of
+        // the three transforms one by one and as a batch, ng 64: 50 and 20, 128: 67 and
+        // 42, 256: 266 and 253, 384: 1389 and 1402, 640: 6557 and 6785).  Larger grids
+        // take them one by one: nothing to gain, and a batch's work area is three
+        // times as large (sides with large prime factors) and its elements pass 2^32.
         int dims[3] = {ng, ng, ng};
-        if (cufftPlanMany(&st->c2r, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3) != CUFFT_SUCCESS) {
-            cufftDestroy(st->r2c);
-            free_state(st);
-            return set_error(ctx, HACC_ECUDA, "cufftPlan3d C2R failed");
+        st->c2r_batch = ng <= kBatchedMax ? 3 : 1;
+        if (st->c2r_batch == 3 &&
+            cufftPlanMany(&st->c2r, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3) != CUFFT_SUCCESS) {
+            cudaGetLastError();   // no room for its work area, say
+            st->c2r_batch = 1;
+        }
+        if (st->c2r_batch == 1) {
+            if (cufftPlan3d(&st->c2r, ng, ng, ng, CUFFT_C2R) != CUFFT_SUCCESS) {
+                cufftDestroy(st->r2c);
+                free_state(st);
+                return set_error(ctx, HACC_ECUDA, "cufftPlan3d C2R failed");
+            }
         }
         st->have_plans = true;
         st->ng = ng;
@@ -365,7 +379,9 @@ hacc_status pm_accel(hacc_ctx *ctx, const hacc_box *box, const hacc_pm *pm, doub
     // fixed-point mass grid and the density behind it), then interleaved into the
     // field grid in one pass
     float *comp = reinterpret_cast<float *>(st->mass);
-    if (cufftExecC2R(st->c2r, st->ak, comp) != CUFFT_SUCCESS) return set_error(ctx, HACC_ECUDA, "cufftExecC2R failed");
+    for (int c = 0; c < 3; c += st->c2r_batch)
+        if (cufftExecC2R(st->c2r, st->ak + c * nm, comp + c * ng3) != CUFFT_SUCCESS)
+            return set_error(ctx, HACC_ECUDA, "cufftExecC2R failed");
     k_pack_components<<<blocks_for((int64_t)ng3), kBlock, 0, s>>>((int64_t)ng3, comp, comp + ng3, comp + 2 * ng3,
                                                                     st->field);
     note_launch();

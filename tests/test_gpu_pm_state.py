@@ -74,3 +74,40 @@ def test_force_scales_with_the_unit_of_length(env, exponent):
         ctx.close()
     rms = (a ** 2).sum(1).mean().sqrt()
     assert float((b - a).abs().max() / rms) <= 1e-4
+
+
+@pytest.mark.parametrize("ng", [256, 258])
+def test_grids_at_the_bound_of_the_batched_transforms(env, ng):
+    torch, hacc = env
+    L = 64.0
+    pos, p = _box(torch, 3000, L, ng)
+    ctx = hacc.Context()
+    try:
+        a = ctx.pm_force(hacc.Box(L=L, ng=ng), hacc.PM(), p).cpu().numpy()
+    finally:
+        ctx.close()
+    ref = opm.pm_accel(pos[:, :3].astype(np.float64), pos[:, 3].astype(np.float64), L, ng)
+    rms = np.sqrt((ref ** 2).sum(1).mean())
+    assert np.abs(a[:, :3] - ref).max() / rms <= 1e-4
+
+
+def test_large_grids_keep_the_work_area_of_one_transform(env):
+    # 514 = 2 x 257: transforms of such sides need a work area, about their own data each.  What the context
+    # holds is its grids (28 bytes a point and 32 a mode) and at most one transform's data for either direction,
+    # with a quarter to spare; three components at once would take half as much again as that in the inverse alone
+    torch, hacc = env
+    ng, L = 514, 128.0
+    _, p = _box(torch, 3000, L, 5)
+    mode_bytes = 8 * ng * ng * (ng // 2 + 1)
+    ctx = hacc.Context()
+    try:
+        ctx.pm_force(hacc.Box(L=L, ng=16), hacc.PM(), p)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        ctx.pm_force(hacc.Box(L=L, ng=ng), hacc.PM(), p, acc=torch.empty_like(p))
+        torch.cuda.synchronize()
+        held = free - torch.cuda.mem_get_info()[0]
+    finally:
+        ctx.close()
+    assert held <= 28 * ng ** 3 + 4 * mode_bytes + 2.5 * mode_bytes
