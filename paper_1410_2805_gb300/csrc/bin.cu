@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(kBlock) k_order_sub(int64_t ncell, const uint3
 // merge-path co-rank.  O(m log^2 m) work per cell of m particles.  The rows come
 // in A and end in B; sh holds kChunk values.  All threads of the block call it.
 constexpr int kChunk = 2048;
-__device__ __noinline__ void order_big_cell(int32_t *A, int32_t *B, int m, int32_t *sh, int tid, int threads) {
+__device__ void order_big_cell(int32_t *A, int32_t *B, int m, int32_t *sh, int tid, int threads) {
     // 1. sorted chunks, in place in A
     for (int base = 0; base < m; base += kChunk) {
         for (int t = tid; t < kChunk; t += threads) sh[t] = base + t < m ? A[base + t] : 0x7fffffff;
@@ -671,8 +671,10 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
 // row (codes below 2^8, rows below 2^24; larger calls take k_order_sub).  Cells
 // above kBigCell are ordered by input row alone; those above kBlockCell by
 // k_order_big (with SUB their rows are copied to perm_tmp first), or, in calls
-// of up to kBigHereMax particles, by their block at the end: the launch costs
-// such a call more than its thousand threads save on a cell that it rarely has.
+// of up to kBigHereMax particles, by their block at the end, from a map of the
+// call's rows in shared memory (hacc_bin of 65536 particles in one cell 111 us,
+// in four 104; by merge sort in k_order_big's thousand threads 966 and 274, in
+// the block's own 2438 and 2039).
 constexpr uint32_t kBlockCell = 2048;
 constexpr int64_t kBigHereMax = (int64_t)1 << 16;
 // Calls of up to this many particles gather in the ordering's blocks: a launch
@@ -847,14 +849,16 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
             rank_stretches(seg, cnt, lane, out, row_mask, heads[w][0], heads[w][1], heads[w][2]))
             continue;
         if (cnt > kBlockCell) {
-            // to the big-cell sort by row, from perm_tmp
-            if (SUB)
-                for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
-            if (lane == 0 && !big_here) {
-                big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
-                atomicOr(&later[q >> 5], 1u << (q & 31));
+            if (!big_here) {
+                // to the big-cell sort by row, from perm_tmp
+                if (SUB)
+                    for (uint32_t e = lane; e < cnt; e += 32) perm_tmp[st + e] = (int32_t)(uint32_t)order_tmp[st + e];
+                if (lane == 0) {
+                    big_list[atomicAdd(big_count, 1)] = (int32_t)(c0 + q);
+                    atomicOr(&later[q >> 5], 1u << (q & 31));
+                }
+                continue;
             }
-            if (!big_here) continue;
         }
         if (cnt > 256) {
             if (lane == 0) wide[atomicAdd(&n_wide, 1)] = q;
@@ -922,11 +926,28 @@ __global__ void __launch_bounds__(kBlock, 5) k_order_rows(int64_t ncell, const u
         __syncthreads();   // slots and first are free
     }
     if (big_here && S1 - S0 > kBlockCell) {
-        __syncthreads();   // the stage is free
+        // big cells by row: the rows, distinct and below kBigHereMax, as the bits of
+        // a map; a row's slot is the number of bits before its own
+        constexpr int kWords = (int)(kBigHereMax / 32), kPer = kWords / kBlock;   // words of a thread: kPer in turn
+        static_assert(kWords <= kOrdCap && kWords % kBlock == 0, "the map takes the stage's place");
         for (int k = 0; k < nw; ++k) {
             const uint32_t cnt = ccount[wide[k]], st = cstart[wide[k]];
-            if (cnt > kBlockCell)
-                order_big_cell(perm_tmp + st, perm + st, (int)cnt, reinterpret_cast<int32_t *>(keys), t, kBlock);
+            if (cnt <= kBlockCell) continue;
+            __syncthreads();   // the stage, or the map before, is free
+            for (int x = t; x < kWords; x += kBlock) keys[x] = 0u;
+            __syncthreads();
+            for (uint32_t e = t; e < cnt; e += kBlock) {
+                const uint32_t r = order_key<SUB>(perm_tmp, order_tmp, st + e) & row_mask;
+                atomicOr(&keys[r >> 5], 1u << (r & 31));
+            }
+            __syncthreads();
+            uint32_t bits = 0;
+#pragma unroll
+            for (int x = 0; x < kPer; ++x) bits += __popc(keys[kPer * t + x]);
+            int32_t *out = perm + st + (uint32_t)block_exclusive(bits, nullptr);
+#pragma unroll
+            for (int x = 0; x < kPer; ++x)
+                for (uint32_t m = keys[kPer * t + x]; m; m &= m - 1u) *out++ = 32 * (kPer * t + x) + __ffs(m) - 1;
         }
     }
     if (!gather.p_out) return;

@@ -31,9 +31,10 @@ def halo_box(counts, n, seed):
 
 
 # (a cell of up to about 4000 particles, one that a ranking by runs of rows cannot take): neighbours in x, far
-# apart in one block of cells, and in the other order; just above the calls whose blocks sort every cell themselves
+# apart in one block of cells, and in the other order; on both sides of the largest call whose blocks sort every cell
 @pytest.mark.parametrize("counts,n", [({0: 3000, 1: 20000}, 100001), ({0: 12000, 7: 2049, 3: 2048}, 65537),
-                                      ({8: 2300, 9: 9000, 10: 2300}, 80000)])
+                                      ({8: 2300, 9: 9000, 10: 2300}, 80000),
+                                      ({0: 2049, 1: 12000, 2: 2048, 3: 2500}, 65536)])
 @pytest.mark.parametrize("call", ["subcycle", "step"])
 def test_neighbouring_dense_cells_keep_their_rows(split_params, counts, n, call):
     import torch
@@ -65,3 +66,29 @@ def test_neighbouring_dense_cells_keep_their_rows(split_params, counts, n, call)
     d -= L * np.round(d / L)
     assert np.abs(d).max() < 2e-5 * L
     assert np.abs(v[:, :3] - vo).max() < 1e-3 * np.sqrt((vo ** 2).sum(1).mean())
+
+
+# cells above the 2048 keys that a block ranks by buckets: all of a call's particles in one cell, several such cells
+# in one block of cells, with smaller ones between them; input in random order and in cell order
+@pytest.mark.parametrize("counts,n", [({0: 65536}, 65536), ({0: 65537}, 65537), ({5: 2049}, 2049),
+                                      ({0: 2049, 1: 2048, 2: 30000, 3: 1, 4: 2050, NC ** 3 - 1: 9000}, 50000)])
+@pytest.mark.parametrize("ordered", [False, True])
+def test_big_cells_are_ordered_by_row(split_params, counts, n, ordered):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1410_2805_gb300 as hacc
+    pos, _ = halo_box(counts, n, seed=n)
+    _, cell_o, ok = oracle.wrap_cell(pos, L, NC)
+    assert ok
+    if ordered:
+        order = np.argsort(cell_o, kind="stable")
+        pos, cell_o = pos[order], cell_o[order]
+    _, start_o, perm_o = oracle.bin_cells(cell_o, NC)
+    ctx = hacc.Context()
+    try:
+        p = torch.from_numpy(pos.copy()).cuda()
+        cell, start, perm = (t.cpu().numpy() for t in ctx.bin(hacc.Box(L=L, nc=NC), np.float32(split_params["r_cut"]), p))
+    finally:
+        ctx.close()
+    assert np.array_equal(cell, cell_o) and np.array_equal(start, start_o) and np.array_equal(perm, perm_o)
