@@ -300,8 +300,8 @@ hacc_status hacc_batch_subcycle(hacc_ctx *ctx, const hacc_split *split, int32_t 
                                 int32_t n_sub, int32_t use_graph, hacc_stream_t stream);
 
 /* Autotuner of the batched launch (a tuning aid of the library; the paper has
- * no counterpart).  For every setting of work-item cap in {0 (cell-wide
- * items), 32, 64, 96, 128, 160} (see hacc_set_item_cap) x queue order (cell order,
+ * no counterpart).  For every setting of work-item cap in HACC_BATCH_TUNE_CAPS
+ * (see hacc_set_item_cap; -1: each box's automatic cap) x queue order (cell order,
  * largest first; see hacc_set_queue_order) x pair-kernel variant, times whole
  * batched ticks as hacc_batch_tick runs them (binning, gathers, the kick and
  * stream pass; each box one sub-cycle of step boxes[b].dt) on scratch copies
@@ -315,6 +315,7 @@ hacc_status hacc_batch_subcycle(hacc_ctx *ctx, const hacc_split *split, int32_t 
  * *chosen (nullable) the setting kept.  The pools are only read (the scratch
  * grows by 32 bytes per pool row).  Synchronises `stream`.  Every setting sums
  * the same pairs. */
+#define HACC_BATCH_TUNE_CAPS {0, 32, 64, 16, 48, -1}
 #define HACC_BATCH_TUNE_SETTINGS 48
 hacc_status hacc_batch_tune(hacc_ctx *ctx, const hacc_split *split, int32_t nbox, const hacc_batch_box *boxes,
                             const float *pos_pool, const float *vel_pool, int32_t reps, double *times_ms,
@@ -425,8 +426,8 @@ hacc_status hacc_sr_force_noalloc(const hacc_box *box, const hacc_split *split, 
 #define HACC_FORCE_VARIANTS 4
 
 /* Autotuner (a tuning aid of the library; the paper has no counterpart):
- * for every setting of work-item cap in {0 (cell-wide items), 16, 24, 32, 48}
- * (see hacc_set_item_cap) x queue order (cell order, largest first; see
+ * for every setting of work-item cap in HACC_TUNE_CAPS (see hacc_set_item_cap;
+ * -1: the automatic cap) x queue order (cell order, largest first; see
  * hacc_set_queue_order) x pair-kernel variant, times one sub-cycle's work on
  * pos_m as hacc_subcycle runs it: the chaining-mesh build (binning, gather
  * into cell order) and the pair-kernel launch that kicks and streams (with
@@ -440,6 +441,7 @@ hacc_status hacc_sr_force_noalloc(const hacc_box *box, const hacc_split *split, 
  * kept.  Synchronises `stream`.  Every setting sums the same pairs (the
  * variants and orders in the same order; the caps in different orders, so
  * results differ by FP32 rounding). */
+#define HACC_TUNE_CAPS {0, 16, -1, 32, 64}
 #define HACC_TUNE_SETTINGS 40
 hacc_status hacc_tune(hacc_ctx *ctx, const hacc_box *box, const hacc_split *split, int64_t n,
                       const float *pos_m, int32_t reps, double *times_ms, int32_t *chosen,

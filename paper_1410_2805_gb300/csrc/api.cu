@@ -108,10 +108,11 @@ hacc_status make_ci_geometry(hacc_ctx *ctx, const hacc_box *box, float r_cut, Ge
     return HACC_OK;
 }
 
-// Item caps the single-box tuner tries (0: cell-wide items of up to kItemMax).
-const int kTuneCaps[] = {0, 16, 24, 32, 48};
-constexpr int kTuneCapCount = 5;
-constexpr int kTuneSettings = kTuneCapCount * 2 * kForceVariants;   // cap x queue order x variant
+// Item caps the single-box tuner tries: the automatic one, which alone shares the
+// items of small boxes, and the others that make a difference (all above
+// kItemMax mean kItemMax).
+const int kTuneCaps[] = HACC_TUNE_CAPS;
+constexpr int kTuneSettings = (int)(sizeof(kTuneCaps) / sizeof(kTuneCaps[0])) * 2 * kForceVariants;
 static_assert(kTuneSettings == HACC_TUNE_SETTINGS, "tuner table size");
 static_assert(sizeof(hacc_ctx::io_ev) / sizeof(void *) >= 3 + kPmChunks, "one event per PM chunk");
 
@@ -484,21 +485,20 @@ hacc_status hacc_tune(hacc_ctx *ctx, const hacc_box *box, const hacc_split *spli
     const float4 *src = reinterpret_cast<const float4 *>(pos_m);
     const float h = 1e-3f;
     // one sub-cycle's chaining-mesh build and pair-kernel launch (kick + stream)
-    auto subcycle_work = [&](int cap, bool first) -> hacc_status {
-        HACC_CUDA(bin_build(g, n, first ? src : w.P, nullptr, 0.0f, w.P, w.b, ctx->d_flags, true, s, cap,
-                            ctx->split_max, nullptr, !first, Gather{w.P, w.Ps, w.V, w.Vs, nullptr, w.IDs}),
+    auto subcycle_work = [&](bool first) -> hacc_status {
+        HACC_CUDA(bin_build(g, n, first ? src : w.P, nullptr, 0.0f, w.P, w.b, ctx->d_flags, true, s,
+                            item_cap_for(ctx, n), ctx->split_max, nullptr, !first, Gather{w.P, w.Ps, w.V, w.Vs, nullptr, w.IDs}),
                   "tuner binning");
         return run_sorted_force(ctx, g, fc, &w, kModeKickDrift, nullptr, nullptr, w.Vs, w.P, h, h, nullptr, s, n);
     };
     for (int k = 0; k < kTuneSettings && st == HACC_OK; ++k) {
-        const int cap = kTuneCaps[k / (2 * kForceVariants)];
+        ctx->item_cap = kTuneCaps[k / (2 * kForceVariants)];
         ctx->queue_order = (k / kForceVariants) % 2;
         ctx->variant = k % kForceVariants;
-        ctx->item_cap = cap;
-        st = subcycle_work(cap, true);   // warm-up, from pos_m
+        st = subcycle_work(true);   // warm-up, from pos_m
         if (st != HACC_OK) break;
         cudaEventRecord(e0, s);
-        for (int r = 0; r < reps && st == HACC_OK; ++r) st = subcycle_work(cap, false);
+        for (int r = 0; r < reps && st == HACC_OK; ++r) st = subcycle_work(false);
         cudaEventRecord(e1, s);
         cudaError_t e = cudaEventSynchronize(e1);
         if (e != cudaSuccess) {

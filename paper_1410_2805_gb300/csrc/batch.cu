@@ -267,9 +267,10 @@ extern "C" hacc_status hacc_batch_tick(hacc_ctx *ctx, const hacc_split *split, i
                     w, s);
 }
 
-// Item caps the batched tuner tries (0: cell-wide items of up to kItemMax);
-// setting k = (cap index * 2 + queue order) * kForceVariants + variant.
-static const int kTuneCaps[] = {0, 32, 64, 96, 128, 160};
+// Item caps the batched tuner tries (-1: each box's automatic one, with which a
+// box's sums are those of its own call); setting k = (cap index * 2 + queue
+// order) * kForceVariants + variant.
+static const int kTuneCaps[] = HACC_BATCH_TUNE_CAPS;
 static constexpr int kTuneSettings = (int)(sizeof(kTuneCaps) / sizeof(kTuneCaps[0])) * 2 * kForceVariants;
 static_assert(kTuneSettings == HACC_BATCH_TUNE_SETTINGS, "tuner table size");
 
