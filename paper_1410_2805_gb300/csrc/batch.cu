@@ -45,7 +45,7 @@ size_t carve_batch(char *base, int64_t n, int64_t ncell, int64_t table_entries, 
     w->IDs = c.take<int32_t>(n);
     w->counter = c.take<int>(1);
     w->tables = c.take<BoxDev>(table_entries);
-    carve_bin(c, n, ncell, &w->b);
+    carve_bin(c, n, ncell, &w->b, true, table_entries);
     return c.off + 256;
 }
 
@@ -176,6 +176,7 @@ hacc_status run_tick(hacc_ctx *ctx, const ForceConsts &fc, const Plan &pl, const
         fl.order = w.b.order;
     }
     fl.boxes = tab;
+    fl.nbox = pl.nbox;
     fl.ids = w.IDs;
     fl.pos_pool = pos_pool;
     fl.vel_pool = vel_pool;
@@ -457,6 +458,7 @@ extern "C" hacc_status hacc_batch_diagnostics(hacc_ctx *ctx, const hacc_split *s
     fl.mass_flag = w.b.mass_flag;
     fl.variant = ctx->variant;
     fl.boxes = w.tables;
+    fl.nbox = pl.nbox;
     fl.ids = w.IDs;
     fl.flags = ctx->d_flags;
     HACC_CUDA_RETURN(sr_force_launch(g0, fc, fl, ctx->num_sms, s), "batched pair potential");

@@ -240,10 +240,11 @@ struct BinBuffers {
     int32_t *order;        // [max_items] work-queue order of the items (heavy_first), or unused
     uint32_t *item_cls;    // [2 kItemClasses] per-class counts and cursors of heavy_first
     int32_t *n_items;      // [1] device
-    int *mass_flag;        // [1] device: nonzero if some mass differs from the first
+    uint32_t *mass_flag;   // device, a bit per box: some mass differs from the box's first
     int32_t *big_list;     // cells too large for the warp-level ordering
     int *big_count;
-    int *work_counter;     // [1] device: cleared by each binning (the force launch that follows it)
+    int *work_counter;     // [2] device: cleared by each binning (the force launch that follows it)
+    size_t zeroed;         // words from count on that a binning clears: count, the counters, mass_flag
     uint8_t *sub;                  // [n] sub-cell code of each input row (item_cap > 0), or null
     unsigned long long *order_tmp; // [n] (sub-cell << 32 | row) in the slots of perm_tmp, or null
 };
@@ -271,7 +272,7 @@ constexpr int64_t kHeavyFirstMinN = (int64_t)1 << 20;   // smaller calls keep th
 cudaError_t items_heavy_first(const BinBuffers &b, int64_t max_items, cudaStream_t s);
 int64_t max_items(int64_t n, int64_t ncell, bool sub_order = true);
 // sub_order = false leaves out the sub-cell arrays (item_cap must then be 0).
-void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_order = true);
+void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_order = true, int64_t nbox = 1);
 
 // Wrap (optionally after a drift x += d v) src into dst and compute keys,
 // counts, the permutation, cell starts and force work items.  vel may be
@@ -377,7 +378,7 @@ struct ForceLaunch {
     const int4 *items;
     const int32_t *n_items;     // device count
     const int32_t *cell_start;
-    int *work_counter;          // zeroed before launch,
+    int *work_counter;          // zeroed before launch (a batch takes two, one per form of the masses),
     bool counter_clear = false; // or by the binning just before it
     bool cull = true;           // select the neighbours per cluster, else by the item's bounds alone
     int mode;
@@ -392,9 +393,10 @@ struct ForceLaunch {
     float *phi_out;
     unsigned long long *within; // non-null: count pairs inside the cutoff
     unsigned long long *evaluated = nullptr;   // with within: count the pairs evaluated (after culling)
-    const int *mass_flag;       // from the binning pass (null: masses differ)
+    const uint32_t *mass_flag;  // from the binning pass (null: masses differ)
     // kModeBatch: geometry and kick/stream factors per box, write-back to the pool
     const BoxDev *boxes = nullptr;
+    int nbox = 1;
     const int32_t *ids = nullptr;     // pool row of each sorted particle
     float4 *pos_pool = nullptr;
     float4 *vel_pool = nullptr;

@@ -99,7 +99,8 @@ struct KParams {
     float *phi_out;
     unsigned long long *within;
     unsigned long long *evaluated;
-    const int *mass_flag;
+    const uint32_t *mass_flag;
+    int nbox;
     float w, delta;   // cell/offset form: cell step (an FP32 value) and the remainder L - nc w of a wrap
     const int32_t *levels;
     KickTable kick;
@@ -637,8 +638,7 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
 }
 
 template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
-__device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMem<CI, POT> &S, int lane,
-                                             float m_uniform, int warp) {
+__device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMem<CI, POT> &S, int lane, int warp) {
     // geometry: the single box of the call, or this item's box of a batch
     int nc = P.nc;
     float L = P.L;
@@ -853,7 +853,7 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
         if (POT) {
             P.phi_out[i] = 0.5f * P.G * p.w * sum[0];
         } else {
-            const float gm = UM ? P.G * m_uniform : P.G;
+            const float gm = UM ? P.G * p.w : P.G;   // UM: p.w is every mass of the box
             float h_kick = P.h_kick, h_drift = P.h_drift;
             if (P.boxes) {
                 h_kick = P.boxes[item.w].h;
@@ -873,8 +873,10 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
     __syncwarp();
 }
 
+// Takes items from the queue of `counter` until none is left; with `mixed` it
+// leaves those of the boxes whose masses call for the other form.
 template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
-__device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S, int lane, float m_uniform) {
+__device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S, int lane, int *counter, bool mixed) {
     const int n_items = uniform(*P.n_items);
     const int warp = SH == kByBlock ? uniform(threadIdx.x >> 5) : 0;
     __shared__ int claimed;
@@ -882,11 +884,11 @@ __device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S,
         int it = 0;
         if (SH == kByBlock) {
             __syncthreads();   // the sums of the item before are read
-            if (threadIdx.x == 0) claimed = atomicAdd(P.work_counter, 1);
+            if (threadIdx.x == 0) claimed = atomicAdd(counter, 1);
             __syncthreads();
             it = uniform(claimed);
         } else {
-            if (lane == 0) it = atomicAdd(P.work_counter, 1);
+            if (lane == 0) it = atomicAdd(counter, 1);
             it = __shfl_sync(0xffffffffu, it, 0);
         }
         if (it >= n_items) break;
@@ -895,7 +897,8 @@ __device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S,
         item.y = uniform(item.y);
         item.z = uniform(item.z);
         item.w = uniform(item.w);
-        process_item<COUNT, POT, EPS0, UM, F, CI, SH>(P, item, S, lane, m_uniform, warp);
+        if (mixed && (P.mass_flag[item.w >> 5] >> (item.w & 31) & 1u) == (UM ? 1u : 0u)) continue;
+        process_item<COUNT, POT, EPS0, UM, F, CI, SH>(P, item, S, lane, warp);
     }
 }
 
@@ -907,11 +910,23 @@ __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
     extern __shared__ __align__(16) char smem[];
     WarpMem<CI, POT> *S = reinterpret_cast<WarpMem<CI, POT> *>(smem) + uniform(threadIdx.x >> 5);
     const int lane = __shfl_xor_sync(0xffffffffu, (threadIdx.x & 31) ^ 1, 1);   // as with uniform(): kept
-    // equal masses (flag left 0 by the binning pass): apply the mass once per i
-    if (!POT && P.mass_flag && uniform(*P.mass_flag) == 0 && uniform(*P.n_items) > 0)
-        work_loop<COUNT, POT, EPS0, !POT, F, CI, SH>(P, *S, lane, P.pos[0].w);
-    else
-        work_loop<COUNT, POT, EPS0, false, F, CI, SH>(P, *S, lane, 0.0f);
+    // equal masses in a box (its bit left 0 by the binning pass): applied once per i.
+    // The boxes of a batch take the form that each takes alone, in two rounds of the
+    // queue where both occur (both forms in one loop spilled registers).
+    unsigned some = ~0u, every = ~0u;
+    if (!POT && P.mass_flag) {
+        some = 0u;
+        for (int k = lane; 32 * k < P.nbox; k += 32) {
+            const unsigned v = P.mass_flag[k];
+            some |= v;
+            every &= P.nbox - 32 * k < 32 ? v | ~0u << (P.nbox - 32 * k) : v;
+        }
+        some = __reduce_or_sync(0xffffffffu, some);
+        every = __reduce_and_sync(0xffffffffu, every);
+    }
+    const bool mixed = !CI && SH != kByBlock && some && ~every;   // (those are never a batch's)
+    if (!POT && ~every) work_loop<COUNT, POT, EPS0, !POT, F, CI, SH>(P, *S, lane, P.work_counter, mixed);
+    if (some) work_loop<COUNT, POT, EPS0, false, F, CI, SH>(P, *S, lane, P.work_counter + mixed, mixed);
 }
 
 template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH = kWhole>
@@ -996,6 +1011,7 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     P.within = fl.within;
     P.evaluated = fl.evaluated;
     P.mass_flag = fl.mass_flag;
+    P.nbox = fl.nbox;
     P.boxes = fl.boxes;
     P.ids = fl.ids;
     P.pos_pool = fl.pos_pool;
