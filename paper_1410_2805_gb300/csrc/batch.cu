@@ -52,12 +52,14 @@ size_t carve_batch(char *base, int64_t n, int64_t ncell, int64_t table_entries, 
 struct Plan {
     int nbox = 0;                 // non-empty boxes
     int64_t n_total = 0, ncell_total = 0;
+    bool frames = false;          // some box holds fewer than 4 cells a side
     std::vector<BoxDev> base;     // geometry and offsets (h, pre, post filled per tick)
 };
 
 hacc_status make_plan(hacc_ctx *ctx, const hacc_split *split, int32_t nbox, const hacc_batch_box *boxes, Plan *pl) {
     if (nbox < 0 || (nbox > 0 && !boxes)) return set_error(ctx, HACC_EINVAL, "bad box list");
     pl->base.clear();
+    pl->frames = false;
     int64_t n_total = 0, ncell_total = 0;
     for (int b = 0; b < nbox; ++b) {
         const hacc_batch_box &bb = boxes[b];
@@ -82,6 +84,7 @@ hacc_status make_plan(hacc_ctx *ctx, const hacc_split *split, int32_t nbox, cons
         if (n_total >= ((int64_t)1 << 31) || ncell_total >= ((int64_t)1 << 31) || bb.offset + bb.n >= ((int64_t)1 << 31))
             return set_error(ctx, HACC_EINVAL, "batch too large (2^31 particles, cells or rows)");
         pl->base.push_back(d);
+        pl->frames |= g.nc < 4;
     }
     pl->nbox = (int)pl->base.size();
     pl->n_total = n_total;
@@ -177,6 +180,7 @@ hacc_status run_tick(hacc_ctx *ctx, const ForceConsts &fc, const Plan &pl, const
     }
     fl.boxes = tab;
     fl.nbox = pl.nbox;
+    fl.frames = pl.frames;
     fl.ids = w.IDs;
     fl.pos_pool = pos_pool;
     fl.vel_pool = vel_pool;
@@ -459,6 +463,7 @@ extern "C" hacc_status hacc_batch_diagnostics(hacc_ctx *ctx, const hacc_split *s
     fl.variant = ctx->variant;
     fl.boxes = w.tables;
     fl.nbox = pl.nbox;
+    fl.frames = pl.frames;
     fl.ids = w.IDs;
     fl.flags = ctx->d_flags;
     HACC_CUDA_RETURN(sr_force_launch(g0, fc, fl, ctx->num_sms, s), "batched pair potential");

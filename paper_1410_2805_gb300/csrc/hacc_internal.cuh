@@ -397,6 +397,7 @@ struct ForceLaunch {
     // kModeBatch: geometry and kick/stream factors per box, write-back to the pool
     const BoxDev *boxes = nullptr;
     int nbox = 1;
+    bool frames = false;        // some box holds fewer than 4 cells a side
     const int32_t *ids = nullptr;     // pool row of each sorted particle
     float4 *pos_pool = nullptr;
     float4 *vel_pool = nullptr;

@@ -46,10 +46,15 @@
 // Periodic images without rounding error: an item whose cell lies within R of
 // a high face (per axis) runs in the frame moved by -L: its own particles and
 // the neighbours of unwrapped rows get -L (they lie in [L/2, L) for nc >= 4R:
-// exact; for smaller nc only those a quarter of a cutoff or more apart are
-// rounded), those of rows that wrap high stay.  Elsewhere the neighbours of
-// rows that wrap low get -L (exact, in [2L/3, L)).  So r_ij = x_j' - x_i'
-// carries only the rounding of one subtraction.
+// exact), those of rows that wrap high stay.  In smaller meshes neighbours of
+// unwrapped rows may lie below L/2, so there such an item runs in a frame for
+// each set of axes, with its own particles moved by -L on just these (exact both
+// ways) and the rows that wrap high on just these as they are, in a form of the
+// kernel of its own (with the frames in the one form, 250 thousand particles of
+// differing masses took 206 us a call instead of 203, the step of the 256^3 box
+// 38.2 ms instead of 37.9).  Elsewhere the neighbours of rows that wrap low get
+// -L (exact, in [L/2, L)).  So r_ij = x_j' - x_i' carries only the rounding of
+// one subtraction.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -149,6 +154,10 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     return r;
 }
 
+__device__ __forceinline__ float4 shift4(float4 v, float tx, float ty, float tz) {
+    return make_float4(__fadd_rn(v.x, tx), __fadd_rn(v.y, ty), __fadd_rn(v.z, tz), v.w);
+}
+
 constexpr int kRound = 64;                // candidates staged per round
 constexpr int kRing = 128;                // list entries held: two chunks
 constexpr int kChunk = 64;                // list entries per call of the pair loop
@@ -173,7 +182,9 @@ static_assert(sizeof(WarpBuf<true>) <= kBufBytes && WarpBuf<false>::kTile % kRou
 
 // A warp's shared memory.  Runs: (first, end, bits, b1) of the sorted
 // particles of each x-run, with (b2, d0) for the cell/offset form; bits 1/2/4:
-// the staged j's x/y/z get -L; in the cell/offset form bits 0-3 and 4-7 hold
+// the staged j's x/y/z get -L; bits 3-5 and b1, for an item in several frames:
+// the one that the run belongs to and the run's end, where end = first leaves it
+// to another frame; in the cell/offset form bits 0-3 and 4-7 hold
 // dy + 2 and dz + 2, bits 8-13 the wrap flags (1/2/4 low in x/y/z, 8/16/32
 // high), and the x cell step of entry j is d0 + (j >= b1) + (j >= b2).
 template <bool CI, bool POT>
@@ -186,6 +197,8 @@ struct WarpMem {
     int2 steps[CI ? kMaxRuns : 1];
     int tile_id[POT ? WarpBuf<true>::kTile : 1];         // sorted index of each entry (the j != i test of the potential)
     int id[POT ? kRing : 1];
+    int frames;                           // 0, or of an item in several frames: their axes, from bit 3 on those of the
+                                          // present one, from bit 6 on its number
     template <bool M>
     __device__ __forceinline__ WarpBuf<M> &as() {
         return *reinterpret_cast<WarpBuf<M> *>(buf);
@@ -196,10 +209,11 @@ struct WarpMem {
 // lane per run: row (dz, dy) of the (2R+1)^2 rows gives run `row` (cells
 // cx-R..cx+R, or the part of them in [0, nc)) and, when rows wrap in x, run
 // span^2 + row (the wrapped part).  fr: axes on which the item runs in the
-// frame moved by -L.  Returns the number of runs.
+// frame moved by -L; with `several`, for the rows that wrap high on just these.
+// Returns the number of runs.
 template <bool CI, bool POT>
 __device__ __forceinline__ int build_runs(const KParams &P, WarpMem<CI, POT> &S, int cbase, int nc, int cx, int cy,
-                                          int cz, int R, int fr, int lane) {
+                                          int cz, int R, int fr, bool several, int lane) {
     const int span = 2 * R + 1, rows = span * span;
     const int lo = cx - R, hi = cx + R;
     const bool wraps = lo < 0 || hi >= nc;
@@ -228,7 +242,7 @@ __device__ __forceinline__ int build_runs(const KParams &P, WarpMem<CI, POT> &S,
             d0 = r ? 1 : -1;
         }
         const int ja = row[ca], jb = row[cb];
-        int bits, b1 = jb;
+        int bits, b1 = jb, end = jb;
         if (CI) {
             bits = (dy + 2) | ((dz + 2) << 4) | (wb << 8);
             // first entries of the run's second and third cell (R = 1)
@@ -237,12 +251,47 @@ __device__ __forceinline__ int build_runs(const KParams &P, WarpMem<CI, POT> &S,
             S.steps[q] = make_int2(b2, d0);
         } else {
             // -L on an axis: rows wrapped low, or every row not wrapped high in the moved frame
-            bits = (wb & 7) | (fr & ~(wb >> 3));
+            bits = (wb & 7) | (several ? wb & 56 : fr & ~(wb >> 3));
+            if (several && wb >> 3 != fr) end = ja;
         }
-        S.runs[q] = make_int4(ja, jb, bits, b1);
+        S.runs[q] = make_int4(ja, end, bits, b1);
     }
     __syncwarp();
     return uniform(nrun);
+}
+
+// Frame r of an item that runs in one for each subset of `axes`: the r-th subset.
+__device__ __forceinline__ int frame_of(int r, int axes) {
+    int f = 0;
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+        if (axes & b) {
+            f |= r & 1 ? b : 0;
+            r >>= 1;
+        }
+    return f;
+}
+
+// From one frame of an item in several to frame r: its particles and bounds
+// moved on the axes that differ, and the runs of the new frame.
+template <bool CI, bool POT>
+__device__ __forceinline__ void change_frame(WarpMem<CI, POT> &S, int axes, int from, int r, float L, int nrun,
+                                             int lane) {
+    const int to = frame_of(r, axes);
+    const float tx = L * (float)((from & 1) - (to & 1)), ty = L * (float)((from >> 1 & 1) - (to >> 1 & 1)),
+                tz = L * (float)((from >> 2) - (to >> 2));
+    __syncwarp();
+    for (int e = lane; e < kItemMax; e += 32) S.own[e] = shift4(S.own[e], tx, ty, tz);
+    if (lane <= kMaxClusters) {
+        S.lo[lane] = shift4(S.lo[lane], tx, ty, tz);
+        S.hi[lane] = shift4(S.hi[lane], tx, ty, tz);
+    }
+    for (int q = lane; q < nrun; q += 32) {
+        const int4 run = S.runs[q];
+        S.runs[q].y = run.z >> 3 == to ? run.w : run.x;
+    }
+    if (lane == 0) S.frames = axes | to << 3 | r << 6;
+    __syncwarp();
 }
 
 // Apply the force on sorted particle i (position x, y, z, mass m) as the
@@ -426,10 +475,6 @@ __device__ __forceinline__ int put3(float d2, float r2, unsigned below, unsigned
 }
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ float4 shift4(float4 v, float tx, float ty, float tz) {
-    return make_float4(__fadd_rn(v.x, tx), __fadd_rn(v.y, ty), __fadd_rn(v.z, tz), v.w);
-}
 
 // This lane's two particles: their negated coordinates, doubled, and their
 // sums over the list entries the lane's group took (one sum per half).
@@ -637,7 +682,7 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
     __syncwarp();
 }
 
-template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH, bool FRAMES>
 __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMem<CI, POT> &S, int lane, int warp) {
     // geometry: the single box of the call, or this item's box of a batch
     int nc = P.nc;
@@ -653,8 +698,21 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
     const int c = item.x - cbase, i0 = item.y, ni = item.z;
     const int cx = c % nc, cy = (c / nc) % nc, cz = c / (nc * nc);
     const int R = P.boxes ? 1 : P.R;
-    // axes on which the item runs in the frame moved by -L
-    const int fr = CI ? 0 : ((cx + R >= nc ? 1 : 0) | (cy + R >= nc ? 2 : 0) | (cz + R >= nc ? 4 : 0));
+    // The rounds of a shared item go to its warps in turn, each run starting with
+    // another warp: most runs are one full round and a part.  The warp of a batch
+    // goes through the parts of a small box's item one after the other, so that
+    // its sums are those of the box in a call of its own.  Of an item in several
+    // frames a part takes its share of the frames, or, where they are fewer than
+    // the parts, its share of the rounds of one (with all frames in every part, a
+    // batch of 500 boxes of 3 cells a side and 1000 particles took 1234 us, now 957).
+    int part = SH == kByBlock ? warp : 0;
+    if (SH == kByBlock) parts = kWarps;
+    // axes on which the item runs in the frame moved by -L, and those of its first frame
+    const int axes = CI ? 0 : ((cx + R >= nc ? 1 : 0) | (cy + R >= nc ? 2 : 0) | (cz + R >= nc ? 4 : 0));
+    const bool several = FRAMES && axes && nc < 4 * R;
+    const int log_frames = several ? __popc(axes) : 0, first_frame = part & ((1 << log_frames) - 1);
+    const int fr = several ? frame_of(first_frame, axes) : axes;
+    int shares = max(1, parts >> log_frames), share = part >> log_frames;   // of the rounds of a frame; this part's
     {
         float4 lo = make_float4(1e30f, 1e30f, 1e30f, 0.0f), hi = make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
 #pragma unroll
@@ -701,7 +759,8 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
         }
     }
     const float r2 = P.T * 1.001f + 1e-3f;
-    const int nrun = build_runs<CI, POT>(P, S, cbase, nc, cx, cy, cz, R, fr, lane);
+    if (FRAMES && lane == 0) S.frames = several ? axes | fr << 3 | first_frame << 6 : 0;
+    const int nrun = build_runs<CI, POT>(P, S, cbase, nc, cx, cy, cz, R, fr, several, lane);
     // In the cell/offset form a wrapped neighbour lies the remainder L - nc w
     // beyond the whole cell steps: moving i by it instead keeps the j side
     // exact (the shifted i is exact too for any i within reach of the face),
@@ -713,24 +772,18 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
     constexpr int kTile = WarpBuf<!UM>::kTile;
     const unsigned below = (1u << lane) - 1u, tile = smem_addr(S.buf);
     int fill = 0;
-    // The rounds of a shared item go to its warps in turn, each run starting with
-    // another warp: most runs are one full round and a part.  The warp of a batch
-    // goes through the parts of a small box's item one after the other, so that
-    // its sums are those of the box in a call of its own.
-    int part = SH == kByBlock ? warp : 0;
-    if (SH == kByBlock) parts = kWarps;
     // the stream of rounds: 64 particles of a run (past its end: its last one
     // again, never kept); the next round's loads are in flight while this one's
     // are tested
     int q = -1, j0 = 0, end = 0, bits = 0, b1 = 0;
     float sx = 0.0f, sy = 0.0f, sz = 0.0f;   // shift of the run's particles
     auto next = [&]() -> bool {
-        j0 += SH == kWhole ? kRound : kRound * parts;
+        j0 += SH == kWhole ? kRound : kRound * shares;
         while (j0 >= end) {
             if (++q >= nrun) return false;
             const int4 run = S.runs[q];
             j0 = uniform(run.x);
-            if (SH != kWhole) j0 += kRound * ((part - q) & (parts - 1));
+            if (SH != kWhole) j0 += kRound * ((share - q) & (shares - 1));
             end = uniform(run.y);
             bits = uniform(run.z);
             b1 = run.w;
@@ -816,6 +869,19 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
             }
         }
         if (fill) flush_tile<COUNT, POT, EPS0, UM, F, CI>(P, S, fill, i0, ni, tx, ty, tz, r2, lane, cnt, evals);
+        if constexpr (FRAMES) {
+            if (const int w = uniform(S.frames)) {   // on to the part's next frame, or the first of the next part
+                const int all = w & 7, r = (w >> 6) + (SH == kWhole ? 1 : parts), n = 1 << __popc(all);
+                const bool on = r < n, first = SH == kByParts && !on && part + 1 < parts;
+                if (on || first) change_frame<CI, POT>(S, all, w >> 3 & 7, on ? r : (part + 1) & (n - 1), L, nrun, lane);
+                if (on) {
+                    fill = 0;
+                    q = -1;
+                    j0 = end = 0;
+                    continue;
+                }
+            }
+        }
         if (SH != kByParts || parts == 1) break;
         if constexpr (SH == kByParts) {
             // the parts' sums are added in order (items of a small box hold at most 32 particles)
@@ -826,6 +892,7 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
             }
             __syncwarp();
             if (++part == parts) break;
+            share = part >> log_frames;
             fill = 0;
             q = -1;
             j0 = end = 0;
@@ -875,7 +942,7 @@ __device__ __forceinline__ void process_item(const KParams &P, int4 item, WarpMe
 
 // Takes items from the queue of `counter` until none is left; with `mixed` it
 // leaves those of the boxes whose masses call for the other form.
-template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH>
+template <bool COUNT, bool POT, bool EPS0, bool UM, int F, bool CI, Sharing SH, bool FRAMES>
 __device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S, int lane, int *counter, bool mixed) {
     const int n_items = uniform(*P.n_items);
     const int warp = SH == kByBlock ? uniform(threadIdx.x >> 5) : 0;
@@ -898,14 +965,15 @@ __device__ __forceinline__ void work_loop(const KParams &P, WarpMem<CI, POT> &S,
         item.z = uniform(item.z);
         item.w = uniform(item.w);
         if (mixed && (P.mass_flag[item.w >> 5] >> (item.w & 31) & 1u) == (UM ? 1u : 0u)) continue;
-        process_item<COUNT, POT, EPS0, UM, F, CI, SH>(P, item, S, lane, warp);
+        process_item<COUNT, POT, EPS0, UM, F, CI, SH, FRAMES>(P, item, S, lane, warp);
     }
 }
 
+// FRAMES: boxes of fewer than 4 R cells a side, whose items may run in several frames.
 // MINB: blocks per SM the register allocation must allow; F: steps of the
 // pair loop unrolled.  The autotuner picks.  SH: the warps of a block share each
 // item (calls of few items, see shared_items).
-template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH>
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH, bool FRAMES>
 __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
     extern __shared__ __align__(16) char smem[];
     WarpMem<CI, POT> *S = reinterpret_cast<WarpMem<CI, POT> *>(smem) + uniform(threadIdx.x >> 5);
@@ -925,13 +993,13 @@ __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
         every = __reduce_and_sync(0xffffffffu, every);
     }
     const bool mixed = !CI && SH != kByBlock && some && ~every;   // (those are never a batch's)
-    if (!POT && ~every) work_loop<COUNT, POT, EPS0, !POT, F, CI, SH>(P, *S, lane, P.work_counter, mixed);
-    if (some) work_loop<COUNT, POT, EPS0, false, F, CI, SH>(P, *S, lane, P.work_counter + mixed, mixed);
+    if (!POT && ~every) work_loop<COUNT, POT, EPS0, !POT, F, CI, SH, FRAMES>(P, *S, lane, P.work_counter, mixed);
+    if (some) work_loop<COUNT, POT, EPS0, false, F, CI, SH, FRAMES>(P, *S, lane, P.work_counter + mixed, mixed);
 }
 
-template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH = kWhole>
+template <bool COUNT, bool POT, bool EPS0, int MINB, int F, bool CI, Sharing SH = kWhole, bool FRAMES = false>
 cudaError_t launch_one(const KParams &P, int num_sms, cudaStream_t s) {
-    auto *k = k_sr_force<COUNT, POT, EPS0, MINB, F, CI, SH>;
+    auto *k = k_sr_force<COUNT, POT, EPS0, MINB, F, CI, SH, FRAMES>;
     const size_t bytes = kWarps * sizeof(WarpMem<CI, POT>);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
@@ -962,14 +1030,14 @@ cudaError_t launch_variant(const KParams &P, int variant, int num_sms, cudaStrea
     }
 }
 
-// Shared items: one variant each, bitwise the same forces.
-template <Sharing SH>
-cudaError_t launch_shared(const KParams &P, bool eps0, bool count, int num_sms, cudaStream_t s) {
+// Shared items and items in several frames: one variant each, bitwise the same forces.
+template <Sharing SH, bool FRAMES>
+cudaError_t launch_form(const KParams &P, bool eps0, bool count, int num_sms, cudaStream_t s) {
     if (count)
-        return eps0 ? launch_one<true, false, true, 4, 1, false, SH>(P, num_sms, s)
-                    : launch_one<true, false, false, 4, 1, false, SH>(P, num_sms, s);
-    return eps0 ? launch_one<false, false, true, 5, 4, false, SH>(P, num_sms, s)
-                : launch_one<false, false, false, 5, 4, false, SH>(P, num_sms, s);
+        return eps0 ? launch_one<true, false, true, 4, 1, false, SH, FRAMES>(P, num_sms, s)
+                    : launch_one<true, false, false, 4, 1, false, SH, FRAMES>(P, num_sms, s);
+    return eps0 ? launch_one<false, false, true, 5, 4, false, SH, FRAMES>(P, num_sms, s)
+                : launch_one<false, false, false, 5, 4, false, SH, FRAMES>(P, num_sms, s);
 }
 
 }  // namespace
@@ -1030,11 +1098,20 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     if (fl.cell_offset)
         return eps0 ? launch_one<false, false, true, 4, 4, true>(P, num_sms, s)
                     : launch_one<false, false, false, 4, 4, true>(P, num_sms, s);
+    const bool frames = fl.boxes ? fl.frames : g.nc < 4 * g.R;
+    if (pot && frames)
+        return eps0 ? launch_one<false, true, true, 4, 1, false, kWhole, true>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 1, false, kWhole, true>(P, num_sms, s);
     if (pot)
         return eps0 ? launch_one<false, true, true, 4, 1, false>(P, num_sms, s)
                     : launch_one<false, true, false, 4, 1, false>(P, num_sms, s);
-    if (fl.sharing == kByBlock) return launch_shared<kByBlock>(P, eps0, count, num_sms, s);
-    if (fl.sharing == kByParts) return launch_shared<kByParts>(P, eps0, count, num_sms, s);
+    if (fl.sharing == kByBlock)
+        return frames ? launch_form<kByBlock, true>(P, eps0, count, num_sms, s)
+                      : launch_form<kByBlock, false>(P, eps0, count, num_sms, s);
+    if (fl.sharing == kByParts)
+        return frames ? launch_form<kByParts, true>(P, eps0, count, num_sms, s)
+                      : launch_form<kByParts, false>(P, eps0, count, num_sms, s);
+    if (frames) return launch_form<kWhole, true>(P, eps0, count, num_sms, s);
     if (count)
         return eps0 ? launch_one<true, false, true, 4, 1, false>(P, num_sms, s)
                     : launch_one<true, false, false, 4, 1, false>(P, num_sms, s);
