@@ -1474,8 +1474,6 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
     b->packed = c.take<unsigned long long>(ncell);
     b->scan_tmp = c.take<unsigned long long>(scan_tmp_elems(ncell));
     b->cell_start = c.take<int32_t>(ncell + 1);
-    b->item_start = nullptr;
-    b->perm_tmp = c.take<int32_t>(n);
     b->perm = c.take<int32_t>(n);
     b->items = c.take<int4>(max_items(n, ncell, sub_order));
     b->order = c.take<int32_t>(max_items(n, ncell, sub_order));
@@ -1484,6 +1482,9 @@ void carve_bin(Carver &c, int64_t n, int64_t ncell, BinBuffers *b, bool sub_orde
     b->big_list = c.take<int32_t>(n / (kBigCell + 1) + 1);
     b->sub = sub_order ? c.take<uint8_t>(n) : nullptr;
     b->order_tmp = sub_order ? c.take<unsigned long long>(n) : nullptr;
+    // a call with sub-cells takes the ranks' place for perm_tmp, which it writes when
+    // they have been read, one without them that of order_tmp (bin_sort)
+    b->perm_tmp = sub_order ? nullptr : c.take<int32_t>(n);
 }
 
 namespace {
@@ -1500,8 +1501,9 @@ cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_it
                      uint32_t row_below, bool stretches, const Gather &gather) {
     cudaError_t e = scan_cells(ncell, n, CellPack{b.count, cap, boxes, nbox}, b, make_items, s);
     if (e != cudaSuccess) return e;
+    int32_t *perm_tmp = b.perm_tmp ? b.perm_tmp : (sub ? b.rank : reinterpret_cast<int32_t *>(b.order_tmp));
     if (n > 0) {
-        k_place<<<blocks_for(n), kBlock, 0, s>>>(n, b.key, b.rank, b.packed, b.perm_tmp, sub, b.order_tmp);
+        k_place<<<blocks_for(n), kBlock, 0, s>>>(n, b.key, b.rank, b.packed, perm_tmp, sub, b.order_tmp);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // cells per block of the ordering: 64, fewer where that leaves SMs without a block
@@ -1510,21 +1512,21 @@ cudaError_t bin_sort(int64_t n, int64_t ncell, const BinBuffers &b, bool make_it
         const bool by_row = !(sub && n > kOrdSubMaxRows);   // in k_order_rows
         const Gather here = by_row && n <= kGatherHereMax ? gather : Gather{};
         if (!by_row)
-            k_order_sub<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
+            k_order_sub<<<blocks_for(ncell * 32), kBlock, 0, s>>>(ncell, b.count, b.packed, perm_tmp, b.perm,
                                                                   b.big_list, b.big_count, b.order_tmp, row_below);
         else if (sub)
-            k_order_rows<true><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
+            k_order_rows<true><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, perm_tmp, b.perm,
                                                                        b.big_list, b.big_count, b.order_tmp,
                                                                        row_below, stretches ? 1 : 0, oc, big_here, here);
         else
-            k_order_rows<false><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, b.perm_tmp, b.perm,
+            k_order_rows<false><<<blocks_for(ncell, oc), kBlock, 0, s>>>(ncell, b.count, b.packed, perm_tmp, b.perm,
                                                                         b.big_list, b.big_count, nullptr, 0u,
                                                                         stretches ? 1 : 0, oc, big_here, here);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // k_order_sub lists cells above kBigCell, k_order_rows those above kBlockCell
         if (!big_here && n > (int64_t)(by_row ? kBlockCell : kBigCell)) {
-            k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, b.perm_tmp, b.perm, b.big_list, b.big_count,
+            k_order_big<<<256, kOrderThreads, 0, s>>>(b.count, b.packed, perm_tmp, b.perm, b.big_list, b.big_count,
                                                       here);
             note_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;

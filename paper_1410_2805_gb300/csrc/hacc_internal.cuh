@@ -233,8 +233,7 @@ struct BinBuffers {
     unsigned long long *packed;  // [ncell] scan workspace
     unsigned long long *scan_tmp;
     int32_t *cell_start;   // [ncell + 1]
-    int32_t *item_start;   // [ncell + 1]
-    int32_t *perm_tmp;     // [n]
+    int32_t *perm_tmp;     // [n] rows in arrival order (without sub-cells; with them, those of big cells)
     int32_t *perm;         // [n]
     int4 *items;           // [max_items]
     int32_t *order;        // [max_items] work-queue order of the items (heavy_first), or unused
@@ -246,7 +245,7 @@ struct BinBuffers {
     int *work_counter;     // [2] device: cleared by each binning (the force launch that follows it)
     size_t zeroed;         // words from count on that a binning clears: count, the counters, mass_flag
     uint8_t *sub;                  // [n] sub-cell code of each input row (item_cap > 0), or null
-    unsigned long long *order_tmp; // [n] (sub-cell << 32 | row) in the slots of perm_tmp, or null
+    unsigned long long *order_tmp; // [n] (sub-cell << 32 | row) in arrival order, or null
 };
 
 // Sorted copies that a binning makes on its way (p_out null: none): slot k gets
