@@ -359,10 +359,12 @@ __device__ __forceinline__ float box_dist2(float4 v, float4 lo, float4 hi) {
 // widths nh (s times them): the distance from them along an axis is
 // s |v - c| + nh, cut to [0, 1] by the saturation of the FMA itself.  Axes past
 // the reach saturate at 1, so a j is within reach when the squares sum to less
-// than 1.  v - c and c - lo are differences of FP32 values, so the test is off
-// by a few ulp of the distance, whatever the side of the box.  Against clamping
-// v to [lo, hi], half the instructions: no minimum and maximum, which run at
-// half the rate, and the subtraction and the squares packed.
+// than 1.  The roundings of c, of v - c and of the half widths and their product
+// with s move a distance by a few ulp of the half width, more than the margin of
+// the limit where a cluster is thousands of cutoffs wide (few particles in wide
+// cells): the half widths are widened by 2^-21, eight such roundings.  Against
+// clamping v to [lo, hi], half the instructions: no minimum and maximum, which
+// run at half the rate, and the subtraction and the squares packed.
 struct Reach {
     float cx, cy, cz, nhx, nhy, nhz, s;
 };
@@ -373,9 +375,10 @@ __device__ __forceinline__ Reach reach_of(float4 lo, float4 hi, float s) {
     b.cx = 0.5f * lo.x + 0.5f * hi.x;
     b.cy = 0.5f * lo.y + 0.5f * hi.y;
     b.cz = 0.5f * lo.z + 0.5f * hi.z;
-    b.nhx = -s * fmaxf(hi.x - b.cx, b.cx - lo.x);
-    b.nhy = -s * fmaxf(hi.y - b.cy, b.cy - lo.y);
-    b.nhz = -s * fmaxf(hi.z - b.cz, b.cz - lo.z);
+    const float wide = -s * (1.0f + 0x1p-21f);
+    b.nhx = wide * fmaxf(hi.x - b.cx, b.cx - lo.x);
+    b.nhy = wide * fmaxf(hi.y - b.cy, b.cy - lo.y);
+    b.nhz = wide * fmaxf(hi.z - b.cz, b.cz - lo.z);
     return b;
 }
 
