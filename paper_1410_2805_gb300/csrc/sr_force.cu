@@ -82,6 +82,11 @@ struct PairConsts {
     f32x2 eps, c0, c1, c2, c3, c4, c5;
 };
 
+// The pair potential's, likewise: U's coefficients and phi0 negated, and -1.
+struct PotConsts {
+    f32x2 u0, u1, u2, u3, u4, u5, u6, phi0, minus;
+};
+
 struct KParams {
     const float4 *__restrict__ pos;
     const int4 *__restrict__ items;
@@ -94,7 +99,6 @@ struct KParams {
     int cull;         // 1: select per cluster; 0: by the item's bounds alone
     float L;
     float T, eps, G;
-    float u0, u1, u2, u3, u4, u5, u6, phi0;
     int mode;
     float4 *out;
     const int32_t *__restrict__ perm;
@@ -115,6 +119,7 @@ struct KParams {
     float4 *vel_pool;
     int *flags;
     PairConsts pair;
+    PotConsts pot;
 };
 
 __device__ __forceinline__ float rsqrt_approx(float x) {
@@ -196,7 +201,7 @@ struct WarpMem {
     int4 runs[kMaxRuns];
     int2 steps[CI ? kMaxRuns : 1];
     int tile_id[POT ? WarpBuf<true>::kTile : 1];         // sorted index of each entry (the j != i test of the potential)
-    int id[POT ? kRing : 1];
+    alignas(8) int id[POT ? kRing : 1];   // those of the list's
     int frames;                           // 0, or of an item in several frames: their axes, from bit 3 on those of the
                                           // present one, from bit 6 on its number
     template <bool M>
@@ -526,34 +531,32 @@ __device__ __forceinline__ void pair_step(const PairConsts &C, float T, unsigned
 }
 
 // The same for the pair potential: phi(s) = -t^(-1/2) - U(t) - phi0 inside
-// the cutoff, U in t = s + eps; A.ax[k] = sum_j m_j phi over j != i.
-template <bool CI, bool POT>
-__device__ __forceinline__ void potential_loop(const KParams &P, WarpMem<CI, POT> &S, int base, int len, int grp,
+// the cutoff, U in t = s + eps; A.ax[k] = sum_j m_j phi over j != i, with the
+// entries' sorted indices at `ids` and i that of the lane's first particle.
+// Packed as the force is, for the same reasons (an entry at a time, the
+// diagnostics of three boxes of 2 million particles took 4.89 ms, now 3.44).
+__device__ __forceinline__ void potential_step(const PotConsts &C, f32x2 eps, float T, unsigned addr, unsigned ids,
                                                int i, Pair &A) {
-    const auto &list = S.template as<true>().list;
-#pragma unroll 1
-    for (int e = base + 2 * grp; e < base + len; e += 16) {
+    const f32x2 X = lds2(addr, 0), Y = lds2(addr, 4 * kRing), Z = lds2(addr, 8 * kRing), M = lds2(addr, 12 * kRing);
+    const f32x2 j = lds2(ids, 0);
+    const int j0 = (int)(uint32_t)j, j1 = (int)(j >> 32);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            float px, py, pz, u, ph[2];
-            unpack2(A.nx[k], px, u);
-            unpack2(A.ny[k], py, u);
-            unpack2(A.nz[k], pz, u);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float dx = list[0][e + h] + px, dy = list[1][e + h] + py, dz = list[2][e + h] + pz;
-                const float t = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, P.eps)));
-                u = __fmaf_rn(P.u6, t, P.u5);
-                u = __fmaf_rn(u, t, P.u4);
-                u = __fmaf_rn(u, t, P.u3);
-                u = __fmaf_rn(u, t, P.u2);
-                u = __fmaf_rn(u, t, P.u1);
-                u = __fmaf_rn(u, t, P.u0);
-                const bool in = t < P.T && S.id[e + h] != i + k;
-                ph[h] = in ? (-rsqrt_approx(t) - u - P.phi0) * list[3][e + h] : 0.0f;
-            }
-            A.ax[k] = add2(A.ax[k], pack2(ph[0], ph[1]));
-        }
+    for (int k = 0; k < 2; ++k) {
+        const f32x2 dx = add2(X, A.nx[k]), dy = add2(Y, A.ny[k]), dz = add2(Z, A.nz[k]);
+        const f32x2 t2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, eps)));
+        float t0, t1;
+        unpack2(t2, t0, t1);
+        const f32x2 r = pack2(rsqrt_approx(t0), rsqrt_approx(t1));
+        f32x2 u = fma2(C.u6, t2, C.u5);   // -U
+        u = fma2(u, t2, C.u4);
+        u = fma2(u, t2, C.u3);
+        u = fma2(u, t2, C.u2);
+        u = fma2(u, t2, C.u1);
+        u = fma2(u, t2, C.u0);
+        u = mul2(add2(fma2(r, C.minus, u), C.phi0), M);
+        float u0, u1;
+        unpack2(u, u0, u1);
+        A.ax[k] = add2(A.ax[k], pack2(t0 < T && j0 != i + k ? u0 : 0.0f, t1 < T && j1 != i + k ? u1 : 0.0f));
     }
 }
 
@@ -576,6 +579,7 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
     const unsigned below = (1u << lane) - 1u;
     const int grp = lane >> 2, slot = lane & 3;
     const unsigned tile = smem_addr(buf.tile), ring = smem_addr(buf.list), mine = ring + 8 * grp;   // the list; this group's entry pairs
+    const unsigned ids = smem_addr(S.id) + 8 * grp;   // POT: the list's sorted indices
     const float T = keep(P.T), s_reach = rsqrtf(r2);
 #pragma unroll 1
     for (int c0 = 0; c0 < ni; c0 += kCluster) {
@@ -624,8 +628,11 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
             if (todo >= kChunk) {
                 __syncwarp();
                 const int base = (at - todo) & (kRing - 1);
-                if (POT) {
-                    potential_loop<CI, POT>(P, S, base, kChunk, grp, i0 + c0 + 2 * slot, A);
+                if constexpr (POT) {
+#pragma unroll F
+                    for (int t = 0; t < kChunk / 16; ++t)
+                        potential_step(P.pot, P.pair.eps, T, mine + 4 * base + 64 * t, ids + 4 * base + 64 * t,
+                                       i0 + c0 + 2 * slot, A);
                 } else {
 #pragma unroll F
                     for (int t = 0; t < kChunk / 16; ++t)
@@ -644,8 +651,10 @@ __device__ __forceinline__ void flush_tile(const KParams &P, WarpMem<CI, POT> &S
                 if (POT) S.id[q] = -1;
             }
             __syncwarp();
-            if (POT) {
-                potential_loop<CI, POT>(P, S, base, len, grp, i0 + c0 + 2 * slot, A);
+            if constexpr (POT) {
+#pragma unroll 1
+                for (int q = 4 * base; q < 4 * (base + len); q += 64)
+                    potential_step(P.pot, P.pair.eps, T, mine + q, ids + q, i0 + c0 + 2 * slot, A);
             } else {
                 // 1 to 4 steps, without the loop's overhead
                 unsigned q = mine + 4 * base;
@@ -1068,9 +1077,8 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     P.G = fc.G;
     P.pair = PairConsts{doubled(fc.eps),   doubled(-fc.q[0]), doubled(-fc.q[1]), doubled(-fc.q[2]),
                         doubled(-fc.q[3]), doubled(-fc.q[4]), doubled(-fc.q[5])};
-    P.u0 = fc.u[0]; P.u1 = fc.u[1]; P.u2 = fc.u[2]; P.u3 = fc.u[3]; P.u4 = fc.u[4]; P.u5 = fc.u[5];
-    P.u6 = fc.u[6];
-    P.phi0 = fc.phi0;
+    P.pot = PotConsts{doubled(-fc.u[0]), doubled(-fc.u[1]), doubled(-fc.u[2]), doubled(-fc.u[3]), doubled(-fc.u[4]),
+                      doubled(-fc.u[5]), doubled(-fc.u[6]), doubled(-fc.phi0),  doubled(-1.0f)};
     P.mode = fl.mode;
     P.out = fl.out;
     P.perm = fl.perm;
@@ -1096,18 +1104,18 @@ cudaError_t sr_force_launch(const Geometry &g, const ForceConsts &fc, const Forc
     const bool count = fl.within != nullptr;
     const int v = fl.variant;
     if (fl.cell_offset && pot)
-        return eps0 ? launch_one<false, true, true, 4, 1, true>(P, num_sms, s)
-                    : launch_one<false, true, false, 4, 1, true>(P, num_sms, s);
+        return eps0 ? launch_one<false, true, true, 4, 4, true>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 4, true>(P, num_sms, s);
     if (fl.cell_offset)
         return eps0 ? launch_one<false, false, true, 4, 4, true>(P, num_sms, s)
                     : launch_one<false, false, false, 4, 4, true>(P, num_sms, s);
     const bool frames = fl.boxes ? fl.frames : g.nc < 4 * g.R;
     if (pot && frames)
-        return eps0 ? launch_one<false, true, true, 4, 1, false, kWhole, true>(P, num_sms, s)
-                    : launch_one<false, true, false, 4, 1, false, kWhole, true>(P, num_sms, s);
+        return eps0 ? launch_one<false, true, true, 4, 4, false, kWhole, true>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 4, false, kWhole, true>(P, num_sms, s);
     if (pot)
-        return eps0 ? launch_one<false, true, true, 4, 1, false>(P, num_sms, s)
-                    : launch_one<false, true, false, 4, 1, false>(P, num_sms, s);
+        return eps0 ? launch_one<false, true, true, 4, 4, false>(P, num_sms, s)
+                    : launch_one<false, true, false, 4, 4, false>(P, num_sms, s);
     if (fl.sharing == kByBlock)
         return frames ? launch_form<kByBlock, true>(P, eps0, count, num_sms, s)
                       : launch_form<kByBlock, false>(P, eps0, count, num_sms, s);
