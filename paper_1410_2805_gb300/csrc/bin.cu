@@ -121,13 +121,25 @@ __global__ void __launch_bounds__(kBlock) k_key(int64_t n, const float4 *__restr
     if (i < n) rank[i] = (int32_t)slot;
 }
 
+constexpr uint32_t kBlockCell = 2048;   // cells above it are ordered apart (see the ordering)
+
 // How cells are cut into work items: the ceil(cnt / kCluster) clusters of a
 // cell of cnt particles become items of at most `clusters` clusters, or of
 // kItemMax particles when cnt > split_max.
-// clusters = 0: the automatic cap of the cell's box (batches).
+// clusters = 0: the automatic cap of the cell's box (batches).  A cell of more than
+// `dense` particles takes items of half of kItemMax at most.
 struct ItemRule {
-    uint32_t clusters, split_max;
+    uint32_t clusters, split_max, dense = 0xffffffffu;
 };
+
+// Cells this far above the mean and kBlockCell are few and most of their box's
+// work: smaller items spread it over the chip (two cells of 30000 particles and
+// one of 20000 among 2 million, a force call: 8.8 ms with items of 64, 5.3 with 32;
+// everywhere dense, 45 particles per unit volume, 32 are 4% slower).
+__host__ __device__ inline uint32_t dense_cell(uint32_t n, uint32_t ncell) {
+    const unsigned long long d = 8ull * (n / ncell + 1);
+    return d < kBlockCell ? kBlockCell : (d < 0xffffffffull ? (uint32_t)d : 0xffffffffu);
+}
 
 // Box of a batch that global cell c belongs to: the last whose first cell is <= c.
 __device__ __forceinline__ int box_of_cell(const BoxDev *__restrict__ boxes, int nbox, int64_t c) {
@@ -142,13 +154,15 @@ __device__ __forceinline__ int box_of_cell(const BoxDev *__restrict__ boxes, int
 
 __device__ __forceinline__ ItemRule rule_of_box(ItemRule r, const BoxDev &b) {
     if (r.clusters == 0) r.clusters = (uint32_t)auto_item_cap(b.n) / kCluster;
+    r.dense = dense_cell((uint32_t)b.n, (uint32_t)b.nc * b.nc * b.nc);
     return r;
 }
 
 __device__ __forceinline__ uint32_t clusters_of(uint32_t cnt) { return (cnt + kCluster - 1) / kCluster; }
 
 __device__ __forceinline__ uint32_t items_of(uint32_t cnt, ItemRule r) {
-    const uint32_t per = cnt > r.split_max ? (uint32_t)(kItemMax / kCluster) : r.clusters;
+    uint32_t per = cnt > r.split_max ? (uint32_t)(kItemMax / kCluster) : r.clusters;
+    if (cnt > r.dense && cnt <= r.split_max) per = min(per, (uint32_t)(kItemMax / kCluster / 2));
     return (clusters_of(cnt) + per - 1) / per;
 }
 
@@ -675,7 +689,6 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_big(const uint32_t *__r
 // call's rows in shared memory (hacc_bin of 65536 particles in one cell 111 us,
 // in four 104; by merge sort in k_order_big's thousand threads 966 and 274, in
 // the block's own 2438 and 2039).
-constexpr uint32_t kBlockCell = 2048;
 constexpr int64_t kBigHereMax = (int64_t)1 << 16;
 // Calls of up to this many particles gather in the ordering's blocks: a launch
 // fewer (250 thousand particles: call 205.5 -> 202 us).  Larger ones hide more
@@ -1558,8 +1571,9 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
     // a cell of a single cluster keeps row order (not with kick counts, whose
     // order an event's items rely on)
     const uint32_t row_below = (item_cap && !sub_level) ? (uint32_t)kCluster : 0u;
-    return bin_sort(n, g.ncell, b, make_items, nullptr, 1, s, item_rule(item_cap, split_max), sub, row_below,
-                    sorted_input, gather);
+    ItemRule rule = item_rule(item_cap, split_max);
+    if (b.sub) rule.dense = dense_cell((uint32_t)n, (uint32_t)g.ncell);   // (without the sub-cell arrays there is room for items of 64 alone)
+    return bin_sort(n, g.ncell, b, make_items, nullptr, 1, s, rule, sub, row_below, sorted_input, gather);
 }
 
 cudaError_t ml_levels(const Geometry &g, int64_t n, const BinBuffers &b, int d, int lmin, int lmax, int32_t *level,
@@ -1641,8 +1655,9 @@ cudaError_t bin_build_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *of
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    return bin_sort(n, g.ncell, b, true, nullptr, 1, s, item_rule(kItemMax, kDefaultSplitMax), b.sub, kCluster,
-                    false, gather);
+    ItemRule rule = item_rule(kItemMax, kDefaultSplitMax);
+    rule.dense = dense_cell((uint32_t)n, (uint32_t)g.ncell);
+    return bin_sort(n, g.ncell, b, true, nullptr, 1, s, rule, b.sub, kCluster, false, gather);
 }
 
 cudaError_t drift_ci(const Geometry &g, int64_t n, int32_t *cell, float4 *off, const float4 *vel, double drift,
