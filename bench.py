@@ -347,7 +347,7 @@ def run_batched(torch, hacc, ctx, split, steps=3, warmup=1, n_sub=10, seed=4):
     de = np.abs((d_end[:, 3] + d_end[:, 4]) - (d_start[:, 3] + d_start[:, 4]))
     energy = de / (d_start[:, 3] + np.abs(d_start[:, 4]))
     energy_ke = de / d_start[:, 3]
-    default_k = 0   # cell-wide items, cell order, variant 0
+    default_k = 0   # items of up to 64 in input-row order (the first cap, 0), cell order, variant 0
     return {"workload": "200 blob-mixture boxes, N log-uniform 16^3..128^3 (total %d), 10 SR sub-cycles per "
                         "step, one batched launch per sub-cycle, CUDA graph" % n,
             "autotune": {"chosen_setting": tune["chosen"], "item_cap": tune["item_cap"], "variant": tune["variant"],
@@ -1122,8 +1122,8 @@ def run_ours(args):
             "autotune": {"setting": tuning["chosen"], "variant": tuning["variant"], "item_cap": tuning["item_cap"],
                          "heavy_first": tuning["heavy_first"], "ms_by_setting": tuning["times_ms"],
                          "settings": "item cap in %s x queue order (cell, largest first) x variants (blocks/SM, "
-                                     "inner loop) = (5,indexed), (4,indexed), (5,pointer-stepped), "
-                                     "(4,pointer-stepped); time = one sub-cycle's chaining-mesh build + "
+                                     "pair steps unrolled) = (5,4), (4,4), (5,2), (4,2); "
+                                     "time = one sub-cycle's chaining-mesh build + "
                                      "kick-and-stream launch" % (list(hacc.TUNE_CAPS),)}}
     if not args.no_batch:
         line["batched"] = run_batched(torch, hacc, ctx, split)

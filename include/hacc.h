@@ -405,7 +405,7 @@ size_t hacc_batch_scratch_bytes(const hacc_split *split, int32_t nbox, const hac
  * HACC_NOALLOC_SCRATCH_BYTES compiled into the library, which every GPU that
  * loads the library holds until the process exits.  The caller owns pos_m
  * (n rows, not modified) and acc (n rows, receives (ax, ay, az, 0)).
- *   - Limit: about 49.3 bytes per particle plus 36 bytes per chaining-mesh cell
+ *   - Limit: about 48.3 bytes per particle plus 36 bytes per chaining-mesh cell
  *     must fit in the array (e.g. 262144 particles with up to 100000 cells);
  *     larger problems return HACC_ENOMEM before anything is enqueued.
  *   - Works on the current CUDA device; `stream` must belong to it
@@ -421,8 +421,9 @@ size_t hacc_batch_scratch_bytes(const hacc_split *split, int32_t nbox, const hac
 hacc_status hacc_sr_force_noalloc(const hacc_box *box, const hacc_split *split, int64_t n,
                                   const float *pos_m, float *acc, hacc_stream_t stream);
 
-/* Number of pair-kernel variants: register budget (96 or 128 per thread) x
- * inner loop (indexed or pointer-stepped); all give bitwise the same forces. */
+/* Number of pair-kernel variants: blocks per SM (5 or 4: 96 or 128 registers a
+ * thread) x steps of the pair loop unrolled (4 or 2); all give bitwise the same
+ * forces. */
 #define HACC_FORCE_VARIANTS 4
 
 /* Autotuner (a tuning aid of the library; the paper has no counterpart):
@@ -474,7 +475,8 @@ hacc_status hacc_set_stencil(hacc_ctx *ctx, int32_t cells_per_rcut);
  * neighbours skipped by the item's bounds alone.
  * cap = -1 (default): by the box's size, 8 particles up to 2^13, 16 up to
  * 3*2^12, 32 up to 2^20, 64 above (small boxes have few items to spread over the
- * chip), and up to 2^16 particles the neighbours of an item are summed in four
+ * chip; the cells of larger boxes above 2048 particles and 8 times the mean take
+ * 32), and up to 2^16 particles the neighbours of an item are summed in four
  * parts, by the four warps of a block; a box of a batch follows its own size, its
  * parts one after the other.  The cell/offset paths use 64,
  * hacc_sr_force_noalloc row order with items of 64 skipped per cluster.
@@ -491,7 +493,11 @@ hacc_status hacc_set_item_cap(hacc_ctx *ctx, int32_t cap, int32_t split_max);
  * other values. */
 hacc_status hacc_set_queue_order(hacc_ctx *ctx, int32_t heavy_first);
 
-/* Select the pair-kernel variant by hand (0 <= variant < HACC_FORCE_VARIANTS). */
+/* Select the pair-kernel variant by hand (0 <= variant < HACC_FORCE_VARIANTS).
+ * Launches that have one form only take that one: with the automatic item cap
+ * boxes of up to 2^16 particles and batches that hold one, boxes of 3 cells a
+ * side (fewer than 8 of the 125-cell stencil) and batches that hold one, counted
+ * launches, potentials and the cell/offset paths. */
 hacc_status hacc_set_variant(hacc_ctx *ctx, int32_t variant);
 
 /* Run statistics kept by a context (instrumentation, not part of the method). */

@@ -387,10 +387,11 @@ class Context:
                                            self._stream(stream)), "hacc_subcycle_ci")
 
     def set_queue_order(self, heavy_first: bool):
-        """Work-item order of large force launches: largest first (True, default) or cell order."""
+        """Work-item order of large force launches: largest first (True) or cell order (False, the default)."""
         self._check(lib().hacc_set_queue_order(self._h, int(bool(heavy_first))), "hacc_set_queue_order")
 
     def set_variant(self, variant: int):
+        """Pair-kernel variant, 0..FORCE_VARIANTS-1, of the launches that have several (hacc_set_variant)."""
         self._check(lib().hacc_set_variant(self._h, int(variant)), "hacc_set_variant")
 
     def set_item_cap(self, cap: int, split_max: int = 0):

@@ -1076,7 +1076,7 @@ hacc_status hacc_subcycle_ml(hacc_ctx *ctx, const hacc_box *box, const hacc_spli
     std::vector<MlEvent> ev = ml_schedule(present, lmax, dt);
     const float half_lim = (float)(half * (1.0 - 1e-5));
     // particles kicked at each event; a small launch splits its cells into
-    // smaller items (down to one lane per particle) so that enough warps share it
+    // smaller items (down to a cluster) so that enough warps share it
     std::vector<int> caps(ev.size());
     for (size_t k = 0; k < ev.size(); ++k) {
         int64_t kicked = 0;

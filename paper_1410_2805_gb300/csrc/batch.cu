@@ -4,8 +4,8 @@
 // hacc_subcycle (Sec. 2.5), but all boxes share one binning pass (global cell
 // ids = the box's cell base + its local id, so one counting sort covers them
 // all) and ONE persistent pair-kernel launch whose warps take work items of
-// every box from a single atomic queue (the work queue of Sec. 3.1, one item
-// per cell or 128-particle slice of a cell).  The pair kernel writes kicked
+// every box from a single atomic queue (the work queue of Sec. 3.1, items of
+// clusters of one cell).  The pair kernel writes kicked
 // and streamed particles straight back to their pool rows, wrapped.
 //
 // Within a cell the particles are ordered by pool row, and a box's items only

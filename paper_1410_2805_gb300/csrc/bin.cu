@@ -410,8 +410,8 @@ __device__ __forceinline__ void gather_row(const Gather &g, int64_t k, int32_t i
 // (distinct), which gives ascending input row within the cell, or the pair
 // (sub-cell code, input row), which groups the cell's particles by sub-cell.
 // k_order_rows serves calls of up to 2^24 rows (the pair as one 32-bit key,
-// code << 24 | row); k_order_sub, one warp per cell, larger ones: a cell that
-// becomes one work item by row, the others by the pair with the row taken
+// code << 24 | row); k_order_sub, one warp per cell, larger ones: a cell of a
+// single cluster by row, the others by the pair with the row taken
 // relative to the cell's smallest row (one 32-bit key when the cell's rows
 // span less than 2^24, else 64-bit keys; codes are below 2^8), cells of up to
 // 256 keys through the register networks above, larger ones by counting.
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kBlock) k_order_sub(int64_t ncell, const uint3
     int32_t *out = perm + s;
     const unsigned long long *seg = order_tmp + s;
     if (cnt <= row_below) {
-        // a cell that becomes one work item keeps row order (cnt <= 160)
+        // a cell of a single cluster keeps row order
         sort_small_cell([&](uint32_t e) { return (uint32_t)seg[e]; }, cnt, lane, out,
                         [](uint32_t k) { return (int32_t)k; });
         return;

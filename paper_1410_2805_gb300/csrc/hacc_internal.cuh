@@ -54,7 +54,7 @@ struct hacc_ctx {
     int64_t ml_rebins = 0;
     int variant = 0;                          // pair-kernel variant (hacc_tune)
     int stencil = 1;                          // single-box force paths: 1 (27 cells) or 2 (125 cells of half width)
-    int item_cap = -1;                        // work-item cap of the force paths (0: cell-wide items, -1: auto)
+    int item_cap = -1;                        // work-item cap of the force paths (hacc_set_item_cap)
     int split_max = hacc::kDefaultSplitMax;   // cells above this many particles keep items of up to kItemMax
     int queue_order = 0;                      // 1: largest work items first (calls of 2^20 particles and more), 0: cell order
     double force_ms = 0.0;
@@ -298,7 +298,7 @@ cudaError_t bin_build(const Geometry &g, int64_t n, const float4 *src, const flo
 // part_base and cell_base): for every tick-scratch index t the particle at
 // pool row boxes[b].row_off + t - part_base is streamed by pre, wrapped,
 // binned into global cell cell_base + local id; dst[t] = its position,
-// id[t] = its pool row.  Work items carry the box in item.w >> 8.  item_cap
+// id[t] = its pool row.  Work items carry the box in item.w.  item_cap
 // as for bin_build (ties in the sub-cell order by scratch index), or -1: each
 // box's automatic cap.
 cudaError_t bin_build_batch(int nbox, const BoxDev *boxes, int64_t n_total, int64_t ncell_total,

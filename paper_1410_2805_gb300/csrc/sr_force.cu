@@ -27,7 +27,7 @@
 // operands are three different registers); scalar arithmetic for the
 // polynomial or the sums, which needs fewer pipe cycles and more slots, is
 // 3-7% slower.  The pairs are half of the instructions, the selecting and
-// staging most of the rest.  So every pair not evaluated counts:
+// staging most of the rest.
 // Why clusters of 8: per particle of a Zel'dovich box, 970 candidates lie in
 // the 27 cells, 655 within reach of a cell's bounds, 390 of an 8-cluster's and
 // 285 of a 4-cluster's, 154 inside the cutoff (a bounding sphere instead of the
