@@ -993,8 +993,12 @@ __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
     // equal masses in a box (its bit left 0 by the binning pass): applied once per i.
     // The boxes of a batch take the form that each takes alone, in two rounds of the
     // queue where both occur (both forms in one loop spilled registers).
+    constexpr bool kBatches = !CI && SH != kByBlock;   // forms that batches take too
     unsigned some = ~0u, every = ~0u;
-    if (!POT && P.mass_flag) {
+    if (!kBatches && !POT && P.mass_flag) {
+        some = uniform(*P.mass_flag);
+        every = some ? ~0u : 0u;
+    } else if (!POT && P.mass_flag) {
         some = 0u;
         for (int k = lane; 32 * k < P.nbox; k += 32) {
             const unsigned v = P.mass_flag[k];
@@ -1004,7 +1008,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_sr_force(KParams P) {
         some = __reduce_or_sync(0xffffffffu, some);
         every = __reduce_and_sync(0xffffffffu, every);
     }
-    const bool mixed = !CI && SH != kByBlock && some && ~every;   // (those are never a batch's)
+    const bool mixed = kBatches && some && ~every;
     if (!POT && ~every) work_loop<COUNT, POT, EPS0, !POT, F, CI, SH, FRAMES>(P, *S, lane, P.work_counter, mixed);
     if (some) work_loop<COUNT, POT, EPS0, false, F, CI, SH, FRAMES>(P, *S, lane, P.work_counter + mixed, mixed);
 }
